@@ -52,8 +52,8 @@ ADJOINT_DEFAULT = "adjoint_broadband_2d_512_teno6_mp"
 FP64_LANES_PER_CLK = 304  # FP64 pipe: 2 lanes per clock per SM x 152 SMs
 
 
-FACE_SOURCES = ("tenom_face.cuh", "tenom_face_fwd.cuh", "tenom_recon.cuh", "tenom_linear.cuh",
-                "tenom_stats.cuh", "teno_coeffs.cuh", "tenom_fastmath.cuh", "tenom_launch.cuh", "tenom_internal.h")
+FACE_SOURCES = ("tenom_screen.cuh", "tenom_nonlinear.cuh", "tenom_face.cuh", "tenom_recon.cuh", "teno_coeffs.cuh",
+                "tenom_fastmath.cuh", "tenom_launch.cuh", "tenom_internal.h")
 
 
 BATCH_SOURCES = FACE_SOURCES + ("tenom_batch.cu", "tenom_batch_kernel.cuh", "tenom_positivity.cuh")
@@ -533,7 +533,7 @@ def face_roofline(name, shape, nv, face_ms, face_launches, clk, probe_flops):
     roof = {"bound": "alu", "achieved": achieved, "peak": probe_inst, "unit": "FP64 inst/s",
             "frac": achieved / probe_inst if achieved else None,
             "traffic": float(fig["dram_bytes_per_launch"]) if fig else None,
-            "kernel": "face_kernel (fused characteristic TENO-M face flux)",
+            "kernel": "screen_kernel + nonlinear_kernel (characteristic TENO-M face flux)",
             "fp64_inst_per_face": ipf, "faces_per_launch": faces_per_launch, "ms_per_launch": face_ms,
             "launches_timed": face_launches,
             "peak_note": "measured: DFMA probe (8 independent FMA chains per thread) in FP64 instructions/s; "

@@ -111,8 +111,9 @@ tenom_status tenom_scheme_default(tenom_scheme* s, int K);
 
 /* Create a context for one grid and scheme.  stream: a cudaStream_t (NULL = legacy
  * default stream) on which every call of this context is ordered.  Allocates the
- * context's device workspace (stage buffer, face buffers, scalars) on the current device:
- * about (nvar * ncell * (1 + dim) + small) * 8 bytes.  On success *ctx owns it. */
+ * context's device workspace (stage buffer, face buffers and face lists, cell primitives,
+ * scalars) on the current device: about (nvar * ncell * (2 + dim) + 2 * ncell) * 8 + 5 * dim *
+ * ncell bytes.  On success *ctx owns it. */
 tenom_status tenom_create(tenom_ctx** ctx, const tenom_grid* grid, const tenom_scheme* scheme, void* stream);
 
 /* Free the context and its workspace (synchronises its stream first).  NULL is a no-op. */
@@ -160,7 +161,7 @@ tenom_status tenom_positivity_limit(tenom_ctx* ctx, const double* U, int axis, c
 tenom_status tenom_face_dump(tenom_ctx* ctx, const double* U, int axis, double* Fhat, uint8_t* flags);
 
 /* Decision statistics of the reconstruction at the state U (device [nvar][ncell]) on the
- * faces of axis `axis`, for logging (not part of a step): the face kernel's characteristic
+ * faces of axis `axis`, for logging (not part of a step): the face sweeps' characteristic
  * sequences (f+ and f- of every field, Section 4) are examined instead of reconstructed,
  * and TENOM_NSTATS counters are ADDED to the caller-owned device array counters_dev (64-bit;
  * the caller zeroes it).  Per split side: [0] sides; [1] sides the certified FP32 cutoff
@@ -210,8 +211,8 @@ tenom_status tenom_batch_stage(tenom_batch* b, int stage, double* U);
 tenom_status tenom_batch_autotune(tenom_batch* b, double* U, int* tile, int* ctas_per_sm);
 tenom_status tenom_batch_set_tiling(tenom_batch* b, int tile, int ctas_per_sm);
 
-/* Size of the static device scratch of tenom_rhs_noalloc: 16 MiB, held on every GPU that
- * loads this library until the process exits. */
+/* Size of the static device scratch for the face fluxes of tenom_rhs_noalloc: 16 MiB, held on
+ * every GPU that loads this library until the process exits (with 4 MiB more for the face lists). */
 #define TENOM_NOALLOC_SCRATCH_BYTES (16u << 20)
 
 /* tenom_rhs without a context and without any device allocation.  The paper has no
@@ -222,7 +223,7 @@ tenom_status tenom_batch_set_tiling(tenom_batch* b, int tile, int ctas_per_sm);
  * scheme, on `stream` (a cudaStream_t; NULL = legacy default stream), with the face-sweep
  * and flux-difference kernels of tenom_rhs.  One difference: tenom_rhs first computes the
  * cells' primitives (velocity, p, H, c, sqrt rho) once per cell into its context's
- * buffer, while this call has no such buffer and the face kernels form them for each
+ * buffer, while this call has no such buffer and the sweep kernels form them for each
  * staged point of their tile; the two round alike except in the last bits, which can
  * flip a cutoff decision that rounding sets (a flat sequence at a zero-gradient boundary);
  * agreement to 1e-13 of each component's largest value is tested.  U and dUdt are caller-owned device arrays as for tenom_rhs; status_dev
@@ -308,8 +309,8 @@ tenom_status tenom_status_word(tenom_ctx* ctx, int* status_host, int reset);
 /* Text of the last error of this context ("" if none).  Valid until the next call. */
 const char* tenom_last_error(const tenom_ctx* ctx);
 
-/* Measurement helper (not part of the method): average duration in ms of the face kernel
- * of axis a over the last tenom_rk3_step/tenom_advance calls, timed with CUDA events on
+/* Measurement helper (not part of the method): average duration in ms of the face sweep
+ * of one axis (its screen and its share of the stage's nonlinear launch) over the last tenom_rk3_step/tenom_advance calls, timed with CUDA events on
  * the context stream when timing is enabled.  enable != 0 turns timing on and resets. */
 tenom_status tenom_kernel_timing(tenom_ctx* ctx, int enable, double* face_ms_per_launch, long long* launches);
 

@@ -11,6 +11,7 @@
 #include "tenom.h"
 #include "tenom_internal.h"
 #include "tenom_adjoint_kernels.cuh"
+#include "tenom_nonlinear.cuh"
 #include "tenom_positivity.cuh"
 
 namespace tenom {
@@ -35,6 +36,32 @@ __global__ void init_state_kernel(const double* __restrict__ prim, double* __res
   }
 }
 
+/* Where a kernel that has a cell's state in registers leaves its primitives for the next
+   face sweeps: P = [velocity (NV - 2), p, c | H, sqrt rho], the last two (the adjoint's and the
+   record kernels') only when full.  The same launch clears the sweeps' list lengths. */
+struct PrimOut {
+  double* P;          /* null: none */
+  unsigned* count;    /* list lengths of the axes */
+  int* status;
+  double gamma;
+  int full;
+};
+
+template <int NV>
+__device__ __forceinline__ void put_prims(const PrimOut& O, long long nc, long long c, const double (&u)[NV], int& st) {
+  constexpr int D = NV - 2;
+  double vel[D], pr, cs;
+  point_prims<NV>(u, O.gamma, vel, pr, cs, st);
+#pragma unroll
+  for (int d = 0; d < D; ++d) O.P[d * nc + c] = vel[d];
+  O.P[D * nc + c] = pr;
+  O.P[(D + 1) * nc + c] = cs;
+  if (O.full) {
+    O.P[(D + 2) * nc + c] = (u[NV - 1] + pr) * rcp_nr(u[0]);
+    O.P[(D + 3) * nc + c] = sqrt(u[0]);
+  }
+}
+
 /* Flux difference -sum_a (F_{a,i+1/2} - F_{a,i-1/2}) / dx_a (Eq. approximateEq) and the
    SSP-RK3 stage combine of one cell: mode 0 out = L (operator), 1 out = Us + dt L (stage
    1), 2 out = cA U0 + cB (Us + dt L) (stages 2, 3); dt = 0 (a step past t_end) keeps Us. */
@@ -51,10 +78,11 @@ struct CellUpdate {
 };
 
 /* the cell update of cell c whose x-face difference F_{x,i+1/2} - F_{x,i-1/2} is dfx; the
-   other axes' faces at fl[a] and fl[a] + fs[a] */
+   other axes' faces at fl[a] and fl[a] + fs[a]; un: the values written */
 template <int NV>
 __device__ __forceinline__ void cell_update(const CellUpdate& A, long long nc, long long c, const double (&dfx)[NV],
-                                            const long long (&fl)[3], const long long (&fs)[3], double dt) {
+                                            const long long (&fl)[3], const long long (&fs)[3], double dt,
+                                            double (&un)[NV]) {
   constexpr int DIM = NV - 2;
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
@@ -66,27 +94,31 @@ __device__ __forceinline__ void cell_update(const CellUpdate& A, long long nc, l
       r = r - (F[fl[a] + fs[a]] - F[fl[a]]) * A.rdx[a];
     }
     if (A.mode == 0) {
-      A.out[v * nc + c] = r;
+      un[v] = r;
     } else if (dt == 0.0) {
       /* a step past t_end: every stage state equals U^n, keep it bit for bit */
-      A.out[v * nc + c] = A.Us[v * nc + c];
+      un[v] = A.Us[v * nc + c];
     } else {
       const double us = A.Us[v * nc + c];
       const double t1 = us + dt * r;
-      A.out[v * nc + c] = (A.mode == 1) ? t1 : A.cA * A.U0[v * nc + c] + A.cB * t1;
+      un[v] = (A.mode == 1) ? t1 : A.cA * A.U0[v * nc + c] + A.cB * t1;
     }
+    A.out[v * nc + c] = un[v];
   }
 }
 
 struct StageArgs {
   CellUpdate cu;       /* faces of every axis, states, dt, 1/dx_a, stage coefficients */
+  PrimOut po;          /* primitives of the stage output, for the next stage's sweeps */
   int n[3];
   long long ncell;
 };
 
 /* Flux difference -sum_a (F_{a,i+1/2} - F_{a,i-1/2})/dx_a (Eq. approximateEq) fused with
-   the SSP-RK3 stage combine (cell_update); 1/dx_a is formed once on the host (an FP64 division per cell and axis
-   would occupy the FP64 pipe longer than the kernel's memory traffic takes). */
+   the SSP-RK3 stage combine (cell_update) and the next stage's primitives (the state is in
+   registers: a pass over it and a launch per stage saved); 1/dx_a is formed once on the host
+   (an FP64 division per cell and axis would occupy the FP64 pipe longer than the kernel's
+   memory traffic takes). */
 template <int NV>
 __global__ void stage_kernel(const StageArgs A) {
   constexpr int DIM = NV - 2;
@@ -95,6 +127,8 @@ __global__ void stage_kernel(const StageArgs A) {
   /* one thread per cell: x from the block's column, y and z from the grid (strided when an
      axis exceeds the grid's 65535 limit) */
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  int st = 0;
+  if (A.po.P && x < 3 && blockIdx.y == 0 && blockIdx.z == 0 && blockIdx.x == 0) A.po.count[x] = 0u;
   if (x >= A.n[0]) return;
   for (int z = blockIdx.z; z < A.n[2]; z += gridDim.z) {
     for (int y = blockIdx.y; y < A.n[1]; y += gridDim.y) {
@@ -110,15 +144,17 @@ __global__ void stage_kernel(const StageArgs A) {
         fl[2] = c;
         fs[2] = (long long)A.n[0] * A.n[1];
       }
-      double dfx[NV];
+      double dfx[NV], un[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const double* F = A.cu.F[0] + v * A.cu.nface[0];
         dfx[v] = F[fx + 1] - F[fx];
       }
-      cell_update<NV>(A.cu, nc, c, dfx, fl, fs, dt);
+      cell_update<NV>(A.cu, nc, c, dfx, fl, fs, dt, un);
+      if (A.po.P) put_prims<NV>(A.po, nc, c, un, st);
     }
   }
+  if (st) atomicOr(A.po.status, st);
 }
 
 static cudaError_t launch_stage_kernel(int nv, const StageArgs& a, cudaStream_t st) {
@@ -130,14 +166,17 @@ static cudaError_t launch_stage_kernel(int nv, const StageArgs& a, cudaStream_t 
   return cudaGetLastError();
 }
 
-/* max_i sum_a (|u_a| + c)/dx_a, reduced with atomicMax on the (positive) bit pattern. */
+/* max_i sum_a (|u_a| + c)/dx_a, reduced with atomicMax on the (positive) bit pattern; with
+   po.P also the cells' primitives for the sweeps of the step's first stage. */
 template <int NV>
 __global__ void signal_speed_kernel(const double* __restrict__ U, long long nc, double gamma, double rdx0,
-                                    double rdx1, double rdx2, unsigned long long* smax, int* status) {
+                                    double rdx1, double rdx2, unsigned long long* smax, int* status,
+                                    const PrimOut po) {
   constexpr int DIM = NV - 2;
   const double rdx[3] = {rdx0, rdx1, rdx2};
   double m = 0.0;
   int st = 0;
+  if (po.P && blockIdx.x == 0 && threadIdx.x < 3) po.count[threadIdx.x] = 0u;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc; c += (long long)gridDim.x * blockDim.x) {
     const double rho = U[c];
     const double rinv = rcp_nr(rho);
@@ -155,6 +194,12 @@ __global__ void signal_speed_kernel(const double* __restrict__ U, long long nc, 
 #pragma unroll
     for (int d = 0; d < DIM; ++d) s += (fabs(vel[d]) + cs) * rdx[d];
     m = (s > m) ? s : m;
+    if (po.P) {
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) po.P[d * nc + c] = vel[d];
+      po.P[DIM * nc + c] = p;
+      po.P[(DIM + 1) * nc + c] = cs;
+    }
   }
   /* warp then block reduction */
 #pragma unroll
@@ -194,25 +239,18 @@ __global__ void finalize_dt_kernel(unsigned long long* smax, double cfl, double*
 
 __global__ void advance_time_kernel(double* t, const double* dt) { *t = *t + *dt; }
 
-/* Compare the Newton-Raphson reciprocal / rsqrt with CUDA's correctly rounded 1.0/x, sqrt. */
-/* per-cell primitives for the face sweeps of one stage: P = [velocity (NV-2), p, H, c, sqrt rho] */
+/* cell primitives of a state for the face sweeps (PrimOut) */
 template <int NV>
-__global__ void prim_kernel(const double* __restrict__ U, long long ncell, double gamma, double* __restrict__ P,
-                            int* status) {
+__global__ void prim_kernel(const double* __restrict__ U, long long ncell, const PrimOut O) {
   int st = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 3) O.count[threadIdx.x] = 0u;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ncell; i += (long long)gridDim.x * blockDim.x) {
-    double u[NV], vel[NV - 2], pr, Hh, c, sr;
+    double u[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) u[q] = U[q * ncell + i];
-    point_prims<NV>(u, gamma, vel, pr, Hh, c, sr, st);
-#pragma unroll
-    for (int d = 0; d < NV - 2; ++d) P[d * ncell + i] = vel[d];
-    P[(NV - 2) * ncell + i] = pr;
-    P[(NV - 1) * ncell + i] = Hh;
-    P[NV * ncell + i] = c;
-    P[(NV + 1) * ncell + i] = sr;
+    put_prims<NV>(O, ncell, i, u, st);
   }
-  if (st) atomicOr(status, st);
+  if (st) atomicOr(O.status, st);
 }
 
 /* Positivity-preserving flux limiter of one forward-Euler stage of length dt (Section 4.4),
@@ -313,6 +351,7 @@ static cudaError_t launch_positivity_kernel(int nv, const PosArgs& p, cudaStream
   return cudaGetLastError();
 }
 
+/* Compare the Newton-Raphson reciprocal / rsqrt with CUDA's correctly rounded 1.0/x, sqrt. */
 __global__ void fastmath_check_kernel(const double* x, double* out, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double v = x[i];
@@ -367,9 +406,13 @@ struct tenom_ctx {
   int nv;
   long long ncell;
   long long nface[3];
+  char* arena;         /* one allocation holding W1, face, P, list, mask and the scalars */
   double* W1;          /* stage buffer */
   double* face[3];     /* face buffers */
   double* P;           /* per-cell primitives of the stage being evaluated ([nvar + 2][ncell]) */
+  unsigned* list[3];   /* per axis: faces left to the nonlinear kernel (capacity nface), */
+  uint8_t* mask[3];    /*   their uncertified fields, */
+  unsigned* count;     /*   and the list lengths */
   double* dt;          /* device dt */
   double* tbuf;        /* device scratch time */
   double* Uhost;       /* device state for tenom_advance_host (allocated on first use) */
@@ -412,6 +455,15 @@ static SchemeDev scheme_dev(const tenom_scheme& s) {
   d.default_d = 1;
   for (int k = 0; k < s.K - 2; ++k)
     if (s.d[k] != ((s.K == 6) ? kDopt6[k] : kDopt8[k])) d.default_d = 0;
+  d.screen = d.default_d && !d.exact_decisions;
+  /* R = (nk C_T)^(-1/6), 0.5 % below; at most 1000 (a tiny or non-positive C_T), at least 1 (nothing
+     is certified) */
+  auto ratio = [&](double ct) {
+    const double r = ct > 1e-20 ? 0.995 * std::pow(1.0 / ((s.K - 2) * ct), 1.0 / 6.0) : 1000.0;
+    return (float)(r < 1000.0 ? (r > 1.0 ? r : 1.0) : 1000.0);
+  };
+  d.quick_r[0] = ratio(s.ct_mode == TENOM_CT_ADAPTIVE ? 1e-7 : s.ct_const);
+  d.quick_r[1] = ratio(1e-10);
   return d;
 }
 
@@ -493,8 +545,11 @@ tenom_status tenom_create(tenom_ctx** out, const tenom_grid* grid, const tenom_s
   for (int a = 0; a < 3; ++a) {
     c->nface[a] = 0;
     c->face[a] = nullptr;
+    c->list[a] = nullptr;
+    c->mask[a] = nullptr;
     if (a < grid->dim) c->nface[a] = c->ncell / grid->n[a] * (grid->n[a] + 1);
   }
+  c->arena = nullptr;
   c->Uhost = nullptr;
   c->adj = nullptr;
   c->adj_flags = nullptr;
@@ -502,17 +557,36 @@ tenom_status tenom_create(tenom_ctx** out, const tenom_grid* grid, const tenom_s
   c->ev_used = 0;
   c->face_ms = 0;
   c->face_launches = 0;
-  cudaError_t e = cudaMalloc(&c->W1, sizeof(double) * c->nv * c->ncell);
-  for (int a = 0; a < grid->dim && e == cudaSuccess; ++a) e = cudaMalloc(&c->face[a], sizeof(double) * c->nv * c->nface[a]);
-  if (e == cudaSuccess) e = cudaMalloc(&c->P, sizeof(double) * (c->nv + 2) * c->ncell);
-  if (e == cudaSuccess) e = cudaMalloc(&c->dt, sizeof(double) * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&c->smax, sizeof(unsigned long long) + sizeof(int) * 2);
-  if (e == cudaSuccess) {
-    c->tbuf = c->dt + 1;
-    c->status = (int*)(c->smax + 1);
-    e = cudaMemsetAsync(c->smax, 0, sizeof(unsigned long long) + sizeof(int) * 2, c->st);
+  /* the whole workspace in one allocation, 256-byte aligned parts */
+  size_t bytes = 0;
+  auto part = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) & ~(size_t)255;
+    return at;
+  };
+  const size_t small = part(256);  /* status, list lengths, CFL maximum, dt, t */
+  const size_t w1 = part(sizeof(double) * c->nv * c->ncell), prims = part(sizeof(double) * (c->nv + 2) * c->ncell);
+  size_t face[3], list[3];
+  for (int a = 0; a < grid->dim; ++a) {
+    face[a] = part(sizeof(double) * c->nv * c->nface[a]);
+    list[a] = part((sizeof(unsigned) + 1) * c->nface[a]);
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->dt, 0, sizeof(double) * 2, c->st);
+  cudaError_t e = cudaMalloc(&c->arena, bytes);
+  if (e == cudaSuccess) {
+    c->W1 = reinterpret_cast<double*>(c->arena + w1);
+    c->P = reinterpret_cast<double*>(c->arena + prims);
+    for (int a = 0; a < grid->dim; ++a) {
+      c->face[a] = reinterpret_cast<double*>(c->arena + face[a]);
+      c->list[a] = reinterpret_cast<unsigned*>(c->arena + list[a]);
+      c->mask[a] = reinterpret_cast<uint8_t*>(c->list[a] + c->nface[a]);
+    }
+    c->smax = reinterpret_cast<unsigned long long*>(c->arena + small);
+    c->dt = reinterpret_cast<double*>(c->arena + small + 64);
+    c->tbuf = c->dt + 1;
+    c->status = reinterpret_cast<int*>(c->arena + small + 128);
+    c->count = reinterpret_cast<unsigned*>(c->arena + small + 192);
+    e = cudaMemsetAsync(c->arena + small, 0, 256, c->st);
+  }
   if (e != cudaSuccess) {
     fprintf(stderr, "tenom_create: %s\n", cudaGetErrorString(e));
     tenom_destroy(c);
@@ -525,11 +599,7 @@ tenom_status tenom_create(tenom_ctx** out, const tenom_grid* grid, const tenom_s
 tenom_status tenom_destroy(tenom_ctx* c) {
   if (!c) return TENOM_OK;
   cudaStreamSynchronize(c->st);
-  cudaFree(c->W1);
-  for (int a = 0; a < 3; ++a) cudaFree(c->face[a]);
-  cudaFree(c->P);
-  cudaFree(c->dt);
-  cudaFree(c->smax);
+  cudaFree(c->arena);
   cudaFree(c->Uhost);
   cudaFree(c->adj);
   cudaFree(c->adj_flags);
@@ -563,8 +633,12 @@ static FaceArgs face_args(tenom_ctx* c, const double* U, int axis, double* F, ui
   FaceArgs a;
   memset(&a, 0, sizeof(a));
   a.U = U;
+  a.P = c->P;
   a.Fhat = F;
   a.flags = flags;
+  a.list = c->list[axis];
+  a.mask = c->mask[axis];
+  a.count = c->count + axis;
   a.status = c->status;
   for (int d = 0; d < 3; ++d) {
     a.n[d] = c->g.n[d];
@@ -577,12 +651,11 @@ static FaceArgs face_args(tenom_ctx* c, const double* U, int axis, double* F, ui
   return a;
 }
 
-/* one face sweep of axis `axis` at U (P: its cell primitives) */
-static cudaError_t launch_faces(tenom_ctx* c, const double* U, int axis, double* F, uint8_t* flags,
-                                double* lin = nullptr, const double* P = nullptr) {
-  FaceArgs a = face_args(c, U, axis, F, flags);
-  a.lin = lin;
-  a.P = P;
+/* Face fluxes at U (c->P: its cell primitives, list lengths zero) of axes a0 .. a1 - 1: the
+   screen of each axis, then the listed faces of all of them in one launch.  flags, lin: one
+   stage's cutoff flags / linearisation per axis, or null. */
+static cudaError_t launch_faces(tenom_ctx* c, const double* U, int a0, int a1, double* const* F, uint8_t* const* flags,
+                                double* const* lin) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (c->timing) {
     while (c->ev.size() < c->ev_used + 2) {
@@ -596,18 +669,57 @@ static cudaError_t launch_faces(tenom_ctx* c, const double* U, int axis, double*
     c->ev_used += 2;
     cudaEventRecord(e0, c->st);
   }
-  cudaError_t e;
-  if (lin) {
-    if (c->nv == 3) e = launch_face_rec_nv3(a, axis, c->s.K, c->s.limiter, c->st);
-    else if (c->nv == 4) e = launch_face_rec_nv4(a, axis, c->s.K, c->s.limiter, c->st);
-    else e = launch_face_rec_nv5(a, axis, c->s.K, c->s.limiter, c->st);
-  } else {
-    if (c->nv == 3) e = launch_face_nv3(a, axis, c->s.K, c->s.limiter, c->st);
-    else if (c->nv == 4) e = launch_face_nv4(a, axis, c->s.K, c->s.limiter, c->st);
-    else e = launch_face_nv5(a, axis, c->s.K, c->s.limiter, c->st);
+  NonlinArgs N;
+  memset(&N, 0, sizeof(N));
+  cudaError_t e = cudaSuccess;
+  for (int a = a0; a < a1 && e == cudaSuccess; ++a) {
+    FaceArgs f = face_args(c, U, a, F[a], flags ? flags[a] : nullptr);
+    f.lin = lin ? lin[a] : nullptr;
+    if (c->nv == 3) e = launch_screen_nv3(f, a, c->s.K, c->st);
+    else if (c->nv == 4) e = launch_screen_nv4(f, a, c->s.K, c->st);
+    else e = launch_screen_nv5(f, a, c->s.K, c->st);
+    N.sch = f.sch;
+    N.Fhat[a] = F[a];
+    N.flags[a] = f.flags;
+    N.lin[a] = f.lin;
+    N.list[a] = f.list;
+    N.mask[a] = f.mask;
+  }
+  N.U = U;
+  N.P = c->P;
+  N.count = c->count;
+  N.status = c->status;
+  for (int d = 0; d < 3; ++d) {
+    N.n[d] = c->g.n[d];
+    N.bc[d] = c->g.bc[d];
+    N.nface[d] = c->nface[d];
+  }
+  N.ncell = c->ncell;
+  N.gamma = c->g.gamma;
+  N.dim = c->g.dim;
+  if (e == cudaSuccess) {
+    if (lin) {
+      if (c->nv == 3) e = launch_nonlinear_rec_nv3(N, c->s.K, c->s.limiter, c->st);
+      else if (c->nv == 4) e = launch_nonlinear_rec_nv4(N, c->s.K, c->s.limiter, c->st);
+      else e = launch_nonlinear_rec_nv5(N, c->s.K, c->s.limiter, c->st);
+    } else {
+      if (c->nv == 3) e = launch_nonlinear_nv3(N, c->s.K, c->s.limiter, c->st);
+      else if (c->nv == 4) e = launch_nonlinear_nv4(N, c->s.K, c->s.limiter, c->st);
+      else e = launch_nonlinear_nv5(N, c->s.K, c->s.limiter, c->st);
+    }
   }
   if (c->timing) cudaEventRecord(e1, c->st);
   return e;
+}
+
+static PrimOut prim_out(tenom_ctx* c, bool full) {
+  PrimOut o;
+  o.P = c->P;
+  o.count = c->count;
+  o.status = c->status;
+  o.gamma = c->g.gamma;
+  o.full = full ? 1 : 0;
+  return o;
 }
 
 static CellUpdate cell_update_args(tenom_ctx* c, const double* U0, const double* Us, double* out, int mode, double cA,
@@ -629,47 +741,46 @@ static CellUpdate cell_update_args(tenom_ctx* c, const double* U0, const double*
   return u;
 }
 
+/* prims: also the output's primitives (1: for the forward sweeps, 2: full) */
 static cudaError_t launch_stage(tenom_ctx* c, const double* U0, const double* Us, double* out, int mode, double cA,
-                                double cB) {
+                                double cB, int prims = 0) {
   StageArgs a;
   memset(&a, 0, sizeof(a));
+  if (prims) a.po = prim_out(c, prims == 2);
   a.cu = cell_update_args(c, U0, Us, out, mode, cA, cB);
   for (int d = 0; d < 3; ++d) a.n[d] = c->g.n[d];
   a.ncell = c->ncell;
   return launch_stage_kernel(c->nv, a, c->st);
 }
 
-/* the cell primitives of U into c->P (read by the face sweeps of this stage) */
-static cudaError_t launch_prims(tenom_ctx* c, const double* U) {
+/* the cell primitives of U into c->P; clears the list lengths */
+static cudaError_t launch_prims(tenom_ctx* c, const double* U, bool full = false) {
   const unsigned nb = ew_blocks(c->ncell);
-  if (c->nv == 3) prim_kernel<3><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, c->P, c->status);
-  else if (c->nv == 4) prim_kernel<4><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, c->P, c->status);
-  else prim_kernel<5><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, c->P, c->status);
+  const PrimOut o = prim_out(c, full);
+  if (c->nv == 3) prim_kernel<3><<<nb, 256, 0, c->st>>>(U, c->ncell, o);
+  else if (c->nv == 4) prim_kernel<4><<<nb, 256, 0, c->st>>>(U, c->ncell, o);
+  else prim_kernel<5><<<nb, 256, 0, c->st>>>(U, c->ncell, o);
   return cudaGetLastError();
-}
-
-/* face fluxes of every axis at U: the cell primitives once, then one sweep per axis */
-static cudaError_t eval_faces(tenom_ctx* c, const double* U) {
-  cudaError_t e = launch_prims(c, U);
-  for (int a = 0; a < c->g.dim && e == cudaSuccess; ++a) e = launch_faces(c, U, a, c->face[a], nullptr, nullptr, c->P);
-  return e;
 }
 
 tenom_status tenom_rhs(tenom_ctx* c, const double* U, double* dUdt) {
   if (!c) return TENOM_E_INVALID;
   if (!aligned8(U) || !aligned8(dUdt) || U == dUdt) return fail(c, TENOM_E_INVALID, "rhs: bad pointers");
-  cudaError_t e = eval_faces(c, U);
+  cudaError_t e = launch_prims(c, U);
+  if (e == cudaSuccess) e = launch_faces(c, U, 0, c->g.dim, c->face, nullptr, nullptr);
   if (e == cudaSuccess) e = launch_stage(c, nullptr, U, dUdt, 0, 0.0, 0.0);
   return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "rhs");
 }
 
-static cudaError_t launch_signal(tenom_ctx* c, const double* U) {
+static cudaError_t launch_signal(tenom_ctx* c, const double* U, bool prims = false) {
+  PrimOut o = prim_out(c, false);
+  if (!prims) o.P = nullptr;
   unsigned nb = ew_blocks(c->ncell);
   const double* dx = c->g.dx;
   const double r0 = 1.0 / dx[0], r1 = 1.0 / dx[1], r2 = 1.0 / dx[2];
-  if (c->nv == 3) signal_speed_kernel<3><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, r0, r1, r2, c->smax, c->status);
-  else if (c->nv == 4) signal_speed_kernel<4><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, r0, r1, r2, c->smax, c->status);
-  else signal_speed_kernel<5><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, r0, r1, r2, c->smax, c->status);
+  if (c->nv == 3) signal_speed_kernel<3><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, r0, r1, r2, c->smax, c->status, o);
+  else if (c->nv == 4) signal_speed_kernel<4><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, r0, r1, r2, c->smax, c->status, o);
+  else signal_speed_kernel<5><<<nb, 256, 0, c->st>>>(U, c->ncell, c->g.gamma, r0, r1, r2, c->smax, c->status, o);
   return cudaGetLastError();
 }
 
@@ -709,20 +820,20 @@ static cudaError_t launch_positivity(tenom_ctx* c, const double* Us) {
   return e;
 }
 
-/* face fluxes of one SSP-RK3 stage at Us: the high-order fluxes, limited when the scheme
+/* face fluxes of one SSP-RK3 stage at Us (c->P: its primitives): the high-order fluxes, limited when the scheme
    asks for positivity */
 static cudaError_t stage_faces(tenom_ctx* c, const double* Us) {
-  cudaError_t e = eval_faces(c, Us);
+  cudaError_t e = launch_faces(c, Us, 0, c->g.dim, c->face, nullptr, nullptr);
   if (e == cudaSuccess && c->s.positivity == TENOM_PP_ON) e = launch_positivity(c, Us);
   return e;
 }
 
-/* three stages; dt already in c->dt */
+/* three stages; dt already in c->dt, the primitives of U in c->P */
 static cudaError_t rk3_core(tenom_ctx* c, double* U) {
   cudaError_t e = stage_faces(c, U);
-  if (e == cudaSuccess) e = launch_stage(c, nullptr, U, c->W1, 1, 0.0, 1.0);
+  if (e == cudaSuccess) e = launch_stage(c, nullptr, U, c->W1, 1, 0.0, 1.0, 1);
   if (e == cudaSuccess) e = stage_faces(c, c->W1);
-  if (e == cudaSuccess) e = launch_stage(c, U, c->W1, c->W1, 2, 0.75, 0.25);
+  if (e == cudaSuccess) e = launch_stage(c, U, c->W1, c->W1, 2, 0.75, 0.25, 1);
   if (e == cudaSuccess) e = stage_faces(c, c->W1);
   if (e == cudaSuccess) e = launch_stage(c, U, c->W1, U, 2, 1.0 / 3.0, 2.0 / 3.0);
   return e;
@@ -733,6 +844,7 @@ tenom_status tenom_rk3_step(tenom_ctx* c, double* U, const double* dt_dev) {
   if (!aligned8(U) || !aligned8(dt_dev)) return fail(c, TENOM_E_INVALID, "rk3_step: bad pointers");
   cudaError_t e = cudaSuccess;
   if (dt_dev != c->dt) e = cudaMemcpyAsync(c->dt, dt_dev, sizeof(double), cudaMemcpyDeviceToDevice, c->st);
+  if (e == cudaSuccess) e = launch_prims(c, U);
   if (e == cudaSuccess) e = rk3_core(c, U);
   return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "rk3_step");
 }
@@ -742,7 +854,7 @@ tenom_status tenom_advance(tenom_ctx* c, double* U, double* t_dev, double t_end,
   if (!aligned8(U) || !aligned8(t_dev) || !(cfl > 0.0) || nsteps < 0 || !(t_end == t_end))
     return fail(c, TENOM_E_INVALID, "advance: bad arguments");
   for (int k = 0; k < nsteps; ++k) {
-    cudaError_t e = launch_signal(c, U);
+    cudaError_t e = launch_signal(c, U, true);
     if (e == cudaSuccess) {
       finalize_dt_kernel<<<1, 1, 0, c->st>>>(c->smax, cfl, c->dt, t_dev, t_end);
       e = cudaGetLastError();
@@ -792,7 +904,12 @@ tenom_status tenom_face_dump(tenom_ctx* c, const double* U, int axis, double* Fh
   if (!aligned8(U) || !aligned8(Fhat)) return fail(c, TENOM_E_INVALID, "face_dump: bad pointers");
   bool t = c->timing;
   c->timing = false;
-  cudaError_t e = launch_faces(c, U, axis, Fhat, flags);
+  double* F[3] = {nullptr, nullptr, nullptr};
+  uint8_t* fl[3] = {nullptr, nullptr, nullptr};
+  F[axis] = Fhat;
+  fl[axis] = flags;
+  cudaError_t e = launch_prims(c, U);
+  if (e == cudaSuccess) e = launch_faces(c, U, axis, axis + 1, F, fl, nullptr);
   c->timing = t;
   return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "face_dump");
 }
@@ -802,10 +919,9 @@ tenom_status tenom_decision_stats(tenom_ctx* c, const double* U, int axis, unsig
   if (!c) return TENOM_E_INVALID;
   if (axis < 0 || axis >= c->g.dim) return fail(c, TENOM_E_INVALID, "decision_stats: bad axis");
   if (!aligned8(U) || !aligned8(counters_dev)) return fail(c, TENOM_E_INVALID, "decision_stats: bad pointers");
-  cudaError_t e = launch_prims(c, U);
+  cudaError_t e = launch_prims(c, U, true);
   if (e == cudaSuccess) {
     FaceArgs a = face_args(c, U, axis, nullptr, nullptr);
-    a.P = c->P;
     a.stats = counters_dev;
     if (c->nv == 3) e = launch_stats_nv3(a, axis, c->s.K, c->s.limiter, c->st);
     else if (c->nv == 4) e = launch_stats_nv4(a, axis, c->s.K, c->s.limiter, c->st);
@@ -836,6 +952,7 @@ tenom_status tenom_kernel_timing(tenom_ctx* c, int enable, double* face_ms_per_l
       ++n;
     }
   }
+  n *= c->g.dim;  /* a pair of events spans one stage's sweeps of every axis */
   if (face_ms_per_launch) *face_ms_per_launch = n ? tot / n : 0.0;
   if (launches) *launches = n;
   c->ev_used = 0;
@@ -894,7 +1011,7 @@ static size_t lin_offset(const tenom_ctx* c, int axis) {
 static cudaError_t adj_sweeps(tenom_ctx* c, const double* U, const uint8_t* flags_stage, const double* lin_stage,
                               const double* w, double* Z) {
   cudaError_t e = cudaMemsetAsync(Z, 0, sizeof(double) * c->nv * c->ncell, c->st);
-  if (e == cudaSuccess) e = launch_prims(c, U);
+  if (e == cudaSuccess) e = launch_prims(c, U, true);
   for (int a = 0; a < c->g.dim && e == cudaSuccess; ++a) {
     AdjArgs A;
     memset(&A, 0, sizeof(A));
@@ -949,9 +1066,10 @@ tenom_status tenom_rhs_record(tenom_ctx* c, const double* U, double* dUdt, doubl
   if (adjoint_unsupported(c, "rhs_record")) return TENOM_E_UNSUPPORTED;
   if (!aligned8(U) || !aligned8(dUdt) || U == dUdt || !aligned8(lin))
     return fail(c, TENOM_E_INVALID, "rhs_record: bad pointers");
-  cudaError_t e = launch_prims(c, U);
-  for (int a = 0; a < c->g.dim && e == cudaSuccess; ++a)
-    e = launch_faces(c, U, a, c->face[a], nullptr, lin + lin_offset(c, a), c->P);
+  cudaError_t e = launch_prims(c, U, true);
+  double* L[3] = {nullptr, nullptr, nullptr};
+  for (int a = 0; a < c->g.dim; ++a) L[a] = lin + lin_offset(c, a);
+  if (e == cudaSuccess) e = launch_faces(c, U, 0, c->g.dim, c->face, nullptr, L);
   if (e == cudaSuccess) e = launch_stage(c, nullptr, U, dUdt, 0, 0.0, 0.0);
   return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "rhs_record");
 }
@@ -970,15 +1088,19 @@ static cudaError_t rk3_record(tenom_ctx* c, double* U, double* U1, double* U2, u
   const size_t fb = tenom_flags_bytes(c);
   const size_t lb = tenom_lin_tape_bytes(c) / sizeof(double);
   const double* src[3] = {U, U1, U2};
-  cudaError_t e = cudaSuccess;
+  const int prims = lin ? 2 : 1;
+  cudaError_t e = launch_prims(c, U, lin != nullptr);
   for (int st = 0; st < 3 && e == cudaSuccess; ++st) {
-    e = launch_prims(c, src[st]);
-    for (int a = 0; a < c->g.dim && e == cudaSuccess; ++a)
-      e = launch_faces(c, src[st], a, c->face[a], fl ? fl + st * fb + flags_offset(c, a) : nullptr,
-                       lin ? lin + st * lb + lin_offset(c, a) : nullptr, c->P);
+    uint8_t* F[3] = {nullptr, nullptr, nullptr};
+    double* L[3] = {nullptr, nullptr, nullptr};
+    for (int a = 0; a < c->g.dim; ++a) {
+      if (fl) F[a] = fl + st * fb + flags_offset(c, a);
+      if (lin) L[a] = lin + st * lb + lin_offset(c, a);
+    }
+    e = launch_faces(c, src[st], 0, c->g.dim, c->face, fl ? F : nullptr, lin ? L : nullptr);
     if (e != cudaSuccess) break;
-    if (st == 0) e = launch_stage(c, nullptr, U, U1, 1, 0.0, 1.0);
-    else if (st == 1) e = launch_stage(c, U, U1, U2, 2, 0.75, 0.25);
+    if (st == 0) e = launch_stage(c, nullptr, U, U1, 1, 0.0, 1.0, prims);
+    else if (st == 1) e = launch_stage(c, U, U1, U2, 2, 0.75, 0.25, prims);
     else e = launch_stage(c, U, U2, U, 2, 1.0 / 3.0, 2.0 / 3.0);
   }
   return e;

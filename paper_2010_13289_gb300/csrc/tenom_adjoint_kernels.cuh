@@ -7,8 +7,8 @@
  *   rebuilds its frozen linear reconstructions and writes its K x NV point adjoints to its
  *   own shared-memory slots, then each staged point gathers the slots of the faces that
  *   touch it and adds the sum to Z.
- * adj_lin_kernel: from the linearisation the record kernels wrote (field_queue_item in
- *   tenom_face_fwd.cuh gives the tape layout); see the comment above it.
+ * adj_lin_kernel: from the linearisation the record kernels wrote (tenom_nonlinear.cuh gives
+ *   the tape layout); see the comment above it.
  * Z is updated with atomics: halo points are shared with the neighbouring tiles and
  * boundary ghosts fold onto their cell. */
 #pragma once
@@ -20,7 +20,7 @@ struct AdjArgs {
   const double* U;       /* state the operator was applied to [NV][ncell] */
   const uint8_t* flags;  /* forward flags of this axis [nface][NV][2], or null */
   const double* lin;     /* recorded linearisation of this axis [NV][2K+2][nface] (adj_lin_kernel) */
-  const double* P;       /* cell primitives of U [NV + 2][ncell] (velocity, p, H, c, sqrt rho), or null */
+  const double* P;       /* cell primitives of U [NV + 2][ncell] (velocity, p, c, H, sqrt rho), or null */
   const double* w;       /* cell adjoint [NV][ncell] */
   double* Z;             /* accumulated L'^T w [NV][ncell] */
   int* status;
@@ -97,9 +97,9 @@ __device__ __forceinline__ void adj_stage(const AdjArgs& A, const AdjTileMap<NV,
       double vel[NV - 2];
 #pragma unroll
       for (int d = 0; d < NV - 2; ++d) vel[d] = __ldg(A.P + d * A.ncell + cell);
-      stage_point_from<NV, AXIS>(u, vel, __ldg(A.P + (NV - 2) * A.ncell + cell), __ldg(A.P + (NV - 1) * A.ncell + cell),
-                                 __ldg(A.P + NV * A.ncell + cell), __ldg(A.P + (NV + 1) * A.ncell + cell), sm, T::NP,
-                                 p);
+      stage_point_from<NV, AXIS>(u, vel, __ldg(A.P + (NV - 2) * A.ncell + cell), __ldg(A.P + NV * A.ncell + cell),
+                                 __ldg(A.P + (NV - 1) * A.ncell + cell), __ldg(A.P + (NV + 1) * A.ncell + cell), sm,
+                                 T::NP, p);
     } else {
       stage_point<NV, AXIS>(u, A.gamma, sm, T::NP, p, st);
     }

@@ -1,18 +1,18 @@
-/* Fused characteristic face-flux kernel (Section 4 of arXiv 2010.13289: Roe-averaged
- * characteristic decomposition, Rusanov / local Lax-Friedrichs splitting, TENO-M per
- * characteristic field and split side, back-projection).
+/* Tiles, staging and the per-lane face flux shared by the face sweeps (Section 4 of arXiv
+ * 2010.13289: Roe-averaged characteristic decomposition, Rusanov / local Lax-Friedrichs
+ * splitting, TENO-M per characteristic field and split side, back-projection).
  *
- * One CTA owns a tile of consecutive faces along the sweep axis, one thread per face:
+ * A sweep of one axis is screen_kernel (tenom_screen.cuh: the central flux of every face and
+ * the certificate that it is the nonlinear one) followed by nonlinear_kernel
+ * (tenom_nonlinear.cuh: the faces left over).  A CTA owns a tile of consecutive faces along the
+ * sweep axis, one thread per face:
  *   axis x : a run of faces of one row (x is contiguous);
  *   axis y,z: contiguous x-columns (lanes) x faces along the axis.
- * (Tile sizes: FaceTile; forward and record kernels use fx_faces / FWD_LANES.)
- * Phase 1 stages the tile's points (faces + K-1 halo points, boundary condition applied
- * at load: periodic wrap or zero-gradient clamp) with every point quantity they need,
- * once, in shared memory (U, velocity, H, sqrt(rho), p, |u -+ c|; the forward and record
- * kernels add FP32 copies and differences for the screen, tenom_face_fwd.cuh).  Phase 2
- * computes each face flux exactly once and writes it to the face buffer [nvar][nface_a];
- * the cell update (flux difference) reads it later, so both neighbouring cells use the
- * same face value.
+ * (Tile sizes: FaceTile; the screen's tiles use fx_faces / FWD_LANES.)  The tile's points
+ * (faces + K-1 halo points, boundary condition applied at load: periodic wrap or
+ * zero-gradient clamp) are staged in shared memory with every point quantity the faces need.
+ * Each face flux is written once to the face buffer [nvar][nface_a]; the cell update (flux
+ * difference) reads it later, so both neighbouring cells use the same face value.
  */
 #pragma once
 #include <cstdint>
@@ -20,7 +20,6 @@
 #include "tenom_linear.cuh"
 #include "tenom_stats.cuh"
 #include "tenom_fastmath.cuh"
-#include "tenom_face_fwd.cuh"
 
 namespace tenom {
 
@@ -28,8 +27,12 @@ struct FaceArgs {
   const double* U;    /* [NV][ncell] */
   double* Fhat;       /* [NV][nface] */
   uint8_t* flags;     /* [nface][NV][2] or null */
-  const double* P;    /* point primitives [NV + 2][ncell] (velocity, p, H, c, sqrt rho), or null */
+  const double* P;    /* point primitives [NV + 2][ncell] (velocity, p, c, H, sqrt rho), or null; the forward
+                         sweeps read velocity, p and c only */
   double* lin;        /* linearisation [NV][2K+2][nface] (record kernels only) */
+  unsigned* list;     /* screen: faces with an uncertified field ([nface]), the fields (bit s), the count */
+  uint8_t* mask;
+  unsigned* count;
   int* status;        /* sticky status word */
   unsigned long long* stats;  /* decision statistics [SC_COUNT] (statistics kernels only) */
   int n[3];
@@ -48,24 +51,20 @@ struct PointLayout {
   static constexpr int cLm = 3 * NV + 1, cLp = 3 * NV + 2;
 };
 
-constexpr int FX_FACES = 128;  /* faces per CTA, x sweeps */
-/* threads (faces) per CTA of the forward and record kernels: 256 for K = 8 in 2D and 3D
-   (one CTA queue over 8 warps, fewer halo points per face: x sweeps 256 faces of a row,
-   y/z sweeps 16 x columns by 16 faces), 128 for K = 6 and for 1D grids (a short line is
-   latency-bound: it runs faster spread over more, smaller CTAs) */
-__host__ __device__ constexpr int fx_faces(int K, int NV) { return (K == 8 && NV > 3) ? 256 : 128; }
+constexpr int FX_FACES = 128;  /* faces per CTA, x sweeps of the statistics kernels and the adjoint */
+/* threads (faces) per CTA of the screen: 256 in 2D and 3D (x sweeps 256 faces of a row, y/z
+   sweeps 16 x columns by 16 faces: 1.3-1.4 staged points per face), 64 for 1D grids (a short
+   line is latency-bound: it runs faster spread over more, smaller CTAs) */
+__host__ __device__ constexpr int fx_faces(int K, int NV) { return (void)K, NV > 3 ? 256 : 64; }
 /* faces per CTA along the axis of the statistics kernels and the adjoint sweeps, y/z
    (x 32 lanes): 4, i.e. 128-thread CTAs */
 __host__ __device__ constexpr int ft_faces(int K) { return (void)K, 4; }
-/* forward and record kernels, y/z sweeps: FWD_LANES x columns by fx_faces(K, NV) / FWD_LANES
-   faces (a warp takes two face rows): with K = 8 the tile stages 23 rows of 16 points for
-   256 faces (1.4 staged points per face; 11 rows of 32 for 128 faces were 2.75) */
+/* screen, y/z sweeps: FWD_LANES x columns by fx_faces(K, NV) / FWD_LANES faces (a warp takes
+   two face rows) */
 constexpr int FWD_LANES = 16;
-/* resident threads per SM the forward and record kernels are compiled for: 512 (4 CTAs of
-   128 threads or 2 of 256), 128 registers a thread (at most about 100 bytes of spills, at
-   K = 8): the latency-bound kernel gains more from the fourth group of warps than it loses
-   to the spills.  Statistics kernels: 3 CTAs of 128 threads, 168 registers. */
-constexpr int FACE_THREADS_PER_SM = 512;
+/* resident threads per SM the screen is compiled for */
+constexpr int SCREEN_THREADS_PER_SM = 768;
+/* statistics kernels: 3 CTAs of 128 threads, 168 registers */
 constexpr int FACE_CTAS_PER_SM_STATS = 3;
 
 template <int NV, int K, int AXIS, bool FWDT = false>
@@ -78,19 +77,7 @@ struct FaceTile {
   static constexpr int NP = ROWS * LANES;        /* points per tile */
   static constexpr int THREADS = FACES * LANES;
   static constexpr size_t SMEM = sizeof(double) * NC * NP;
-  /* forward and record kernels (FwdFace): their point layout, one field queue per warp,
-     then the FP32 copies of the point data and the queue lengths */
-  static constexpr int NCF = PointLayoutF<NV>::NC;
-  static constexpr size_t FQDOUBLES = (size_t)(THREADS / 32) * FQCAP * fq_rows<NV>();
-  static constexpr size_t SMEM_FWD = sizeof(double) * ((size_t)NCF * NP + FQDOUBLES) +
-                                     sizeof(float) * (size_t)PointLayoutF<NV>::NF * NP + sizeof(int) * (THREADS / 32);
 };
-
-/* dynamic shared memory of face_kernel<..., REC, STATS> */
-template <int NV, int K, int AXIS, bool REC, bool STATS>
-constexpr size_t face_smem() {
-  return !STATS ? FaceTile<NV, K, AXIS, true>::SMEM_FWD : FaceTile<NV, K, AXIS>::SMEM;
-}
 
 __device__ __forceinline__ int bc_wrap(int j, int n, int bc) {
   if (bc == 0) {
@@ -101,10 +88,10 @@ __device__ __forceinline__ int bc_wrap(int j, int n, int bc) {
 }
 
 /* Primitive quantities of one point: velocity, pressure p = (gamma - 1)(E - rho|u|^2/2),
-   total enthalpy H = (E + p)/rho, sound speed c = sqrt(gamma p / rho), sqrt(rho). */
+   sound speed c = sqrt(gamma p / rho). */
 template <int NV>
 __device__ __forceinline__ void point_prims(const double (&u)[NV], double gamma, double (&vel)[NV - 2], double& pr,
-                                            double& Hh, double& c, double& sr, int& st) {
+                                            double& c, int& st) {
   constexpr int D = NV - 2;
   const double rho = u[0];
   const double rinv = rcp_nr(rho);
@@ -116,10 +103,17 @@ __device__ __forceinline__ void point_prims(const double (&u)[NV], double gamma,
   }
   pr = (gamma - 1.0) * (u[NV - 1] - 0.5 * ke);
   c = sqrt(gamma * pr * rinv);
-  Hh = (u[NV - 1] + pr) * rinv;
-  sr = sqrt(rho);
   if (!ipos(rho)) st |= ST_RHO;
   if (!ipos(pr)) st |= ST_P;
+}
+
+/* ... and total enthalpy H = (E + p)/rho, sqrt(rho). */
+template <int NV>
+__device__ __forceinline__ void point_prims(const double (&u)[NV], double gamma, double (&vel)[NV - 2], double& pr,
+                                            double& Hh, double& c, double& sr, int& st) {
+  point_prims<NV>(u, gamma, vel, pr, c, st);
+  Hh = (u[NV - 1] + pr) * rcp_nr(u[0]);
+  sr = sqrt(u[0]);
 }
 
 /* Point quantities of the Euler equations for sweep axis AXIS, written to the tile from U
@@ -324,34 +318,28 @@ __device__ __forceinline__ void face_flux_smem(const double* sm, int NP, int jf,
   }
 }
 
-template <int NV, int K, int LIM, int AXIS, bool REC = false, bool STATS = false>
-__global__ void __launch_bounds__(FaceTile<NV, K, AXIS, !STATS>::THREADS,
-                                  STATS ? FACE_CTAS_PER_SM_STATS : FACE_THREADS_PER_SM / FaceTile<NV, K, AXIS, !STATS>::THREADS)
-face_kernel(const FaceArgs A) {
-  using T = FaceTile<NV, K, AXIS, !STATS>;
-  constexpr int H = T::H;
+/* Decision statistics of the faces of one axis (both split sides of every field in FP64 and
+   certified form), counted into A.stats; A.P holds the full primitives. */
+template <int NV, int K, int LIM, int AXIS>
+__global__ void __launch_bounds__(FaceTile<NV, K, AXIS>::THREADS, FACE_CTAS_PER_SM_STATS)
+stats_kernel(const FaceArgs A) {
+  using T = FaceTile<NV, K, AXIS>;
+  constexpr int H = T::H, D = NV - 2;
   extern __shared__ double sm[];
   const int tid = threadIdx.x;
-
-  /* --- tile coordinates --- */
   const int na = A.n[AXIS];
-  int f0, x0 = 0, o1 = 0, o2 = 0;
+  const int f0 = blockIdx.y * T::FACES;
+  int x0 = 0, o1 = 0, o2 = 0;
   if (AXIS == 0) {
     const int row = blockIdx.x;          /* y + ny * z */
     o1 = row % A.n[1];
     o2 = row / A.n[1];
-    f0 = blockIdx.y * T::FACES;
   } else {
     x0 = blockIdx.x * T::LANES;
-    f0 = blockIdx.y * T::FACES;
     o2 = blockIdx.z;                     /* AXIS 1: z ; AXIS 2: y */
   }
-  const long long sx = 1, sy = A.n[0], sz = (long long)A.n[0] * A.n[1];
-  const long long sa = (AXIS == 0) ? sx : (AXIS == 1 ? sy : sz);
-
-  /* --- phase 1: point quantities --- */
-  constexpr bool FWD = !STATS;  /* forward and record kernels: the screened face flux */
-  float* smf = reinterpret_cast<float*>(sm + (size_t)T::NCF * T::NP + T::FQDOUBLES);  /* forward kernels */
+  const long long sy = A.n[0], sz = (long long)A.n[0] * A.n[1];
+  const long long sa = (AXIS == 0) ? 1 : (AXIS == 1 ? sy : sz);
   int st = 0;
   for (int p = tid; p < T::NP; p += T::THREADS) {
     const int lane = (AXIS == 0) ? 0 : (p % T::LANES);
@@ -365,126 +353,30 @@ face_kernel(const FaceArgs A) {
       base = x + (AXIS == 1 ? sz * o2 : sy * o2);
     }
     const long long cell = base + sa * j;
-    double u[NV];
+    double u[NV], vel[D];
 #pragma unroll
     for (int q = 0; q < NV; ++q) u[q] = __ldg(A.U + q * A.ncell + cell);
-    if constexpr (FWD) {
-      double vel[NV - 2], pr, Hh, cs, sr;
-      if (A.P) {  /* primitives computed once per cell per stage (prim_kernel) */
 #pragma unroll
-        for (int d = 0; d < NV - 2; ++d) vel[d] = __ldg(A.P + d * A.ncell + cell);
-        pr = __ldg(A.P + (NV - 2) * A.ncell + cell);
-        Hh = __ldg(A.P + (NV - 1) * A.ncell + cell);
-        cs = __ldg(A.P + NV * A.ncell + cell);
-        sr = __ldg(A.P + (NV + 1) * A.ncell + cell);
-      } else {
-        point_prims<NV>(u, A.gamma, vel, pr, Hh, cs, sr, st);
-      }
-      stage_point_fwd<NV, AXIS>(u, vel, pr, Hh, cs, sr, sm, smf, T::NP, p);
-    } else if (A.P) {  /* primitives computed once per cell per stage (prim_kernel) */
-      double vel[NV - 2];
-#pragma unroll
-      for (int d = 0; d < NV - 2; ++d) vel[d] = __ldg(A.P + d * A.ncell + cell);
-      stage_point_from<NV, AXIS>(u, vel, __ldg(A.P + (NV - 2) * A.ncell + cell), __ldg(A.P + (NV - 1) * A.ncell + cell),
-                                 __ldg(A.P + NV * A.ncell + cell), __ldg(A.P + (NV + 1) * A.ncell + cell), sm, T::NP,
-                                 p);
-    } else {
-      stage_point<NV, AXIS>(u, A.gamma, sm, T::NP, p, st);
-    }
+    for (int d = 0; d < D; ++d) vel[d] = __ldg(A.P + d * A.ncell + cell);
+    stage_point_from<NV, AXIS>(u, vel, __ldg(A.P + D * A.ncell + cell), __ldg(A.P + (D + 2) * A.ncell + cell),
+                               __ldg(A.P + (D + 1) * A.ncell + cell), __ldg(A.P + (D + 3) * A.ncell + cell), sm, T::NP,
+                               p);
   }
   __syncthreads();
-  int* wq_n = reinterpret_cast<int*>(smf + (size_t)PointLayoutF<NV>::NF * T::NP);  /* forward: queue lengths */
-  if constexpr (FWD) {  /* differences to the next point along the axis, for the screen */
-    for (int p = tid; p < T::NP - T::LANES; p += T::THREADS) stage_differences_fwd<NV, AXIS>(sm, smf, T::NP, p, p + T::LANES);
-    __syncthreads();
-  }
-
-  /* --- phase 2: one face per thread --- */
   const int lane = (AXIS == 0) ? 0 : (tid % T::LANES);
   const int jf = (AXIS == 0) ? tid : (tid / T::LANES);
-  const int f = f0 + jf;
-  const int xg = x0 + lane;
-  /* forward kernels on a periodic axis compute faces 0 .. n-1 only: face n has the same
-     stencil points as face 0, and face 0's lanes write it to both places (face_grid sizes
-     those launches for n faces, which drops the nearly empty last tile of every line) */
-  const bool wrapped = FWD && A.bc[AXIS] == 0;
-  bool active = (wrapped ? f < na : f <= na) && (AXIS == 0 || xg < A.n[0]);
-  const unsigned am = __ballot_sync(0xffffffffu, active);  /* the lanes sharing the warp's queue */
-  unsigned cnt[STATS ? SC_COUNT : 1];
+  unsigned cnt[SC_COUNT];
 #pragma unroll
-  for (int q = 0; q < (STATS ? SC_COUNT : 1); ++q) cnt[q] = 0u;
-  double Fh[NV];
-  /* face linear index (n_a + 1 entries along the axis) */
-  long long flin = 0;
-  if (AXIS == 0) flin = f + (long long)(A.n[0] + 1) * (o1 + (long long)A.n[1] * o2);
-  else if (AXIS == 1) flin = xg + (long long)A.n[0] * (f + (long long)(A.n[1] + 1) * o2);
-  else flin = xg + (long long)A.n[0] * (o2 + (long long)A.n[1] * f);
-  uint8_t* const flg = (active && A.flags) ? A.flags + flin * NV * 2 : nullptr;
-  if constexpr (FWD) {
-    /* screen every field, queue the rest; the CTA works through the queues together (more
-       than one round only when a warp's queue fills) */
-    constexpr int W = T::THREADS / 32;
-    double* const fq0 = sm + (size_t)T::NCF * T::NP;
-    double* const fq = fq0 + (size_t)(tid >> 5) * FQCAP * fq_rows<NV>();
-    FwdFace<NV, K, LIM, AXIS, T::LANES, REC> F;
-    if (active) F.begin(sm, T::NP, jf, lane, A.gamma, st);
-    /* record kernels: the tape row of the face in tile row r, x column x0 + c */
-    auto tape = [&](int r, int c) -> double* {
-      const long long fr = f0 + r, xr = x0 + c;
-      if (AXIS == 0) return A.lin + fr + (long long)(A.n[0] + 1) * (o1 + (long long)A.n[1] * o2);
-      if (AXIS == 1) return A.lin + xr + (long long)A.n[0] * (fr + (long long)(A.n[1] + 1) * o2);
-      return A.lin + xr + (long long)A.n[0] * (o2 + (long long)A.n[1] * fr);
-    };
-    const int rot = (int)((blockIdx.x + blockIdx.y + blockIdx.z) % W);
-    bool again = true;
-#pragma unroll 1
-    while (again) {
-      bool stopped = false;
-      int mine = 0;
-      if (active && F.s_next < NV) {
-        stopped = !F.fields(smf, T::NP, jf, lane, A.sch, flg, fq, am, REC ? A.lin + flin : nullptr, A.nface);
-        mine = F.nq;
-      }
-      const int wn = __reduce_max_sync(0xffffffffu, mine);
-      if ((tid & 31) == 0) wq_n[tid >> 5] = wn;
-      __syncthreads();
-      field_queue_cta<NV, K, LIM, AXIS, T::LANES, T::THREADS, REC>(sm, T::NP, fq0, wq_n, A.sch, st, rot, tape,
-                                                                   A.nface);
-      again = __syncthreads_or(stopped);
-      if (active) F.readback(fq, flg, A.sch);
-    }
-    if (active) F.finish(Fh);
+  for (int q = 0; q < SC_COUNT; ++q) cnt[q] = 0u;
+  if (f0 + jf <= na && (AXIS == 0 || x0 + lane < A.n[0])) {
+    double Fh[NV];
+    face_flux_smem<NV, K, LIM, AXIS, T::LANES, true>(sm, T::NP, jf, lane, A.gamma, A.sch, Fh, nullptr, st, cnt);
   }
-  if (active) {
-    if constexpr (!FWD)
-      face_flux_smem<NV, K, LIM, AXIS, T::LANES, STATS>(sm, T::NP, jf, lane, A.gamma, A.sch, Fh, flg, st, cnt);
-    if constexpr (!STATS) {
+  /* warp sums, one 64-bit atomic per counter and warp */
 #pragma unroll
-      for (int v = 0; v < NV; ++v) A.Fhat[v * A.nface + flin] = Fh[v];
-      if (wrapped && f == 0) {  /* face n of the line */
-        long long fn;
-        if (AXIS == 0) fn = na + (long long)(A.n[0] + 1) * (o1 + (long long)A.n[1] * o2);
-        else if (AXIS == 1) fn = xg + (long long)A.n[0] * (na + (long long)(A.n[1] + 1) * o2);
-        else fn = xg + (long long)A.n[0] * (o2 + (long long)A.n[1] * na);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) A.Fhat[v * A.nface + fn] = Fh[v];
-        if (A.flags) {
-#pragma unroll
-          for (int e = 0; e < 2 * NV; ++e) A.flags[fn * NV * 2 + e] = A.flags[flin * NV * 2 + e];
-        }
-        if constexpr (REC) {  /* the tape rows, complete after the last queue round's barrier */
-#pragma unroll 1
-          for (int r = 0; r < NV * (2 * K + 2); ++r) A.lin[r * A.nface + fn] = A.lin[r * A.nface + flin];
-        }
-      }
-    }
-  }
-  if constexpr (STATS) {  /* warp sums, one 64-bit atomic per counter and warp */
-#pragma unroll
-    for (int q = 0; q < SC_COUNT; ++q) {
-      const unsigned w = __reduce_add_sync(0xffffffffu, cnt[q]);
-      if ((tid & 31) == 0 && w) atomicAdd(A.stats + q, (unsigned long long)w);
-    }
+  for (int q = 0; q < SC_COUNT; ++q) {
+    const unsigned w = __reduce_add_sync(0xffffffffu, cnt[q]);
+    if ((tid & 31) == 0 && w) atomicAdd(A.stats + q, (unsigned long long)w);
   }
   if (st) atomicOr(A.status, st);
 }

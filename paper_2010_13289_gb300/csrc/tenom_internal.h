@@ -5,24 +5,28 @@
 
 namespace tenom {
 
-/* Launch the face kernel of (NV, K, limiter, axis); returns a CUDA error code. */
-cudaError_t launch_face_nv3(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
-cudaError_t launch_face_nv4(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
-cudaError_t launch_face_nv5(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
-/* The same, also writing the face linearisation to a.lin (record kernels). */
-cudaError_t launch_face_rec_nv3(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
-cudaError_t launch_face_rec_nv4(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
-cudaError_t launch_face_rec_nv5(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
-/* The face kernel's decision statistics (tenom_stats.cuh) added to a.stats; no fluxes. */
+struct NonlinArgs;
+/* The screen of one axis (K = 6 or 8), also recording the linearisation when a.lin is set. */
+cudaError_t launch_screen_nv3(const FaceArgs& a, int axis, int K, cudaStream_t st);
+cudaError_t launch_screen_nv4(const FaceArgs& a, int axis, int K, cudaStream_t st);
+cudaError_t launch_screen_nv5(const FaceArgs& a, int axis, int K, cudaStream_t st);
+/* The faces the screens listed, every axis in one launch (K, limiter). */
+cudaError_t launch_nonlinear_nv3(const NonlinArgs& a, int K, int lim, cudaStream_t st);
+cudaError_t launch_nonlinear_nv4(const NonlinArgs& a, int K, int lim, cudaStream_t st);
+cudaError_t launch_nonlinear_nv5(const NonlinArgs& a, int K, int lim, cudaStream_t st);
+/* The same, also writing the linearisation of the listed fields to a.lin (record kernels). */
+cudaError_t launch_nonlinear_rec_nv3(const NonlinArgs& a, int K, int lim, cudaStream_t st);
+cudaError_t launch_nonlinear_rec_nv4(const NonlinArgs& a, int K, int lim, cudaStream_t st);
+cudaError_t launch_nonlinear_rec_nv5(const NonlinArgs& a, int K, int lim, cudaStream_t st);
+/* Decision statistics (tenom_stats.cuh) added to a.stats; no fluxes. */
 cudaError_t launch_stats_nv3(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
 cudaError_t launch_stats_nv4(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
 cudaError_t launch_stats_nv5(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st);
 
 /* Launch geometry of a face sweep (kept in one place for the tests of the host logic):
-   tiles over the n_a + 1 faces of a line, or over n_a faces (wrapped: a forward kernel on
-   a periodic axis, whose face n_a is face 0's copy); fwd_tile: the forward and record
-   kernels' tiles (fx_faces(K, nv) along x; FWD_LANES x columns in y/z), else FX_FACES along x
-   and 32 x columns x ft_faces(K). */
+   tiles over the n_a + 1 faces of a line, or over n_a faces (wrapped: the screen of a
+   periodic axis, whose face n_a is face 0's copy); fwd_tile: the screen's tiles (fx_faces(K, nv)
+   along x; FWD_LANES x columns in y/z), else FX_FACES along x and 32 x columns x ft_faces(K). */
 inline void face_grid(int nv, int axis, const int* n, int K, dim3* grid, dim3* block, bool wrapped = false,
                       bool fwd_tile = false) {
   const int nf = n[axis] + (wrapped ? 0 : 1);

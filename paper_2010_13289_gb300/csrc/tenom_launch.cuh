@@ -7,6 +7,8 @@
 #include <atomic>
 #include <mutex>
 #include "tenom_internal.h"
+#include "tenom_screen.cuh"
+#include "tenom_nonlinear.cuh"
 #include "tenom_adjoint_kernels.cuh"
 
 namespace tenom {
@@ -50,39 +52,85 @@ static cudaError_t launch_tile(Kern kern, AttrOnce& attr, size_t smem, int nv, i
   return cudaLaunchKernel((const void*)kern, grid, block, argv, smem, st);
 }
 
-/* forward face sweep (REC: also record the linearisation; STATS: decision statistics
-   instead of fluxes) */
-template <int NV, int K, int LIM, int AXIS, bool REC, bool STATS>
-static cudaError_t launch_face_one(const FaceArgs& a, cudaStream_t st) {
+/* screen of one axis (REC: also record the linearisation of the certified fields) */
+template <int NV, int K, int AXIS, bool REC>
+static cudaError_t launch_screen_one(const FaceArgs& a, cudaStream_t st) {
   static AttrOnce attr;
-  return launch_tile(face_kernel<NV, K, LIM, AXIS, REC, STATS>, attr, face_smem<NV, K, AXIS, REC, STATS>(), NV, AXIS,
-                     a.n, K, st, &a, !STATS && a.bc[AXIS] == 0, !STATS);
+  return launch_tile(screen_kernel<NV, K, AXIS, REC>, attr, screen_smem<NV, K, AXIS>(), NV, AXIS, a.n, K, st, &a,
+                     a.bc[AXIS] == 0, true);
 }
 
-template <int NV, int AXIS, bool REC, bool STATS>
-static cudaError_t launch_face_axis(const FaceArgs& a, int K, int lim, cudaStream_t st) {
+template <int NV, int K, bool REC>
+static cudaError_t launch_screen_k(const FaceArgs& a, int axis, cudaStream_t st) {
+  if (axis == 0) return launch_screen_one<NV, K, 0, REC>(a, st);
+  if constexpr (NV >= 4)
+    if (axis == 1) return launch_screen_one<NV, K, 1, REC>(a, st);
+  if constexpr (NV >= 5)
+    if (axis == 2) return launch_screen_one<NV, K, 2, REC>(a, st);
+  return cudaErrorNotSupported;
+}
+
+template <int NV>
+static cudaError_t launch_screen_nv(const FaceArgs& a, int axis, int K, cudaStream_t st) {
+  if (K == 6) return a.lin ? launch_screen_k<NV, 6, true>(a, axis, st) : launch_screen_k<NV, 6, false>(a, axis, st);
+  return a.lin ? launch_screen_k<NV, 8, true>(a, axis, st) : launch_screen_k<NV, 8, false>(a, axis, st);
+}
+
+/* the listed faces of every axis */
+template <int NV, int K, int LIM, bool REC>
+static cudaError_t launch_nonlinear_one(const NonlinArgs& a, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  nonlinear_kernel<NV, K, LIM, REC><<<sms * NL_CTAS_PER_SM, NL_THREADS, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <int NV, int K, bool REC>
+static cudaError_t launch_nonlinear_k(const NonlinArgs& a, int lim, cudaStream_t st) {
+  if (lim == LIM_MP) return launch_nonlinear_one<NV, K, LIM_MP, REC>(a, st);
+  if (lim == LIM_TVD5) return launch_nonlinear_one<NV, K, LIM_TVD5, REC>(a, st);
+  if constexpr (!REC)  /* Van Albada: forward only (no frozen linear form to record) */
+    if (lim == LIM_VA) return launch_nonlinear_one<NV, K, LIM_VA, false>(a, st);
+  return cudaErrorNotSupported;
+}
+
+template <int NV, bool REC>
+static cudaError_t launch_nonlinear_nv(const NonlinArgs& a, int K, int lim, cudaStream_t st) {
+  if (K == 6) return launch_nonlinear_k<NV, 6, REC>(a, lim, st);
+  if (K == 8) return launch_nonlinear_k<NV, 8, REC>(a, lim, st);
+  return cudaErrorNotSupported;
+}
+
+/* decision statistics */
+template <int NV, int K, int LIM, int AXIS>
+static cudaError_t launch_stats_one(const FaceArgs& a, cudaStream_t st) {
+  static AttrOnce attr;
+  return launch_tile(stats_kernel<NV, K, LIM, AXIS>, attr, FaceTile<NV, K, AXIS>::SMEM, NV, AXIS, a.n, K, st, &a);
+}
+
+template <int NV, int AXIS>
+static cudaError_t launch_stats_axis(const FaceArgs& a, int K, int lim, cudaStream_t st) {
   if (K == 6) {
-    if (lim == LIM_MP) return launch_face_one<NV, 6, LIM_MP, AXIS, REC, STATS>(a, st);
-    if (lim == LIM_TVD5) return launch_face_one<NV, 6, LIM_TVD5, AXIS, REC, STATS>(a, st);
-    if constexpr (!REC)  /* Van Albada: forward only (no frozen linear form to record) */
-      if (lim == LIM_VA) return launch_face_one<NV, 6, LIM_VA, AXIS, false, STATS>(a, st);
+    if (lim == LIM_MP) return launch_stats_one<NV, 6, LIM_MP, AXIS>(a, st);
+    if (lim == LIM_TVD5) return launch_stats_one<NV, 6, LIM_TVD5, AXIS>(a, st);
+    if (lim == LIM_VA) return launch_stats_one<NV, 6, LIM_VA, AXIS>(a, st);
   } else if (K == 8) {
-    if (lim == LIM_MP) return launch_face_one<NV, 8, LIM_MP, AXIS, REC, STATS>(a, st);
-    if (lim == LIM_TVD5) return launch_face_one<NV, 8, LIM_TVD5, AXIS, REC, STATS>(a, st);
-    if constexpr (!REC)
-      if (lim == LIM_VA) return launch_face_one<NV, 8, LIM_VA, AXIS, false, STATS>(a, st);
+    if (lim == LIM_MP) return launch_stats_one<NV, 8, LIM_MP, AXIS>(a, st);
+    if (lim == LIM_TVD5) return launch_stats_one<NV, 8, LIM_TVD5, AXIS>(a, st);
+    if (lim == LIM_VA) return launch_stats_one<NV, 8, LIM_VA, AXIS>(a, st);
   }
   return cudaErrorNotSupported;
 }
 
-template <int NV, bool REC, bool STATS = false>
-static cudaError_t launch_face_nv(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st) {
-  static_assert(!(REC && STATS), "statistics kernels do not record");
-  if (axis == 0) return launch_face_axis<NV, 0, REC, STATS>(a, K, lim, st);
+template <int NV>
+static cudaError_t launch_stats_nv(const FaceArgs& a, int axis, int K, int lim, cudaStream_t st) {
+  if (axis == 0) return launch_stats_axis<NV, 0>(a, K, lim, st);
   if constexpr (NV >= 4)
-    if (axis == 1) return launch_face_axis<NV, 1, REC, STATS>(a, K, lim, st);
+    if (axis == 1) return launch_stats_axis<NV, 1>(a, K, lim, st);
   if constexpr (NV >= 5)
-    if (axis == 2) return launch_face_axis<NV, 2, REC, STATS>(a, K, lim, st);
+    if (axis == 2) return launch_stats_axis<NV, 2>(a, K, lim, st);
   return cudaErrorNotSupported;
 }
 

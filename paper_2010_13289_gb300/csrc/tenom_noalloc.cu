@@ -9,11 +9,16 @@
 
 #include "tenom.h"
 #include "tenom_internal.h"
+#include "tenom_nonlinear.cuh"
 
 namespace tenom {
 
-/* first 256 bytes: status word; then the face buffers, axis after axis */
-static __device__ __align__(256) double g_noalloc_scratch[TENOM_NOALLOC_SCRATCH_BYTES / sizeof(double)];
+/* first 256 bytes: status word, list lengths; then the face buffers, axis after axis; after
+   TENOM_NOALLOC_SCRATCH_BYTES the face lists of the nonlinear kernel: 5 bytes per face, at most
+   (16 MiB / 8) / 3 faces (1D), 3.4 MiB */
+static constexpr size_t kListBytes = 4u << 20;
+static __device__ __align__(256) double g_noalloc_scratch[(TENOM_NOALLOC_SCRATCH_BYTES + kListBytes) / sizeof(double)];
+static_assert(5 * (TENOM_NOALLOC_SCRATCH_BYTES / sizeof(double) / 3 + 1) + 64 <= kListBytes, "face lists fit");
 
 static constexpr long long kStatusDoubles = 256 / sizeof(double);
 static constexpr int kMaxDevices = 64;
@@ -80,10 +85,9 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
   }
   cudaStream_t st = (cudaStream_t)stream;
   int* status = status_dev ? status_dev : reinterpret_cast<int*>(scratch);
-  if (!status_dev) {
-    e = cudaMemsetAsync(status, 0, sizeof(int), st);  /* the shared word keeps the last call's bits */
-    if (e != cudaSuccess) return TENOM_E_CUDA;
-  }
+  unsigned* count = reinterpret_cast<unsigned*>(scratch) + 16;
+  e = cudaMemsetAsync(scratch, 0, 256, st);  /* the shared status word and the list lengths keep the last call's values */
+  if (e != cudaSuccess) return TENOM_E_CUDA;
   double* F[3] = {nullptr, nullptr, nullptr};
   long long off = kStatusDoubles;
   for (int a = 0; a < grid->dim; ++a) {
@@ -102,12 +106,41 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
   fa.ncell = ncell;
   fa.gamma = grid->gamma;
   fa.sch = scheme_for_device(*scheme);
+  NonlinArgs na;
+  memset(&na, 0, sizeof(na));
+  unsigned* list = reinterpret_cast<unsigned*>(scratch + cap);
+  uint8_t* mask = reinterpret_cast<uint8_t*>(list + nface[0] + nface[1] + nface[2]);
   for (int a = 0; a < grid->dim && e == cudaSuccess; ++a) {
     fa.Fhat = F[a];
     fa.nface = nface[a];
-    if (nv == 3) e = launch_face_nv3(fa, a, scheme->K, scheme->limiter, st);
-    else if (nv == 4) e = launch_face_nv4(fa, a, scheme->K, scheme->limiter, st);
-    else e = launch_face_nv5(fa, a, scheme->K, scheme->limiter, st);
+    fa.list = list;
+    fa.mask = mask;
+    fa.count = count + a;
+    list += nface[a];
+    mask += nface[a];
+    if (nv == 3) e = launch_screen_nv3(fa, a, scheme->K, st);
+    else if (nv == 4) e = launch_screen_nv4(fa, a, scheme->K, st);
+    else e = launch_screen_nv5(fa, a, scheme->K, st);
+    na.Fhat[a] = F[a];
+    na.list[a] = fa.list;
+    na.mask[a] = fa.mask;
+  }
+  na.U = U;
+  na.count = count;
+  na.status = status;
+  for (int d = 0; d < 3; ++d) {
+    na.n[d] = fa.n[d];
+    na.bc[d] = fa.bc[d];
+    na.nface[d] = nface[d];
+  }
+  na.ncell = ncell;
+  na.gamma = fa.gamma;
+  na.dim = grid->dim;
+  na.sch = fa.sch;
+  if (e == cudaSuccess) {
+    if (nv == 3) e = launch_nonlinear_nv3(na, scheme->K, scheme->limiter, st);
+    else if (nv == 4) e = launch_nonlinear_nv4(na, scheme->K, scheme->limiter, st);
+    else e = launch_nonlinear_nv5(na, scheme->K, scheme->limiter, st);
   }
   if (e == cudaSuccess) e = launch_rhs_divergence(nv, F, grid->n, grid->dx, ncell, nface, dUdt, st);
   if (e != cudaSuccess) {
