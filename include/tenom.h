@@ -212,7 +212,8 @@ tenom_status tenom_batch_autotune(tenom_batch* b, double* U, int* tile, int* cta
 tenom_status tenom_batch_set_tiling(tenom_batch* b, int tile, int ctas_per_sm);
 
 /* Size of the static device scratch for the face fluxes of tenom_rhs_noalloc: 16 MiB, held on
- * every GPU that loads this library until the process exits (with 4 MiB more for the face lists). */
+ * every GPU that loads this library until the process exits (with 20 MiB more for the face lists and the
+ * cell primitives). */
 #define TENOM_NOALLOC_SCRATCH_BYTES (16u << 20)
 
 /* tenom_rhs without a context and without any device allocation.  The paper has no
@@ -220,13 +221,8 @@ tenom_status tenom_batch_set_tiling(tenom_batch* b, int tile, int ctas_per_sm);
  * once they are running -- code living inside another framework's memory pool or
  * allocator hook, or a latency-critical loop that cannot accept the implicit device
  * synchronisation of cudaMalloc/cudaFree.  It computes dUdt = L(U) for the given grid and
- * scheme, on `stream` (a cudaStream_t; NULL = legacy default stream), with the face-sweep
- * and flux-difference kernels of tenom_rhs.  One difference: tenom_rhs first computes the
- * cells' primitives (velocity, p, H, c, sqrt rho) once per cell into its context's
- * buffer, while this call has no such buffer and the sweep kernels form them for each
- * staged point of their tile; the two round alike except in the last bits, which can
- * flip a cutoff decision that rounding sets (a flat sequence at a zero-gradient boundary);
- * agreement to 1e-13 of each component's largest value is tested.  U and dUdt are caller-owned device arrays as for tenom_rhs; status_dev
+ * scheme, on `stream` (a cudaStream_t; NULL = legacy default stream), with the kernels of
+ * tenom_rhs: agreement to 1e-13 of each component's largest value is tested.  U and dUdt are caller-owned device arrays as for tenom_rhs; status_dev
  * is an optional caller-owned device int that receives TENOM_ST_* bits (ORed in, the
  * caller clears it); with NULL the bits go to a word inside the scratch and are not
  * reported.

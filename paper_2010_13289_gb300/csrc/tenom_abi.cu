@@ -464,6 +464,13 @@ static SchemeDev scheme_dev(const tenom_scheme& s) {
   };
   d.quick_r[0] = ratio(s.ct_mode == TENOM_CT_ADAPTIVE ? 1e-7 : s.ct_const);
   d.quick_r[1] = ratio(1e-10);
+  const double b3 = s.mp_beta / 3.0;
+  d.fixed = d.default_d && s.weights == TENOM_W_TENOM && (s.limiter == TENOM_LIM_MP || s.limiter == TENOM_LIM_TVD5) &&
+            s.mp_alpha >= 0.0 && s.mp_alpha < 8.0 && b3 >= 0.0 && b3 < 8.0;
+  if (d.fixed) {
+    d.alpha_q60 = (long long)(s.mp_alpha * 1152921504606846976.0);
+    d.beta_third_q60 = (long long)(b3 * 1152921504606846976.0);
+  }
   return d;
 }
 
@@ -696,6 +703,7 @@ static cudaError_t launch_faces(tenom_ctx* c, const double* U, int a0, int a1, d
   }
   N.ncell = c->ncell;
   N.gamma = c->g.gamma;
+  N.rgm1 = 1.0 / (c->g.gamma - 1.0);
   N.dim = c->g.dim;
   if (e == cudaSuccess) {
     if (lin) {
@@ -753,14 +761,17 @@ static cudaError_t launch_stage(tenom_ctx* c, const double* U0, const double* Us
   return launch_stage_kernel(c->nv, a, c->st);
 }
 
+static cudaError_t launch_prim_kernel(int nv, const double* U, long long ncell, const PrimOut& o, cudaStream_t st) {
+  const unsigned nb = ew_blocks(ncell);
+  if (nv == 3) prim_kernel<3><<<nb, 256, 0, st>>>(U, ncell, o);
+  else if (nv == 4) prim_kernel<4><<<nb, 256, 0, st>>>(U, ncell, o);
+  else prim_kernel<5><<<nb, 256, 0, st>>>(U, ncell, o);
+  return cudaGetLastError();
+}
+
 /* the cell primitives of U into c->P; clears the list lengths */
 static cudaError_t launch_prims(tenom_ctx* c, const double* U, bool full = false) {
-  const unsigned nb = ew_blocks(c->ncell);
-  const PrimOut o = prim_out(c, full);
-  if (c->nv == 3) prim_kernel<3><<<nb, 256, 0, c->st>>>(U, c->ncell, o);
-  else if (c->nv == 4) prim_kernel<4><<<nb, 256, 0, c->st>>>(U, c->ncell, o);
-  else prim_kernel<5><<<nb, 256, 0, c->st>>>(U, c->ncell, o);
-  return cudaGetLastError();
+  return launch_prim_kernel(c->nv, U, c->ncell, prim_out(c, full), c->st);
 }
 
 tenom_status tenom_rhs(tenom_ctx* c, const double* U, double* dUdt) {
@@ -1243,6 +1254,17 @@ SchemeDev scheme_for_device(const tenom_scheme& s) {
   if (!anyd)
     for (int k = 0; k < t.K - 2; ++k) t.d[k] = (t.K == 6) ? kDopt6[k] : kDopt8[k];
   return scheme_dev(t);
+}
+
+cudaError_t launch_primitives(int nv, const double* U, long long ncell, double gamma, double* P, unsigned* count,
+                              int* status, cudaStream_t st) {
+  PrimOut o;
+  o.P = P;
+  o.count = count;
+  o.status = status;
+  o.gamma = gamma;
+  o.full = 0;
+  return launch_prim_kernel(nv, U, ncell, o, st);
 }
 
 cudaError_t launch_rhs_divergence(int nv, double* const F[3], const int n[3], const double dx[3], long long ncell,

@@ -27,13 +27,13 @@ struct FaceArgs {
   const double* U;    /* [NV][ncell] */
   double* Fhat;       /* [NV][nface] */
   uint8_t* flags;     /* [nface][NV][2] or null */
-  const double* P;    /* point primitives [NV + 2][ncell] (velocity, p, c, H, sqrt rho), or null; the forward
-                         sweeps read velocity, p and c only */
+  const double* P;    /* point primitives [NV + 2][ncell] (velocity, p, c, H, sqrt rho); the screen reads
+                         velocity, p and c only */
   double* lin;        /* linearisation [NV][2K+2][nface] (record kernels only) */
   unsigned* list;     /* screen: faces with an uncertified field ([nface]), the fields (bit s), the count */
   uint8_t* mask;
   unsigned* count;
-  int* status;        /* sticky status word */
+  int* status;        /* sticky status word (statistics) */
   unsigned long long* stats;  /* decision statistics [SC_COUNT] (statistics kernels only) */
   int n[3];
   int bc[3];
@@ -80,6 +80,7 @@ struct FaceTile {
 };
 
 __device__ __forceinline__ int bc_wrap(int j, int n, int bc) {
+  if (j >= 0 && j < n) return j;
   if (bc == 0) {
     j %= n;
     return j < 0 ? j + n : j;

@@ -53,6 +53,10 @@ namespace tenom {
 tenom_status check_grid_scheme(const tenom_grid* g, const tenom_scheme* s, std::string* msg);
 /* Device copy of a scheme (all-zero d_k replaced by the maximal-order weights). */
 SchemeDev scheme_for_device(const tenom_scheme& s);
+/* The forward sweeps' cell primitives of U (velocity, p, c: [nv][ncell]) into P; clears the three
+   list lengths at count. */
+cudaError_t launch_primitives(int nv, const double* U, long long ncell, double gamma, double* P, unsigned* count,
+                              int* status, cudaStream_t st);
 /* dUdt = -sum_a (F_a[f+1] - F_a[f]) / dx_a from face buffers F[a] ([nv][nface_a]). */
 cudaError_t launch_rhs_divergence(int nv, double* const F[3], const int n[3], const double dx[3], long long ncell,
                                   const long long nface[3], double* out, cudaStream_t st);

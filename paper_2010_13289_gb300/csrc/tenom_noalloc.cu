@@ -14,10 +14,11 @@
 namespace tenom {
 
 /* first 256 bytes: status word, list lengths; then the face buffers, axis after axis; after
-   TENOM_NOALLOC_SCRATCH_BYTES the face lists of the nonlinear kernel: 5 bytes per face, at most
-   (16 MiB / 8) / 3 faces (1D), 3.4 MiB */
+   TENOM_NOALLOC_SCRATCH_BYTES the face lists of the nonlinear kernel (5 bytes per face, at most
+   (16 MiB / 8) / 3 faces in 1D, 3.4 MiB) and the cell primitives (nvar values per cell, never
+   more than the face fluxes) */
 static constexpr size_t kListBytes = 4u << 20;
-static __device__ __align__(256) double g_noalloc_scratch[(TENOM_NOALLOC_SCRATCH_BYTES + kListBytes) / sizeof(double)];
+static __device__ __align__(256) double g_noalloc_scratch[(2 * TENOM_NOALLOC_SCRATCH_BYTES + kListBytes) / sizeof(double)];
 static_assert(5 * (TENOM_NOALLOC_SCRATCH_BYTES / sizeof(double) / 3 + 1) + 64 <= kListBytes, "face lists fit");
 
 static constexpr long long kStatusDoubles = 256 / sizeof(double);
@@ -86,8 +87,11 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
   cudaStream_t st = (cudaStream_t)stream;
   int* status = status_dev ? status_dev : reinterpret_cast<int*>(scratch);
   unsigned* count = reinterpret_cast<unsigned*>(scratch) + 16;
-  e = cudaMemsetAsync(scratch, 0, 256, st);  /* the shared status word and the list lengths keep the last call's values */
-  if (e != cudaSuccess) return TENOM_E_CUDA;
+  if (!status_dev) {
+    e = cudaMemsetAsync(status, 0, sizeof(int), st);  /* the shared word keeps the last call's bits */
+    if (e != cudaSuccess) return TENOM_E_CUDA;
+  }
+  double* P = scratch + cap + kListBytes / sizeof(double);
   double* F[3] = {nullptr, nullptr, nullptr};
   long long off = kStatusDoubles;
   for (int a = 0; a < grid->dim; ++a) {
@@ -97,6 +101,7 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
   FaceArgs fa;
   memset(&fa, 0, sizeof(fa));
   fa.U = U;
+  fa.P = P;
   fa.flags = nullptr;
   fa.status = status;
   for (int d = 0; d < 3; ++d) {
@@ -106,6 +111,7 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
   fa.ncell = ncell;
   fa.gamma = grid->gamma;
   fa.sch = scheme_for_device(*scheme);
+  e = launch_primitives(nv, U, ncell, grid->gamma, P, count, status, st);  /* clears the list lengths */
   NonlinArgs na;
   memset(&na, 0, sizeof(na));
   unsigned* list = reinterpret_cast<unsigned*>(scratch + cap);
@@ -126,6 +132,7 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
     na.mask[a] = fa.mask;
   }
   na.U = U;
+  na.P = P;
   na.count = count;
   na.status = status;
   for (int d = 0; d < 3; ++d) {
@@ -135,6 +142,7 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
   }
   na.ncell = ncell;
   na.gamma = fa.gamma;
+  na.rgm1 = 1.0 / (fa.gamma - 1.0);
   na.dim = grid->dim;
   na.sch = fa.sch;
   if (e == cudaSuccess) {

@@ -7,22 +7,36 @@
  * speeds; (1) the uncertified (face, field) pairs of the chunk, ordered by field so that a
  * warp mostly runs one kind of projection, are spread over the CTA's threads: projection of
  * the K points, decisions and reconstruction of both split sides; (2) a thread per face
- * composes the flux from those fields and from l_s . Fc of the certified ones.  The list is
- * dense, so every step runs in full warps whatever share of the faces needs it; when there
+ * composes the flux.  The list is dense, so every step runs in full warps whatever share of the faces needs it; when there
  * are few faces a chunk is smaller, so that they spread over all SMs.
  *
  * The kernel is written in the axis's own frame: component 1 is the momentum along the axis,
  * 2 .. NV-2 the tangential ones in increasing axis order (fields: 0 u-c, 1 entropy,
- * 2 .. NV-2 shear, NV-1 u+c). */
+ * 2 .. NV-2 shear, NV-1 u+c).
+ *
+ * FIX: a nonsmooth side only adds its limiter's correction sum_k d_k (limited_k - f_k), in fixed
+ * point (tenom_fixed.cuh), and the face flux is Fc + sum_s r_s correction_s (the smooth part of
+ * every field sums to Fc, R L = I): what is left of FP64 per field is the projection, in full
+ * warps, whatever the decisions.  A side whose two centre values are below 2^-10 of the
+ * stencil's largest (a contaminated candidate would leave its rounding on a far smaller flux)
+ * and values outside the fixed-point range take the general FP64 reconstruction, as do all
+ * other schemes (!FIX).
+ *
+ * What bounds it (ncu, 64^3 turbulence TENO8, 4 of 5 fields of 98 % of the faces listed): FP64
+ * pipe 69 % busy, then waiting at the CTA's barriers.  Per 3-sweep launch 2.9 ms in FP64 (the
+ * limiter's divergent lanes and, for any lane the FP32 filter left undecided, the whole warp in
+ * FP64 decisions), 1.9 ms with fixed-point corrections and the second pass, 1.45 ms with the
+ * rolled loops and called rare paths (instruction fetch had been the largest stall). */
 #pragma once
 #include "tenom_recon.cuh"
 #include "tenom_face.cuh"
+#include "tenom_fixed.cuh"
 
 namespace tenom {
 
 struct NonlinArgs {
   const double* U;           /* [NV][ncell] */
-  const double* P;           /* cell primitives (velocity, p, c, ..), or null: formed here */
+  const double* P;           /* cell primitives (velocity, p, c, ..) */
   double* Fhat[3];           /* face fluxes per axis, holding Fc of every face */
   uint8_t* flags[3];         /* [nface][NV][2] or null */
   double* lin[3];            /* linearisation (record kernels) */
@@ -35,6 +49,7 @@ struct NonlinArgs {
   long long ncell;
   long long nface[3];
   double gamma;
+  double rgm1;               /* 1 / (gamma - 1) */
   int dim;
   SchemeDev sch;
 };
@@ -50,7 +65,117 @@ struct NlRow {
                        N = D + 8;
 };
 
-template <int NV, int K, int LIM, bool REC>
+/* bc_wrap for a point at most half a stencil outside the line (a periodic line has at least
+   K/2 cells) */
+__device__ __forceinline__ int bc_near(int j, int n, int bc) {
+  if (bc == 0) return j < 0 ? j + n : (j >= n ? j - n : j);
+  return j < 0 ? 0 : (j >= n ? n - 1 : j);
+}
+
+/* The rare FP64 paths of the fixed-point kernel, called rather than inlined: they are larger
+   than the path every item takes, and instruction fetch is what that path waits for.  w, g: the
+   item's W and G/2 of point q at q * NL_THREADS; side 1: the mirrored stencil of f-. */
+template <int K>
+__device__ __forceinline__ void split_side(const double* w, const double* g, double ha, int side, double (&v)[K]) {
+#pragma unroll
+  for (int q = 0; q < K; ++q) {
+    const int p = (side ? K - 1 - q : q) * NL_THREADS;
+    v[q] = fma(side ? -ha : ha, w[p], g[p]);
+  }
+}
+template <int K>
+__device__ __noinline__ unsigned decide_cold(const double* w, const double* g, double ha, int side, const SchemeDev& S,
+                                             int& st) {
+  double v[K];
+  split_side<K>(w, g, ha, side, v);
+  unsigned b;
+  int e;
+  teno_decide_fp64<K>(v, S, b, e, st);
+  return b | ((unsigned)((e - 7) & 3) << 6);
+}
+template <int K, int LIM>
+__device__ __noinline__ double general_cold(const double* w, const double* g, double ha, unsigned fl, const SchemeDev& S) {
+  constexpr unsigned allk = (1u << (K - 2)) - 1u;
+  double f = 0.0;
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    double v[K];
+    split_side<K>(w, g, ha, side, v);
+    f += teno_general<K, LIM>(v, S, fl >> (8 * side) & allk);
+  }
+  return f;
+}
+
+/* Both split sides of an item from its projected W and G/2 (columns w, g in shared memory):
+   decisions, and the corrections of the nonsmooth sides in fixed point.  Returns false when the
+   FP32 filter leaves a side undecided and `defer` is set.  Dx: K - 1 scratch words of the item's
+   thread.  em: biased exponent of a power of two above every |G/2| + |alpha W/2|.  The loops over
+   the points are rolled and everything rare is called, to keep the code that an item runs
+   small (unrolled 4 or 8 times: 256^3 step 64 ms against 59, 64^3 turbulence 5.6 against 5.1). */
+template <int K, int LIM>
+__device__ __forceinline__ bool fixed_item(const double* w, const double* g, double ha, int em, long long* Dx,
+                                           const SchemeDev& S, bool defer, unsigned& fl, double& fsum, bool& direct,
+                                           int& st) {
+  constexpr int c = K / 2 - 1, TH = NL_THREADS;
+  constexpr unsigned allk = (1u << (K - 2)) - 1u;
+  const bool inside = em >= 1023 - 40 && em <= 1023 + 40;
+  const float unit = __int_as_float((inside ? em - 1076 + 127 : 0) << 23);  /* 2^(em - 1076) */
+  Acc96 acc;
+  fl = 0u;
+  direct = false;
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    unsigned zero = 0u;
+    int ec = 0, es;  /* exponents of the larger of the two centre values and of the side's largest */
+    auto expo = [](double x) -> int { return (int)((unsigned)__double2hiint(x) >> 20 & 0x7ffu); };
+    {
+      const int p0 = side ? (K - 1) * TH : 0, dp = side ? -TH : TH;
+      const double hs = side ? -ha : ha;
+      double v0 = fma(hs, w[p0], g[p0]);
+      long long x0 = to_fixed(v0, em);
+      es = expo(v0);
+#pragma unroll 1
+      for (int t = 0; t < K - 1; ++t) {
+        const int p = p0 + (t + 1) * dp;
+        const double v1 = fma(hs, w[p], g[p]);
+        const long long x1 = to_fixed(v1, em);
+        Dx[t * TH] = x1 - x0;
+        zero |= dbits(v1) == dbits(v0) ? 1u << t : 0u;
+        es = max(es, expo(v1));
+        if (t == c) ec = max(expo(v0), expo(v1));
+        x0 = x1;
+        v0 = v1;
+      }
+    }
+    float d[K - 1];
+#pragma unroll
+    for (int t = 0; t < K - 1; ++t) d[t] = __ll2float_rz(Dx[t * TH]) * unit;
+    unsigned b = 0;
+    int e = 7;
+    if (S.exact_decisions || !inside || !cutoff_filter<K>(d, 1.01f * unit, zero, S, b, e)) {
+      if (defer) return false;
+      const unsigned f = decide_cold<K>(w, g, ha, side, S, st);
+      b = f & allk;
+      e = 7 + (int)(f >> 6);
+    }
+    fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
+    if (b != allk) {
+      if (!inside || ec < es - 10) {
+        direct = true;
+      } else {
+        long long D[K - 1];
+#pragma unroll
+        for (int t = 0; t < K - 1; ++t) D[t] = Dx[t * TH];
+        fixed_correction<K, LIM>(D, b, S, acc);
+      }
+    }
+  }
+  fsum = direct ? general_cold<K, LIM>(w, g, ha, fl, S)
+                : acc.value() * (__hiloint2double((em - 1076 + 1023) << 20, 0) * (1.0 / fixed_den<K, LIM>()));
+  return true;
+}
+
+template <int NV, int K, int LIM, bool REC, bool FIX>
 __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(const NonlinArgs A) {
   using R = NlRow<NV>;
   constexpr int D = NV - 2, H = K / 2, TH = NL_THREADS, W = TH / 32;
@@ -60,7 +185,12 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
   __shared__ long long s_base[TH];
   __shared__ int s_f[TH];
   __shared__ unsigned s_cm[TH];             /* certified and found-central fields */
+  __shared__ unsigned s_dir[TH];            /* fields whose s_fs is f+ + f- (else the correction to l_s . Fc) */
   __shared__ unsigned short s_item[NV * TH];
+  __shared__ unsigned short s_later[FIX ? NV * TH : 1];
+  __shared__ double s_w[FIX ? K * TH : 1], s_g[FIX ? K * TH : 1];  /* an item's W and G/2 */
+  __shared__ long long s_D[FIX ? (K - 1) * TH : 1];
+  __shared__ int s_nlater;
   __shared__ int s_wc[NV * W + 1];
   const int tid = threadIdx.x, wid = tid >> 5, ln = tid & 31;
   int st = 0;
@@ -71,15 +201,16 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
     cnt[a] = c < A.nface[a] ? c : A.nface[a];
     total += cnt[a];
   }
-  long long chunk = (total + gridDim.x - 1) / gridDim.x;
-  chunk = chunk < 8 ? 8 : (chunk > TH ? TH : chunk);
-  const long long nch0 = (cnt[0] + chunk - 1) / chunk, nch1 = (cnt[1] + chunk - 1) / chunk,
-                  nch2 = (cnt[2] + chunk - 1) / chunk;
+  /* faces per chunk: NL_THREADS, or fewer (8 at least) when that leaves CTAs without one */
+  int sh = 7;
+  while (sh > 3 && (total >> sh) < gridDim.x) --sh;
+  const long long chunk = 1ll << sh;
+  const long long nch0 = (cnt[0] + chunk - 1) >> sh, nch1 = (cnt[1] + chunk - 1) >> sh, nch2 = (cnt[2] + chunk - 1) >> sh;
 
 #pragma unroll 1
   for (long long ch = blockIdx.x; ch < nch0 + nch1 + nch2; ch += gridDim.x) {
     const int ax = ch < nch0 ? 0 : (ch < nch0 + nch1 ? 1 : 2);
-    const long long i0 = (ch - (ax == 0 ? 0 : (ax == 1 ? nch0 : nch0 + nch1))) * chunk;
+    const long long i0 = (ch - (ax == 0 ? 0 : (ax == 1 ? nch0 : nch0 + nch1))) << sh;
     const int nf = (int)((cnt[ax] - i0) < chunk ? (cnt[ax] - i0) : chunk);  /* faces of this chunk */
     const int na = A.n[ax], bc = A.bc[ax];
     const long long sa = ax == 0 ? 1 : (ax == 1 ? (long long)A.n[0] : (long long)A.n[0] * A.n[1]);
@@ -94,23 +225,9 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
     const double* up[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) up[v] = A.U + gc(v) * A.ncell;
-    const double* const Pn = A.P ? A.P + ax * A.ncell : nullptr;
-    const double* const Pp = A.P ? A.P + D * A.ncell : nullptr;
-    const double* const Pc = A.P ? A.P + (D + 1) * A.ncell : nullptr;
-    /* normal velocity and pressure of a cell */
-    auto normal = [&](long long cell, const double (&u)[NV], double& un, double& p) {
-      if (A.P) {
-        un = __ldg(Pn + cell);
-        p = __ldg(Pp + cell);
-      } else {
-        const double rinv = rcp_nr(u[0]);
-        double ke = 0.0;
-#pragma unroll
-        for (int d = 1; d <= D; ++d) ke += u[d] * (u[d] * rinv);
-        un = u[1] * rinv;
-        p = (A.gamma - 1.0) * (u[NV - 1] - 0.5 * ke);
-      }
-    };
+    const double* const Pn = A.P + ax * A.ncell;  /* normal velocity, pressure, sound speed */
+    const double* const Pp = A.P + D * A.ncell;
+    const double* const Pc = A.P + (D + 1) * A.ncell;
 
     /* ---- (0) Roe state and LLF speeds, one thread per face ---- */
     unsigned mask = 0u;
@@ -133,59 +250,82 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
         base = (long long)x + (ax == 1 ? (long long)A.n[0] * A.n[1] * hi : (long long)A.n[0] * lo);
       }
       if (bc == 0 && f == 0) fcopy = flin + na * (ax == 0 ? 1ll : (ax == 1 ? (long long)A.n[0] : sa));
-      double sr[2], Hh[2], v[2][D];
+      /* Roe average of the face's two cells; c~^2 in its cancellation-free form (weighted c^2 plus
+         (gamma - 1)/2 wl wr |dv|^2), H~ = c~^2/(gamma - 1) + |u~|^2/2 */
+      double sr[2], cs[2], v[2][D];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const long long cell = base + sa * bc_wrap(f - 1 + e, na, bc);
-        double u[NV], un, p;
+        const long long cell = base + sa * bc_near(f - 1 + e, na, bc);
+        const double rho = __ldg(up[0] + cell);
+        sr[e] = rho * rsqrt_nr(rho);
+        cs[e] = __ldg(Pc + cell);
 #pragma unroll
-        for (int q = 0; q < NV; ++q) u[q] = __ldg(up[q] + cell);
-        normal(cell, u, un, p);
-        const double rinv = rcp_nr(u[0]);
-        Hh[e] = (u[NV - 1] + p) * rinv;
-        sr[e] = u[0] * rsqrt_nr(u[0]);
-        v[e][0] = un;
-#pragma unroll
-        for (int d = 1; d < D; ++d) v[e][d] = u[1 + d] * rinv;
+        for (int d = 0; d < D; ++d) v[e][d] = __ldg(A.P + (gc(1 + d) - 1) * A.ncell + cell);
       }
-      const double wsum = rcp_nr(sr[0] + sr[1]);
-      double q2 = 0.0;
+      const double gm1 = A.gamma - 1.0;
+      const double ws = rcp_nr(sr[0] + sr[1]), wl = sr[0] * ws, wr = sr[1] * ws;
+      double q2 = 0.0, dv2 = 0.0;
 #pragma unroll
       for (int d = 0; d < D; ++d) {
-        const double x = (sr[0] * v[0][d] + sr[1] * v[1][d]) * wsum;
-        q2 += x * x;
+        const double x = fma(wl, v[0][d], wr * v[1][d]), y = v[1][d] - v[0][d];
+        q2 = fma(x, x, q2);
+        dv2 = fma(y, y, dv2);
         s_row[(R::u + d) * TH + tid] = x;
       }
-      const double Ht = (sr[0] * Hh[0] + sr[1] * Hh[1]) * wsum;
-      const double c2 = (A.gamma - 1.0) * (Ht - 0.5 * q2);
-      if (!ipos(c2)) st |= ST_ROE;
+      const double c2 = fma(wl * cs[0], cs[0], fma(wr * cs[1], cs[1], 0.5 * gm1 * (wl * wr) * dv2));
+      if (!(c2 > 0.0)) st |= ST_ROE;
       const double ci = rsqrt_nr(c2);
-      const double b1 = (A.gamma - 1.0) * (ci * ci);
-      s_row[R::H * TH + tid] = Ht;
+      const double b1 = gm1 * (ci * ci);
+      s_row[R::H * TH + tid] = fma(c2, A.rgm1, 0.5 * q2);
       s_row[R::ci * TH + tid] = ci;
       s_row[R::ct * TH + tid] = c2 * ci;
       s_row[R::b1 * TH + tid] = b1;
       s_row[R::b2 * TH + tid] = 0.5 * q2 * b1;
-      /* LLF: alpha_s = max over the K stencil points of |lambda_s|, one per eigenvalue family */
+      /* LLF: alpha_s = max over the K stencil points of |lambda_s|, one per eigenvalue family.  The
+         largest |u -+ c| is found in FP32 (each within 5u (|u| + c)) and formed in FP64 where it is
+         the only candidate; ties within the error take all K points in FP64 */
       double am = 0.0, a0 = 0.0, ap = 0.0;
-#pragma unroll
+      float bm = -1.f, bp = -1.f, sm = -1.f, sp = -1.f, ah = 0.f;
+      int qm = 0, qp = 0;
+      auto speeds = [&](int q, double& un, double& c) {
+        const long long cell = base + sa * bc_near(f - H + q, na, bc);
+        un = __ldg(Pn + cell);
+        c = __ldg(Pc + cell);
+      };
+#pragma unroll 1
       for (int q = 0; q < K; ++q) {
-        const long long cell = base + sa * bc_wrap(f - H + q, na, bc);
-        double un, cs;
-        if (A.P) {
-          un = __ldg(Pn + cell);
-          cs = __ldg(Pc + cell);
-        } else {
-          double u[NV], vel[D], p;
-          int s2 = 0;
-#pragma unroll
-          for (int w = 0; w < NV; ++w) u[w] = __ldg(up[w] + cell);
-          point_prims<NV>(u, A.gamma, vel, p, cs, s2);
-          un = vel[0];
-        }
-        am = imax_nonneg(am, iabs(un - cs));
+        double un, c;
+        speeds(q, un, c);
         a0 = imax_nonneg(a0, iabs(un));
-        ap = imax_nonneg(ap, iabs(un + cs));
+        const float uf = f32_rz(un), cf = f32_rz(c);
+        const float xm = fabsf(uf - cf), xp = fabsf(uf + cf);
+        ah = fmaxf(ah, fabsf(uf) + cf);
+        sm = fmaxf(sm, fminf(xm, bm));
+        sp = fmaxf(sp, fminf(xp, bp));
+        if (xm > bm) {
+          bm = xm;
+          qm = q;
+        }
+        if (xp > bp) {
+          bp = xp;
+          qp = q;
+        }
+      }
+      const float tie = 10.f * 5.9604645e-8f * ah;
+      if (bm - sm > tie && bp - sp > tie && ah < 1e30f && ah > 1e-30f) {
+        double un, c;
+        speeds(qm, un, c);
+        am = iabs(un - c);
+        speeds(qp, un, c);
+        ap = iabs(un + c);
+      } else {
+#pragma unroll 1
+        for (int q = 0; q < K; ++q) {
+          double un, c;
+          speeds(q, un, c);
+          am = imax_nonneg(am, iabs(un - c));
+          ap = imax_nonneg(ap, iabs(un + c));
+        }
       }
       s_row[R::am * TH + tid] = am;
       s_row[R::a0 * TH + tid] = a0;
@@ -193,6 +333,7 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       s_base[tid] = base;
       s_f[tid] = f;
       s_cm[tid] = A.sch.default_d ? (allf & ~mask) : 0u;
+      s_dir[tid] = 0u;
     }
     /* the chunk's (face, field) items, field after field */
 #pragma unroll
@@ -220,24 +361,30 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       if (mask >> s & 1u) s_item[s_wc[s * W + wid] + __popc(b & ((1u << ln) - 1u))] = (unsigned short)(tid | (s << 8));
     }
     const int nitem = s_wc[NV * W];
+    if (tid == 0) s_nlater = 0;
     __syncthreads();
 
-    /* ---- (1) one (face, field) per thread ---- */
+    /* ---- (1) one (face, field) per thread; FIX: what the FP32 filter leaves undecided comes
+       again in a second pass, in warps of its own ---- */
 #pragma unroll 1
-    for (int it = tid; it < nitem; it += TH) {
-      const int fc = s_item[it] & 255, s = s_item[it] >> 8;
+    for (int pass = 0; pass < (FIX ? 2 : 1); ++pass) {
+    const int npass = pass ? s_nlater : nitem;
+#pragma unroll 1
+    for (int it = tid; it < npass; it += TH) {
+      const unsigned item = pass ? s_later[it] : s_item[it];
+      const int fc = item & 255, s = item >> 8;
       auto row = [&](int r) -> double { return s_row[r * TH + fc]; };
       const bool acoustic = s == 0 || s == NV - 1, shear = s >= 2 && s <= NV - 2;
       const double ha = 0.5 * row(s == 0 ? R::am : (s == NV - 1 ? R::ap : R::a0));
       /* left eigenvector l_s (closed form of R^{-1}); shear: l = e_t - u_t e_0 */
       double l[NV];
       if (acoustic) {
-        const double sg = (s == 0) ? 1.0 : -1.0, ci = row(R::ci), b1 = row(R::b1), un = row(R::u);
-        l[0] = 0.5 * (row(R::b2) + sg * un * ci);
-        l[1] = 0.5 * (-b1 * un - sg * ci);
+        const double ci = (s == 0) ? 0.5 * row(R::ci) : -0.5 * row(R::ci), b1 = 0.5 * row(R::b1), un = row(R::u);
+        l[0] = fma(un, ci, 0.5 * row(R::b2));
+        l[1] = -fma(b1, un, ci);
 #pragma unroll
-        for (int d = 1; d < D; ++d) l[1 + d] = -0.5 * b1 * row(R::u + d);
-        l[NV - 1] = 0.5 * b1;
+        for (int d = 1; d < D; ++d) l[1 + d] = -b1 * row(R::u + d);
+        l[NV - 1] = b1;
       } else if (s == 1) {
         const double b1 = row(R::b1);
         l[0] = 1.0 - row(R::b2);
@@ -252,66 +399,78 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       const double* const ut = A.U + gc(shear ? s : 1) * A.ncell;
       const long long base = s_base[fc];
       const int f = s_f[fc];
-      double wv[K], hgv[K];
-#pragma unroll
-      for (int q = 0; q < K; ++q) {
-        const long long cell = base + sa * bc_wrap(f - H + q, na, bc);
-        double un, pq, w, kap;
-        if (A.P && shear) {
-          un = __ldg(Pn + cell);
+      /* W and G/2 of stencil point q, G = l . F = u_n W + p (l_n + u_n l_E) */
+      auto project = [&](int q, double& w, double& hg) {
+        const long long cell = base + sa * bc_near(f - H + q, na, bc);
+        const double un = __ldg(Pn + cell);
+        if (shear) {
           w = fma(l[0], __ldg(up[0] + cell), __ldg(ut + cell));
-          pq = 0.0;
-          kap = 0.0;
+          hg = 0.5 * un * w;
         } else {
-          double u[NV];
+          w = l[0] * __ldg(up[0] + cell);
 #pragma unroll
-          for (int v = 0; v < NV; ++v) u[v] = __ldg(up[v] + cell);
-          normal(cell, u, un, pq);
-          if (shear) {
-            w = fma(l[0], u[0], __ldg(ut + cell));
-            kap = 0.0;
-          } else {
-            w = l[0] * u[0];
-#pragma unroll
-            for (int v = 1; v < NV; ++v) w = fma(l[v], u[v], w);
-            kap = fma(un, l[NV - 1], l[1]);
-          }
+          for (int v = 1; v < NV; ++v) w = fma(l[v], __ldg(up[v] + cell), w);
+          hg = 0.5 * fma(__ldg(Pp + cell), fma(un, l[NV - 1], l[1]), un * w);
         }
-        wv[q] = w;
-        hgv[q] = 0.5 * fma(pq, kap, un * w);  /* G/2, G = l . F = u_n W + p (l_n + u_n l_E) */
-      }
-      /* the two split sides through one copy of the decisions and the reconstruction:
-         f+ on g+_q = G_q/2 + (alpha/2) W_q, f- on g-_q = G_q/2 - (alpha/2) W_q mirrored about
-         x_{i+1/2} */
-      unsigned fl = 0u, sm2 = 0u;
+      };
+      unsigned fl = 0u;
       double fsum = 0.0;
-      double op[REC ? K : 1], om[REC ? K : 1];  /* frozen linear weights of f+ and f- */
+      bool direct = !FIX;
+      double wv[REC ? K : 1], op[REC ? K : 1], om[REC ? K : 1];  /* W; frozen linear weights of f+ and f- */
+      if constexpr (FIX) {
+        int eg = 0, ew = 0;
 #pragma unroll 1
-      for (int side = 0; side < 2; ++side) {
-        double v[K];
-#pragma unroll
-        for (int q = 0; q < K; ++q) v[q] = side ? fma(-ha, wv[K - 1 - q], hgv[K - 1 - q]) : fma(ha, wv[q], hgv[q]);
-        unsigned b = 0;
-        int e = 7;
-        if (!teno_decide_fast<K>(v, A.sch, b, e)) teno_decide_fp64<K>(v, A.sch, b, e, st);
-        if constexpr (REC) {
-          double wt[K];
-          fsum += teno_general<K, LIM, true>(v, A.sch, b, wt);
-#pragma unroll
-          for (int q = 0; q < K; ++q) {
-            if (side) om[q] = wt[q];
-            else op[q] = wt[q];
-          }
-        } else {
-          fsum += teno_general<K, LIM>(v, A.sch, b);
+        for (int q = 0; q < K; ++q) {
+          double w, hg;
+          project(q, w, hg);
+          s_w[q * TH + tid] = w;
+          s_g[q * TH + tid] = hg;
+          eg = max(eg, (int)((unsigned)__double2hiint(hg) >> 20 & 0x7ffu));
+          ew = max(ew, (int)((unsigned)__double2hiint(w) >> 20 & 0x7ffu));
         }
-        fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
-        sm2 += (b == allk) ? 1u : 0u;
+        /* |v| <= |G/2| + |alpha W/2| < 2^(em - 1022) */
+        const int em = 1 + max(eg, ew + (int)((unsigned)__double2hiint(ha) >> 20 & 0x7ffu) - 1022);
+        if (!fixed_item<K, LIM>(s_w + tid, s_g + tid, ha, em, s_D + tid, A.sch, pass == 0 && nitem > TH, fl, fsum,
+                                direct, st)) {
+          s_later[atomicAdd(&s_nlater, 1)] = (unsigned short)item;
+          continue;
+        }
+      } else {
+        double w[K], hg[K];
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          project(q, w[q], hg[q]);
+          if constexpr (REC) wv[q] = w[q];
+        }
+        /* the two split sides through one copy of the decisions and the reconstruction: f+ on
+           g+_q = G_q/2 + (alpha/2) W_q, f- on g-_q = G_q/2 - (alpha/2) W_q mirrored about x_{i+1/2} */
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+          double v[K];
+#pragma unroll
+          for (int q = 0; q < K; ++q) v[q] = side ? fma(-ha, w[K - 1 - q], hg[K - 1 - q]) : fma(ha, w[q], hg[q]);
+          unsigned b = 0;
+          int e = 7;
+          if (!teno_decide_fast<K>(v, A.sch, b, e)) teno_decide_fp64<K>(v, A.sch, b, e, st);
+          if constexpr (REC) {
+            double wt[K];
+            fsum += teno_general<K, LIM, true>(v, A.sch, b, wt);
+#pragma unroll
+            for (int q = 0; q < K; ++q) {
+              if (side) om[q] = wt[q];
+              else op[q] = wt[q];
+            }
+          } else {
+            fsum += teno_general<K, LIM>(v, A.sch, b);
+          }
+          fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
+        }
       }
       s_fs[s * TH + fc] = fsum;
       /* a field found all smooth on both sides is central after all: the flux does not depend on
          which test decided */
-      if (sm2 == 2u && A.sch.default_d) atomicOr(&s_cm[fc], 1u << s);
+      if ((fl & (allk | allk << 8)) == (allk | allk << 8) && A.sch.default_d) atomicOr(&s_cm[fc], 1u << s);
+      else if (direct) atomicOr(&s_dir[fc], 1u << s);
       const bool copy = bc == 0 && f == 0;
       const long long fi = A.list[ax][i0 + fc];
       const long long fcp = fi + na * (ax == 0 ? 1ll : (ax == 1 ? (long long)A.n[0] : sa));
@@ -342,46 +501,56 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       }
     }
     __syncthreads();
+    }
 
-    /* ---- (2) Fhat = Fc when every field is central, else sum_s r_s fs with fs = l_s . Fc for
-       the central fields.  Both sums go through the vectors the eigenvectors share:
-       a = (b2, -b1 u, b1) and b = (u_n, -e_n, 0)/c give l_{u-c} = (a + b)/2, l_{u+c} = (a - b)/2,
-       l_entropy = e_0 - a, l_shear = e_t - u_t e_0, and with sigma = f_{u-c} + f_{u+c},
-       delta = (f_{u+c} - f_{u-c}) c:  F_0 = sigma + f_1,  F_d = (sigma + f_1) u_d + (delta if
-       d = n, else f_shear(d)),  F_E = sigma H + delta u_n + f_1 |u|^2/2 + sum_t f_t u_t. ---- */
+    /* ---- (2) Fhat = Fc when every field is central; Fc + sum_s r_s correction_s when the others
+       are corrections; else sum_s r_s fs with fs = l_s . Fc (+ correction) for the fields that are
+       not direct.  Both sums go through the vectors the eigenvectors share: a = (b2, -b1 u, b1)
+       and b = (u_n, -e_n, 0)/c give l_{u-c} = (a + b)/2, l_{u+c} = (a - b)/2, l_entropy = e_0 - a,
+       l_shear = e_t - u_t e_0, and with sigma = f_{u-c} + f_{u+c}, delta = (f_{u+c} - f_{u-c}) c:
+       F_0 = sigma + f_1,  F_d = (sigma + f_1) u_d + (delta if d = n, else f_shear(d)),
+       F_E = sigma H + delta u_n + f_1 |u|^2/2 + sum_t f_t u_t. ---- */
     if (tid < nf && s_cm[tid] != allf) {
-      const unsigned cm = s_cm[tid];
+      const unsigned cm = s_cm[tid], dir = s_dir[tid];
       auto row = [&](int r) -> double { return s_row[r * TH + tid]; };
       double* const Fo = A.Fhat[ax];
-      double Fc[NV], ut[D], fs[NV], Fh[NV], q2 = 0.0, uF = 0.0;
+      double Fc[NV], ut[D], fs[NV], Fh[NV], q2 = 0.0;
 #pragma unroll
       for (int v = 0; v < NV; ++v) Fc[v] = Fo[gc(v) * nface + flin];
 #pragma unroll
+      for (int s = 0; s < NV; ++s) fs[s] = (cm >> s & 1u) ? 0.0 : s_fs[s * TH + tid];
+#pragma unroll
       for (int d = 0; d < D; ++d) {
         ut[d] = row(R::u + d);
-        q2 += ut[d] * ut[d];
-        uF = fma(ut[d], Fc[1 + d], uF);
+        q2 = fma(ut[d], ut[d], q2);
       }
-      const double a = fma(row(R::b2), Fc[0], row(R::b1) * (Fc[NV - 1] - uF));
-      const double b = row(R::ci) * fma(ut[0], Fc[0], -Fc[1]);
-      fs[0] = (cm & 1u) ? 0.5 * (a + b) : s_fs[tid];
-      fs[NV - 1] = (cm >> (NV - 1) & 1u) ? 0.5 * (a - b) : s_fs[(NV - 1) * TH + tid];
-      fs[1] = (cm >> 1 & 1u) ? Fc[0] - a : s_fs[TH + tid];
+      if (dir) {
+        double uF = 0.0;
 #pragma unroll
-      for (int s = 2; s <= NV - 2; ++s)
-        fs[s] = (cm >> s & 1u) ? fma(-ut[s - 1], Fc[0], Fc[s]) : s_fs[s * TH + tid];
+        for (int d = 0; d < D; ++d) uF = fma(ut[d], Fc[1 + d], uF);
+        const double a = fma(row(R::b2), Fc[0], row(R::b1) * (Fc[NV - 1] - uF));
+        const double b = row(R::ci) * fma(ut[0], Fc[0], -Fc[1]);
+        if (!(dir & 1u)) fs[0] += 0.5 * (a + b);
+        if (!(dir >> (NV - 1) & 1u)) fs[NV - 1] += 0.5 * (a - b);
+        if (!(dir >> 1 & 1u)) fs[1] += Fc[0] - a;
+#pragma unroll
+        for (int s = 2; s <= NV - 2; ++s)
+          if (!(dir >> s & 1u)) fs[s] += fma(-ut[s - 1], Fc[0], Fc[s]);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Fc[v] = 0.0;
+      }
       const double sigma = fs[0] + fs[NV - 1];
       const double delta = (fs[NV - 1] - fs[0]) * row(R::ct);
       const double m = sigma + fs[1];
       double FE = fma(sigma, row(R::H), fma(delta, ut[0], 0.5 * q2 * fs[1]));
-      Fh[0] = m;
-      Fh[1] = fma(m, ut[0], delta);
+      Fh[0] = Fc[0] + m;
+      Fh[1] = Fc[1] + fma(m, ut[0], delta);
 #pragma unroll
       for (int s = 2; s <= NV - 2; ++s) {
-        Fh[s] = fma(m, ut[s - 1], fs[s]);
+        Fh[s] = Fc[s] + fma(m, ut[s - 1], fs[s]);
         FE = fma(ut[s - 1], fs[s], FE);
       }
-      Fh[NV - 1] = FE;
+      Fh[NV - 1] = Fc[NV - 1] + FE;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         Fo[gc(v) * nface + flin] = Fh[v];

@@ -38,6 +38,8 @@ struct SchemeDev {
   int exact_decisions;   /* 1: decide the cutoff in FP64 only (no certified FP32 filter) */
   int screen;            /* 1: faces are screened (default_d and FP32 decisions allowed), 0: every face is nonlinear */
   float quick_r[2];      /* quick_smooth's ratio bound (nk C_T)^(-1/6): [0] for C_T (1e-7 when adaptive), [1] for 1e-10 */
+  int fixed;             /* 1: the limiter's corrections run in fixed point (tenom_fixed.cuh) */
+  long long alpha_q60, beta_third_q60;  /* mp_alpha, mp_beta / 3 times 2^60 (fixed only) */
   float ct_const_f;       /* ct_const rounded to FP32 (certified filter) */
   double ct_const;
   double mp_alpha;
@@ -248,7 +250,9 @@ __device__ __forceinline__ float sqrt_up(float x) {
 /* Certified single-precision evaluation of the cutoff decisions delta_k (and of [beta] of
    TENO8A).  FP32 runs on the SM's wide FP32 pipe; GB300's FP64 pipe is the bottleneck.
    An indicator beta = sum_j w_j t_j^2, t_j = sum_i m_ji D_i, is evaluated with every t_j
-   within Eb sum_i |m_ji| of its exact value, Eb = 12 u max|D| (u = 2^-24: D truncated to
+   within Eb sum_i |m_ji| of its exact value, Eb = 12 u max|D| + E with the maximum over the
+   indicator's own differences (E: an absolute error of the D's besides their truncation, 0 for
+   FP64 differences; zero: bit t set where D_t is exactly zero; u = 2^-24: D truncated to
    FP32, relative error below 2u -- a difference below the FP32 normal range becomes 0, an
    absolute error far below the bound -- and a dot product of at most 7 terms with rounded
    coefficients), so sqrt(beta) is within sqrt(kk) Eb (beta_norm) and beta within
@@ -259,24 +263,22 @@ __device__ __forceinline__ float sqrt_up(float x) {
    to stay in range) and the comparison gamma_k < C_T sum gamma (quotients by the fast
    division, whose 2-ulp error the bounds include).  A decision is returned only when the whole
    interval lies on one side; otherwise (and for out-of-range data or an indicator that may
-   vanish, where epsilon = 1e-40 matters) the caller decides in FP64.  Certified decisions
+   vanish, where epsilon = 1e-40 matters) the caller decides in FP64.  Candidates on exactly
+   constant stencils (the constant states of a shock tube) are decided here too: their
+   gamma = (1 + tau/1e-40)^6 leaves every other candidate nonsmooth.  Certified decisions
    equal the exact-arithmetic decisions, hence those of the FP64 path except where that
    path is itself within its rounding of the threshold (an adaptive-precision predicate in
    the sense of Shewchuk's robust geometric predicates). */
 template <int K>
-__device__ __forceinline__ bool cutoff_filter(const double (&D)[K - 1], const SchemeDev& S, unsigned& bits, int& ex) {
+__device__ __forceinline__ bool cutoff_filter(const float (&d)[K - 1], float E, unsigned zero, const SchemeDev& S,
+                                              unsigned& bits, int& ex) {
   constexpr int c = K / 2 - 1;
   constexpr int nk = K - 2;
   const float u = 5.9604645e-8f;
-  float d[K - 1];
   float dmax = 0.f;
 #pragma unroll
-  for (int t = 0; t < K - 1; ++t) {
-    d[t] = f32_rz(D[t]);
-    dmax = fmaxf(dmax, fabsf(d[t]));
-  }
+  for (int t = 0; t < K - 1; ++t) dmax = fmaxf(dmax, fabsf(d[t]));
   if (!(dmax <= 1e15f) || (dmax > 0.f && dmax < 1e-15f)) return false;
-  const float Eb = 12.f * u * dmax;
   float b[nk], e[nk];
   b[0] = beta0<c - 1, false, float>(d);
   b[1] = beta1<c, false, float>(d);
@@ -290,19 +292,39 @@ __device__ __forceinline__ bool cutoff_filter(const double (&D)[K - 1], const Sc
   } else {
     bK = betaK6<0, false, float>(d);
   }
-  auto err_of = [&](float bb, float kk) {
+  constexpr int first[6] = {c - 1, c, c - 2, c, c - 3, c}, count[6] = {2, 2, 2, 3, 3, 4};
+  constexpr unsigned allD = (1u << (K - 1)) - 1u;
+  auto err_of = [&](float bb, float kk, float dm, bool constant) {
+    const float Eb = fmaf(12.f * u, dm, constant ? 0.f : E);
     return fmaf(Eb, fmaf(2.f, sqrt_up(bb * kk), kk * Eb), 20.f * u * bb) * (1.f + 16.f * u);
   };
+  unsigned flat = 0u;  /* candidates on a constant stencil: beta_k = 0 exactly */
 #pragma unroll
-  for (int k = 0; k < nk; ++k) e[k] = err_of(b[k], beta_norm(k));
+  for (int k = 0; k < nk; ++k) {
+    float dm = 0.f;
+#pragma unroll
+    for (int t = 0; t < count[k]; ++t) dm = fmaxf(dm, fabsf(d[first[k] + t]));
+    const unsigned own = ((1u << count[k]) - 1u) << first[k];
+    const bool constant = (zero & own) == own;
+    flat |= constant ? 1u << k : 0u;
+    e[k] = err_of(b[k], beta_norm(k), dm, constant);
+  }
   const float comb = (b[1] + b[2] + 4.f * b[0]) * (1.f / 6.f);
   const float tau = fabsf(bK - comb);
-  const float dtau = (err_of(bK, BetaNorm<K>::kK) + (e[1] + e[2] + 4.f * e[0]) * (1.f / 6.f)) * (1.f + 8.f * u) +
+  const float dtau = (err_of(bK, BetaNorm<K>::kK, dmax, zero == allD) + (e[1] + e[2] + 4.f * e[0]) * (1.f / 6.f)) * (1.f + 8.f * u) +
                      8.f * u * (bK + comb);
   const float tl = fmaxf(tau - dtau, 0.f), th = tau + dtau;
+  if (th == 0.f) flat = 0u;  /* every candidate has gamma = 1 */
+  /* tau certain to a factor of 4 and far above epsilon; tau <= 1e8 keeps gamma finite in FP64 */
+  if (flat && !(tl >= 1e-25f && th <= 4.f * tl && th <= 1e8f)) return false;
   float xl[nk], xh[nk], xm = 1.f;
 #pragma unroll
   for (int k = 0; k < nk; ++k) {
+    if (flat >> k & 1u) {
+      xl[k] = 1.f;
+      xh[k] = 1.f;
+      continue;
+    }
     const float bl = b[k] - e[k], bh = (b[k] + e[k]) * (1.f + 2.f * u);
     if (bl < 1e-30f) {
       if (th != 0.f) return false;  /* beta_k may vanish: epsilon matters */
@@ -334,6 +356,9 @@ __device__ __forceinline__ bool cutoff_filter(const double (&D)[K - 1], const Sc
   float CTf = S.ct_const_f;
   ex = 7;
   if (S.ct_mode == CT_ADAPTIVE) {
+    /* E moves eta by at most 8 E / max(|d|, sqrt(eps) = 5e-4) and beta by 32 times that: below the
+       1e-4 margin (FP32 rounding: 32 x 12 u) for E <= 1e-10 */
+    if (!(E <= 1e-10f)) return false;
     const float xi = 1e-3f, Cr = 0.23f, a1 = 10.5f, a2 = 3.5f;
     const float eps = 0.9f * Cr / (1.f - 0.9f * Cr) * xi * xi;
     float eh = 0.f;
@@ -347,13 +372,17 @@ __device__ __forceinline__ bool cutoff_filter(const double (&D)[K - 1], const Sc
     const float om = 1.f - m;
     const float g = om * om * om * om * (1.f + 4.f * m);
     const float beta = a1 - a2 * (1.f - g);
-    if (fabsf(beta - rintf(beta)) < 1e-3f) return false;
+    if (fabsf(beta - rintf(beta)) < 1e-4f) return false;
     int x = (int)floorf(beta);
     x = x < 7 ? 7 : (x > 10 ? 10 : x);
     ex = x;
     CTf = x == 7 ? 1e-7f : (x == 8 ? 1e-8f : (x == 9 ? 1e-9f : 1e-10f));
   }
   if (!(CTf >= 1e-30f)) return false;  /* C_T below the FP32 normal range: decide in FP64 */
+  if (flat) {  /* (x_j / x_flat)^6 <= (5e-40 / 1e-30)^6 for the others, 1 / (number of flat ones) for these */
+    bits = flat;
+    return CTf < 0.1f;
+  }
   const float thl = CTf * (1.f - 2.f * u) * Sl * (1.f - u), thh = CTf * (1.f + 2.f * u) * Sh * (1.f + u);
   unsigned bt = 0;
 #pragma unroll
@@ -506,10 +535,14 @@ __device__ __forceinline__ void teno_decide_fp64(const double (&v)[K], const Sch
 template <int K>
 __device__ __forceinline__ bool teno_decide_fast(const double (&v)[K], const SchemeDev& S, unsigned& bits, int& ex) {
   if (S.exact_decisions) return false;
-  double D[K - 1];
+  float d[K - 1];
+  unsigned zero = 0u;
 #pragma unroll
-  for (int t = 0; t < K - 1; ++t) D[t] = v[t + 1] - v[t];
-  return cutoff_filter<K>(D, S, bits, ex);
+  for (int t = 0; t < K - 1; ++t) {
+    d[t] = f32_rz(v[t + 1] - v[t]);  /* below 2^-126: beta < 1e-74, as good as zero beside epsilon */
+    zero |= d[t] == 0.f ? 1u << t : 0u;
+  }
+  return cutoff_filter<K>(d, 0.f, zero, S, bits, ex);
 }
 
 /* every candidate smooth with the maximal-order d_k: sum_k d_k f_k is the K-point central

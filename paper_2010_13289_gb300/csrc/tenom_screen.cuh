@@ -38,9 +38,10 @@ namespace tenom {
    Bounds: each form beta = sum_j w_j t_j^2 is evaluated with t_j within Eb sum_i |m_ji| of its
    exact value, Eb = E + 10 u max|d| (dot product of at most 7 terms with rounded
    coefficients), so |sqrt(beta) - sqrt(beta_exact)| <= sqrt(kk) Eb, and 2 sqrt(beta kk) Eb <=
-   s beta + kk Eb^2 / s with s = 1/32 turns that into beta (1 -+ s) -+ kk (1 + 1/s) Eb^2; the
-   constants below (0.966, 1.0315, 0.0314, 1.04) add the 20 u relative rounding of the sums of
-   squares.  No square root, division or interval arithmetic: about a third of the work of
+   s beta + kk Eb^2 / s turns that into beta (1 -+ s) -+ kk (1 + 1/s) Eb^2, with s = 1/32 for the
+   beta_k and s = 2^-11 for tau (tau's bound is what a candidate near a critical point, with a
+   beta_k far below the others', is compared with); the constants below (0.966, 1.0315, 4.95e-4,
+   1.04) add the 20 u relative rounding of the sums of squares.  No square root, division or interval arithmetic: about a third of the work of
    bounding every gamma_k, and it fails on few smooth sides (per face of the 256^3 solenoidal
    state 0.17 fields are truly nonsmooth).
    Adaptive C_T (TENO8A): 1e-7, the largest, always holds; where the least of the four eta is
@@ -55,7 +56,7 @@ __device__ __forceinline__ bool quick_smooth(const float (&d)[K - 1], float E, c
 #pragma unroll
   for (int t = 0; t < K - 1; ++t) dm = fmaxf(dm, fabsf(d[t]));
   const float Eb = fmaf(10.f * u, dm, E);
-  const float e2 = 33.f * Eb * Eb;
+  const float eb2 = Eb * Eb, e2 = 33.f * eb2;
   const float b0 = beta0<c - 1, false, float>(d), b1 = beta1<c, false, float>(d), b2 = beta2<c - 2, false, float>(d);
   const float b3 = beta3<c, false, float>(d);
   float lo = fminf(fmaf(-1.04f * beta_norm(0), e2, b0), fmaf(-1.04f * beta_norm(1), e2, fminf(b1, b2)));
@@ -71,7 +72,7 @@ __device__ __forceinline__ bool quick_smooth(const float (&d)[K - 1], float E, c
     bK = betaK6<0, false, float>(d);
   }
   const float comb = (b1 + b2 + 4.f * b0) * (1.f / 6.f);
-  const float T = fabsf(bK - comb) + fmaf(0.0314f, bK + comb, (1.04f * (BetaNorm<K>::kK + 6.f)) * e2);
+  const float T = fabsf(bK - comb) + fmaf(4.95e-4f, bK + comb, (2060.f * (BetaNorm<K>::kK + 6.f)) * eb2);
   float R = S.quick_r[0];
   if (S.ct_mode == CT_ADAPTIVE) {
     /* 2 |a b| - 0.2 (a^2 + b^2) over the four neighbouring pairs, |a|, |b| known to within Eb */
@@ -154,7 +155,7 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
   /* Roe state of points H - 1 | H */
   const float rl = val(L::R, H - 1), rr = val(L::R, H);
   const float sl = __fsqrt_rn(rl), wl = __fdividef(sl, sl + __fsqrt_rn(rr)), wr = 1.f - wl;
-  float dv2 = 0.f, q2 = 0.f, wn[K], vt[D];
+  float dv2 = 0.f, q2 = 0.f, wn[K] = {}, vt[D];
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const float dv = dif(L::V + d, H - 1);
@@ -433,7 +434,6 @@ screen_kernel(const FaceArgs A) {
   const long long sa = (AXIS == 0) ? 1 : (AXIS == 1 ? sy : sz);
 
   /* --- stage the tile's points: F in FP64, the screen's point data in FP32 --- */
-  int st = 0;
   for (int p = tid; p < NP; p += T::THREADS) {
     const int lane = (AXIS == 0) ? 0 : (p % T::LANES);
     const int row = (AXIS == 0) ? p : (p / T::LANES);
@@ -449,14 +449,11 @@ screen_kernel(const FaceArgs A) {
     double u[NV], vel[D], pr, cs;
 #pragma unroll
     for (int q = 0; q < NV; ++q) u[q] = __ldg(A.U + q * A.ncell + cell);
-    if (A.P) {  /* primitives computed once per cell per stage */
+    /* primitives computed once per cell per stage */
 #pragma unroll
-      for (int d = 0; d < D; ++d) vel[d] = __ldg(A.P + d * A.ncell + cell);
-      pr = __ldg(A.P + D * A.ncell + cell);
-      cs = __ldg(A.P + (D + 1) * A.ncell + cell);
-    } else {
-      point_prims<NV>(u, A.gamma, vel, pr, cs, st);
-    }
+    for (int d = 0; d < D; ++d) vel[d] = __ldg(A.P + d * A.ncell + cell);
+    pr = __ldg(A.P + D * A.ncell + cell);
+    cs = __ldg(A.P + (D + 1) * A.ncell + cell);
     double F[NV];
     F[0] = u[1 + AXIS];
 #pragma unroll
@@ -582,7 +579,6 @@ screen_kernel(const FaceArgs A) {
       A.mask[pos] = (uint8_t)bad;
     }
   }
-  if (st) atomicOr(A.status, st);
 }
 
 }  // namespace tenom
