@@ -869,7 +869,7 @@ def run_le_blanc(args):
     """Le Blanc problem (Section 4.4.2, Eq. Leblanc): 900 cells on [0, 9], gamma = 5/3,
     TENO8-MP with the minmod curvature and beta = 1 and the positivity-preserving flux
     limiter (Section 4.4), CFL 0.4, to t = 6, timed end to end on the device (a 900-cell
-    grid is launch-bound: about 16 launches per step).  Also times the limiter's cost on the
+    grid is latency-bound: its steps run in launches of one cluster).  Also times the limiter's cost on the
     2D 2048^2 broadband workload (step time with the limiter over step time without) and
     512 Le Blanc problems of log-uniform size 128..8192 through the batched launch, with and
     without the limiter."""

@@ -12,7 +12,7 @@
 #include "tenom_internal.h"
 #include "tenom_adjoint_kernels.cuh"
 #include "tenom_nonlinear.cuh"
-#include "tenom_positivity.cuh"
+#include "tenom_line.cuh"
 
 namespace tenom {
 
@@ -850,10 +850,45 @@ static cudaError_t rk3_core(tenom_ctx* c, double* U) {
   return e;
 }
 
+/* 1D grids that one cluster covers advance in one launch (line_kernel) */
+static bool is_line(const tenom_ctx* c) { return c->nv == 3 && c->ncell <= line_cells_max(c->s.K); }
+
+/* nsteps steps of a short line: CFL steps from *t_dev, or one of length *dt_dev */
+static cudaError_t launch_line(tenom_ctx* c, double* U, const double* dt_dev, double* t_dev, double t_end, double cfl,
+                               int nsteps) {
+  LineArgs a;
+  memset(&a, 0, sizeof(a));
+  a.U = U;
+  a.W1 = c->W1;
+  a.W2 = c->P;  /* the primitives' buffer, unused here */
+  a.dt = dt_dev;
+  a.t = t_dev;
+  a.t_end = t_end;
+  a.cfl = cfl;
+  a.rdx = 1.0 / c->g.dx[0];
+  a.gamma = c->g.gamma;
+  a.rgm1 = 1.0 / (c->g.gamma - 1.0);
+  a.n = c->g.n[0];
+  a.bc = c->g.bc[0];
+  a.status = c->status;
+  a.sch = scheme_dev(c->s);
+  const bool pp = c->s.positivity == TENOM_PP_ON;
+  cudaError_t e = cudaSuccess;
+  for (int done = 0; done < nsteps && e == cudaSuccess; done += a.nsteps) {
+    a.nsteps = nsteps - done < 256 ? nsteps - done : 256;  /* a launch stays in the tens of milliseconds */
+    e = c->s.K == 6 ? launch_line_k6(a, c->s.limiter, pp, c->st) : launch_line_k8(a, c->s.limiter, pp, c->st);
+  }
+  return e;
+}
+
 tenom_status tenom_rk3_step(tenom_ctx* c, double* U, const double* dt_dev) {
   if (!c) return TENOM_E_INVALID;
   if (!aligned8(U) || !aligned8(dt_dev)) return fail(c, TENOM_E_INVALID, "rk3_step: bad pointers");
   cudaError_t e = cudaSuccess;
+  if (is_line(c)) {
+    e = launch_line(c, U, dt_dev, nullptr, 0.0, 0.0, 1);
+    return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "rk3_step");
+  }
   if (dt_dev != c->dt) e = cudaMemcpyAsync(c->dt, dt_dev, sizeof(double), cudaMemcpyDeviceToDevice, c->st);
   if (e == cudaSuccess) e = launch_prims(c, U);
   if (e == cudaSuccess) e = rk3_core(c, U);
@@ -864,6 +899,10 @@ tenom_status tenom_advance(tenom_ctx* c, double* U, double* t_dev, double t_end,
   if (!c) return TENOM_E_INVALID;
   if (!aligned8(U) || !aligned8(t_dev) || !(cfl > 0.0) || nsteps < 0 || !(t_end == t_end))
     return fail(c, TENOM_E_INVALID, "advance: bad arguments");
+  if (is_line(c)) {
+    const cudaError_t e = launch_line(c, U, nullptr, t_dev, t_end, cfl, nsteps);
+    return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "advance");
+  }
   for (int k = 0; k < nsteps; ++k) {
     cudaError_t e = launch_signal(c, U, true);
     if (e == cudaSuccess) {

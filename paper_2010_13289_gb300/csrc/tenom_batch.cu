@@ -108,8 +108,9 @@ static StageFn pick_stage(int K, int lim, int tile, bool pp) {
 
 /* dynamic shared memory of the stage kernel of (K, tile): the kernel's own layout */
 static size_t stage_smem(int K, int tile) {
-  if (K == 6) return tile == 64 ? BatchTile<6, 64>::SMEM : (tile == 128 ? BatchTile<6, 128>::SMEM : BatchTile<6, 256>::SMEM);
-  return tile == 64 ? BatchTile<8, 64>::SMEM : (tile == 128 ? BatchTile<8, 128>::SMEM : BatchTile<8, 256>::SMEM);
+  if (K == 6)
+    return tile == 64 ? sizeof(LineTile<6, 64>) : (tile == 128 ? sizeof(LineTile<6, 128>) : sizeof(LineTile<6, 256>));
+  return tile == 64 ? sizeof(LineTile<8, 64>) : (tile == 128 ? sizeof(LineTile<8, 128>) : sizeof(LineTile<8, 256>));
 }
 
 }  // namespace tenom
@@ -196,6 +197,7 @@ static BatchArgs batch_args(tenom_batch* b, int stage) {
   a.status = b->status_d;
   a.total = b->total;
   a.gamma = b->gamma;
+  a.rgm1 = 1.0 / (b->gamma - 1.0);
   a.sch = scheme_for_device(b->s);
   return a;
 }

@@ -3,7 +3,7 @@
    tenom_batch_pp.cu (with it). */
 #pragma once
 #include "tenom_internal.h"
-#include "tenom_positivity.cuh"
+#include "tenom_line.cuh"
 
 namespace tenom {
 
@@ -19,14 +19,8 @@ struct BatchArgs {
   int* status;
   long long total;
   double gamma;
+  double rgm1;  /* 1 / (gamma - 1) */
   SchemeDev sch;
-};
-
-template <int K, int TILE>
-struct BatchTile {
-  static constexpr int NV = 3;
-  static constexpr int NP = TILE + K - 1;
-  static constexpr size_t SMEM = sizeof(double) * (PointLayout<3>::NC * NP + NV * TILE);
 };
 
 /* stage: 1 -> out = Us + dt L(Us); 2,3 -> out = cA U0 + cB (Us + dt L(Us)).  Compiled for
@@ -36,10 +30,9 @@ template <int K, int LIM, int TILE, bool PP>
 __global__ void __launch_bounds__(TILE, 512 / TILE)
 batch_stage_kernel(const BatchArgs A, const double* __restrict__ Us, const double* __restrict__ U0, double* out,
                    int mode, double cA, double cB) {
-  using T = BatchTile<K, TILE>;
-  constexpr int NV = 3, H = K / 2, NP = T::NP;
-  extern __shared__ double sm[];
-  double* Fs = sm + PointLayout<3>::NC * NP;
+  constexpr int NV = 3;
+  extern __shared__ double dyn[];
+  LineTile<K, TILE>& S = *reinterpret_cast<LineTile<K, TILE>*>(dyn);
   __shared__ int s_item;
   const int tid = threadIdx.x;
   int st = 0;
@@ -55,42 +48,14 @@ batch_stage_kernel(const BatchArgs A, const double* __restrict__ Us, const doubl
     if (dt == 0.0) continue;  /* finished problem (uniform across the CTA) */
     const int n = A.n[j];
     const long long off = A.off[j];
-    const int bc = A.bc[j];
-    for (int p = tid; p < NP; p += TILE) {
-      const int jj = bc_wrap(f0 - H + p, n, bc);
-      double u[NV];
-#pragma unroll
-      for (int q = 0; q < NV; ++q) u[q] = Us[q * A.total + off + jj];
-      stage_point<NV, 0>(u, A.gamma, sm, NP, p, st);
-    }
-    __syncthreads();
-    if (f0 + tid <= n) {
-      double Fh[NV];
-      face_flux_smem<NV, K, LIM, 0, 1>(sm, NP, tid, 0, A.gamma, A.sch, Fh, nullptr, st);
-      if constexpr (PP) {
-        /* positivity limiter of this stage (length dt, 1D: mu = 2 dt/dx) on the face between
-           staged points tid + H - 1 and tid + H; a face computed by two items is limited
-           identically by both */
-        using L = PointLayout<NV>;
-        const double mu = 2.0 * dt / A.dx[j];
-        double Ua[NV], Ub[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          Ua[v] = sm[(L::cU + v) * NP + tid + H - 1];
-          Ub[v] = sm[(L::cU + v) * NP + tid + H];
-        }
-        positivity_face<NV, 0>(Ua, Ub, Fh, mu, A.gamma, f32_rz(mu), f32_rz(A.gamma - 1.0));
-      }
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Fs[v * TILE + tid] = Fh[v];
-    }
-    __syncthreads();
+    const double rdx = 1.0 / A.dx[j];
+    line_stage(S, Us + off, A.total, n, A.bc[j], f0, TILE, A.gamma, st);
+    line_fluxes<K, LIM, TILE, PP>(S, n, f0, TILE, A.gamma, A.rgm1, A.sch, 2.0 * dt * rdx, st);
     const int c = f0 + tid;
     if (tid < TILE - 1 && c < n) {
-      const double dxj = A.dx[j];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const double r = 0.0 - (Fs[v * TILE + tid + 1] - Fs[v * TILE + tid]) / dxj;
+        const double r = 0.0 - (S.F[v * TILE + tid + 1] - S.F[v * TILE + tid]) * rdx;
         const long long g = v * A.total + off + c;
         const double t1 = Us[g] + dt * r;
         out[g] = (mode == 1) ? t1 : cA * U0[g] + cB * t1;

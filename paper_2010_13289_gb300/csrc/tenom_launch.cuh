@@ -26,7 +26,7 @@ struct AttrOnce {
 };
 
 template <class Kern>
-static cudaError_t ensure_smem_attr(Kern kern, AttrOnce& attr, size_t smem) {
+static cudaError_t ensure_smem_attr(Kern kern, AttrOnce& attr, size_t smem, bool wide_cluster = false) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -35,6 +35,8 @@ static cudaError_t ensure_smem_attr(Kern kern, AttrOnce& attr, size_t smem) {
   std::lock_guard<std::mutex> lock(attr.mu);
   if (attr.done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess && wide_cluster) /* clusters of more than 8 CTAs */
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   attr.done[dev].store(true, std::memory_order_release);
   return cudaSuccess;

@@ -1,0 +1,8 @@
+/* Short-line instantiations for the 6-point stencil. */
+#include "tenom_line_kernel.cuh"
+
+namespace tenom {
+
+cudaError_t launch_line_k6(const LineArgs& a, int lim, bool pp, cudaStream_t st) { return launch_line_k<6>(a, lim, pp, st); }
+
+}  // namespace tenom

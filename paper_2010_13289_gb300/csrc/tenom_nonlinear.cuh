@@ -72,6 +72,218 @@ __device__ __forceinline__ int bc_near(int j, int n, int bc) {
   return j < 0 ? 0 : (j >= n ? n - 1 : j);
 }
 
+/* face_rows' view of a face of the grid: its line starts at cell `base` with stride sa */
+template <int NV, int K>
+struct GridFace {
+  const double *rho, *vel[NV - 2], *un, *c;
+  long long base, sa;
+  int f, na, bc;
+  __device__ __forceinline__ long long cell(int q) const { return base + sa * bc_near(f - K / 2 + q, na, bc); }
+  __device__ __forceinline__ void centre(int e, double& r, double& cs, double (&v)[NV - 2]) const {
+    const long long x = cell(K / 2 - 1 + e);
+    r = __ldg(rho + x);
+    cs = __ldg(c + x);
+#pragma unroll
+    for (int d = 0; d < NV - 2; ++d) v[d] = __ldg(vel[d] + x);
+  }
+  __device__ __forceinline__ void speed(int q, double& u, double& cs) const {
+    const long long x = cell(q);
+    u = __ldg(un + x);
+    cs = __ldg(c + x);
+  }
+  __device__ __forceinline__ void speed32(int, double u, double cs, float& uf, float& cf) const {
+    uf = f32_rz(u);
+    cf = f32_rz(cs);
+  }
+};
+
+/* Roe state and LLF speeds of one face into its row (entry r at row[r * TH]).  src.centre(e, rho,
+   c, v): density, sound speed and velocity (normal first) of the face's left (0) and right (1)
+   cell; src.speed(q, u_n, c): stencil point q, speed32: truncated to FP32.  c~^2 in its cancellation-free form (weighted c^2
+   plus (gamma - 1)/2 wl wr |dv|^2), H~ = c~^2/(gamma - 1) + |u~|^2/2. */
+template <int NV, int K, int TH, class Src>
+__device__ __forceinline__ void face_rows(const Src& src, double* row, double gm1, double rgm1, int& st) {
+  using R = NlRow<NV>;
+  constexpr int D = NV - 2;
+  double sr[2], cs[2], v[2][D];
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    double rho;
+    src.centre(e, rho, cs[e], v[e]);
+    sr[e] = rho * rsqrt_nr(rho);
+  }
+  const double ws = rcp_nr(sr[0] + sr[1]), wl = sr[0] * ws, wr = sr[1] * ws;
+  double q2 = 0.0, dv2 = 0.0;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const double x = fma(wl, v[0][d], wr * v[1][d]), y = v[1][d] - v[0][d];
+    q2 = fma(x, x, q2);
+    dv2 = fma(y, y, dv2);
+    row[(R::u + d) * TH] = x;
+  }
+  const double c2 = fma(wl * cs[0], cs[0], fma(wr * cs[1], cs[1], 0.5 * gm1 * (wl * wr) * dv2));
+  if (!(c2 > 0.0)) st |= ST_ROE;
+  const double ci = rsqrt_nr(c2);
+  const double b1 = gm1 * (ci * ci);
+  row[R::H * TH] = fma(c2, rgm1, 0.5 * q2);
+  row[R::ci * TH] = ci;
+  row[R::ct * TH] = c2 * ci;
+  row[R::b1 * TH] = b1;
+  row[R::b2 * TH] = 0.5 * q2 * b1;
+  /* LLF: alpha_s = max over the K stencil points of |lambda_s|, one per eigenvalue family.  The
+     largest |u -+ c| is found in FP32 (each within 5u (|u| + c)) and formed in FP64 where it is
+     the only candidate; ties within the error take all K points in FP64 */
+  double am = 0.0, a0 = 0.0, ap = 0.0;
+  float bm = -1.f, bp = -1.f, sm = -1.f, sp = -1.f, ah = 0.f;
+  int qm = 0, qp = 0;
+#pragma unroll 1
+  for (int q = 0; q < K; ++q) {
+    double un, c;
+    src.speed(q, un, c);
+    a0 = imax_nonneg(a0, iabs(un));
+    float uf, cf;
+    src.speed32(q, un, c, uf, cf);
+    const float xm = fabsf(uf - cf), xp = fabsf(uf + cf);
+    ah = fmaxf(ah, fabsf(uf) + cf);
+    sm = fmaxf(sm, fminf(xm, bm));
+    sp = fmaxf(sp, fminf(xp, bp));
+    if (xm > bm) {
+      bm = xm;
+      qm = q;
+    }
+    if (xp > bp) {
+      bp = xp;
+      qp = q;
+    }
+  }
+  const float tie = 10.f * 5.9604645e-8f * ah;
+  if (bm - sm > tie && bp - sp > tie && ah < 1e30f && ah > 1e-30f) {
+    double un, c;
+    src.speed(qm, un, c);
+    am = iabs(un - c);
+    src.speed(qp, un, c);
+    ap = iabs(un + c);
+  } else {
+#pragma unroll 1
+    for (int q = 0; q < K; ++q) {
+      double un, c;
+      src.speed(q, un, c);
+      am = imax_nonneg(am, iabs(un - c));
+      ap = imax_nonneg(ap, iabs(un + c));
+    }
+  }
+  row[R::am * TH] = am;
+  row[R::a0 * TH] = a0;
+  row[R::ap * TH] = ap;
+}
+
+/* left eigenvector l_s of a face's row (closed form of R^{-1}; shear: l = e_t - u_t e_0, l[0] only);
+   returns alpha_s / 2 */
+template <int NV, int TH>
+__device__ __forceinline__ double left_vector(const double* face, int s, double (&l)[NV]) {
+  using R = NlRow<NV>;
+  constexpr int D = NV - 2;
+  auto row = [&](int r) -> double { return face[r * TH]; };
+  if (s == 0 || s == NV - 1) {
+    const double ci = (s == 0) ? 0.5 * row(R::ci) : -0.5 * row(R::ci), b1 = 0.5 * row(R::b1), un = row(R::u);
+    l[0] = fma(un, ci, 0.5 * row(R::b2));
+    l[1] = -fma(b1, un, ci);
+#pragma unroll
+    for (int d = 1; d < D; ++d) l[1 + d] = -b1 * row(R::u + d);
+    l[NV - 1] = b1;
+  } else if (s == 1) {
+    const double b1 = row(R::b1);
+    l[0] = 1.0 - row(R::b2);
+#pragma unroll
+    for (int d = 0; d < D; ++d) l[1 + d] = b1 * row(R::u + d);
+    l[NV - 1] = -b1;
+  } else {
+    l[0] = -row(R::u + (s - 1));
+#pragma unroll
+    for (int v = 1; v < NV; ++v) l[v] = 0.0;
+  }
+  return 0.5 * row(s == 0 ? R::am : (s == NV - 1 ? R::ap : R::a0));
+}
+
+/* Both split sides of a field from its W and G/2 in FP64, through one copy of the decisions and the
+   reconstruction: f+ on g+_q = G_q/2 + (alpha/2) W_q, f- on g-_q = G_q/2 - (alpha/2) W_q mirrored
+   about x_{i+1/2}; adds f+ + f- to fsum.  REC: op, om receive the frozen linear weights. */
+template <int K, int LIM, bool REC>
+__device__ __forceinline__ void general_sides(const double (&w)[K], const double (&hg)[K], double ha, const SchemeDev& S,
+                                              unsigned& fl, double& fsum, double* op, double* om, int& st) {
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    double v[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) v[q] = side ? fma(-ha, w[K - 1 - q], hg[K - 1 - q]) : fma(ha, w[q], hg[q]);
+    unsigned b = 0;
+    int e = 7;
+    if (!teno_decide_fast<K>(v, S, b, e)) teno_decide_fp64<K>(v, S, b, e, st);
+    if constexpr (REC) {
+      double wt[K];
+      fsum += teno_general<K, LIM, true>(v, S, b, wt);
+#pragma unroll
+      for (int q = 0; q < K; ++q) {
+        if (side) om[q] = wt[q];
+        else op[q] = wt[q];
+      }
+    } else {
+      fsum += teno_general<K, LIM>(v, S, b);
+    }
+    fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
+  }
+}
+
+/* Face flux from the central one, F = Fc on entry (components in the axis's frame): Fc + sum_s r_s
+   correction_s; when a field is direct (dir), sum_s r_s fs with fs = l_s . Fc (+ correction) for
+   the others.  cm: central fields.  Both sums go through the vectors the eigenvectors share: a =
+   (b2, -b1 u, b1) and b = (u_n, -e_n, 0)/c give l_{u-c} = (a + b)/2, l_{u+c} = (a - b)/2,
+   l_entropy = e_0 - a, l_shear = e_t - u_t e_0, and with sigma = f_{u-c} + f_{u+c}, delta =
+   (f_{u+c} - f_{u-c}) c:  F_0 = sigma + f_1,  F_d = (sigma + f_1) u_d + (delta if d = n, else
+   f_shear(d)),  F_E = sigma H + delta u_n + f_1 |u|^2/2 + sum_t f_t u_t. */
+template <int NV, int TH>
+__device__ __forceinline__ void compose(const double* face, const double* fsv, unsigned cm, unsigned dir,
+                                        double (&F)[NV]) {
+  using R = NlRow<NV>;
+  constexpr int D = NV - 2;
+  auto row = [&](int r) -> double { return face[r * TH]; };
+  double ut[D], fs[NV], q2 = 0.0;
+#pragma unroll
+  for (int s = 0; s < NV; ++s) fs[s] = (cm >> s & 1u) ? 0.0 : fsv[s * TH];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    ut[d] = row(R::u + d);
+    q2 = fma(ut[d], ut[d], q2);
+  }
+  if (dir) {
+    double uF = 0.0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) uF = fma(ut[d], F[1 + d], uF);
+    const double a = fma(row(R::b2), F[0], row(R::b1) * (F[NV - 1] - uF));
+    const double b = row(R::ci) * fma(ut[0], F[0], -F[1]);
+    if (!(dir & 1u)) fs[0] += 0.5 * (a + b);
+    if (!(dir >> (NV - 1) & 1u)) fs[NV - 1] += 0.5 * (a - b);
+    if (!(dir >> 1 & 1u)) fs[1] += F[0] - a;
+#pragma unroll
+    for (int s = 2; s <= NV - 2; ++s)
+      if (!(dir >> s & 1u)) fs[s] += fma(-ut[s - 1], F[0], F[s]);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) F[v] = 0.0;
+  }
+  const double sigma = fs[0] + fs[NV - 1];
+  const double delta = (fs[NV - 1] - fs[0]) * row(R::ct);
+  const double m = sigma + fs[1];
+  double FE = fma(sigma, row(R::H), fma(delta, ut[0], 0.5 * q2 * fs[1]));
+  F[0] += m;
+  F[1] += fma(m, ut[0], delta);
+#pragma unroll
+  for (int s = 2; s <= NV - 2; ++s) {
+    F[s] += fma(m, ut[s - 1], fs[s]);
+    FE = fma(ut[s - 1], fs[s], FE);
+  }
+  F[NV - 1] += FE;
+}
+
 /* The rare FP64 paths of the fixed-point kernel, called rather than inlined: they are larger
    than the path every item takes, and instruction fetch is what that path waits for.  w, g: the
    item's W and G/2 of point q at q * NL_THREADS; side 1: the mirrored stencil of f-. */
@@ -250,86 +462,18 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
         base = (long long)x + (ax == 1 ? (long long)A.n[0] * A.n[1] * hi : (long long)A.n[0] * lo);
       }
       if (bc == 0 && f == 0) fcopy = flin + na * (ax == 0 ? 1ll : (ax == 1 ? (long long)A.n[0] : sa));
-      /* Roe average of the face's two cells; c~^2 in its cancellation-free form (weighted c^2 plus
-         (gamma - 1)/2 wl wr |dv|^2), H~ = c~^2/(gamma - 1) + |u~|^2/2 */
-      double sr[2], cs[2], v[2][D];
+      GridFace<NV, K> src;
+      src.rho = up[0];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const long long cell = base + sa * bc_near(f - 1 + e, na, bc);
-        const double rho = __ldg(up[0] + cell);
-        sr[e] = rho * rsqrt_nr(rho);
-        cs[e] = __ldg(Pc + cell);
-#pragma unroll
-        for (int d = 0; d < D; ++d) v[e][d] = __ldg(A.P + (gc(1 + d) - 1) * A.ncell + cell);
-      }
-      const double gm1 = A.gamma - 1.0;
-      const double ws = rcp_nr(sr[0] + sr[1]), wl = sr[0] * ws, wr = sr[1] * ws;
-      double q2 = 0.0, dv2 = 0.0;
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        const double x = fma(wl, v[0][d], wr * v[1][d]), y = v[1][d] - v[0][d];
-        q2 = fma(x, x, q2);
-        dv2 = fma(y, y, dv2);
-        s_row[(R::u + d) * TH + tid] = x;
-      }
-      const double c2 = fma(wl * cs[0], cs[0], fma(wr * cs[1], cs[1], 0.5 * gm1 * (wl * wr) * dv2));
-      if (!(c2 > 0.0)) st |= ST_ROE;
-      const double ci = rsqrt_nr(c2);
-      const double b1 = gm1 * (ci * ci);
-      s_row[R::H * TH + tid] = fma(c2, A.rgm1, 0.5 * q2);
-      s_row[R::ci * TH + tid] = ci;
-      s_row[R::ct * TH + tid] = c2 * ci;
-      s_row[R::b1 * TH + tid] = b1;
-      s_row[R::b2 * TH + tid] = 0.5 * q2 * b1;
-      /* LLF: alpha_s = max over the K stencil points of |lambda_s|, one per eigenvalue family.  The
-         largest |u -+ c| is found in FP32 (each within 5u (|u| + c)) and formed in FP64 where it is
-         the only candidate; ties within the error take all K points in FP64 */
-      double am = 0.0, a0 = 0.0, ap = 0.0;
-      float bm = -1.f, bp = -1.f, sm = -1.f, sp = -1.f, ah = 0.f;
-      int qm = 0, qp = 0;
-      auto speeds = [&](int q, double& un, double& c) {
-        const long long cell = base + sa * bc_near(f - H + q, na, bc);
-        un = __ldg(Pn + cell);
-        c = __ldg(Pc + cell);
-      };
-#pragma unroll 1
-      for (int q = 0; q < K; ++q) {
-        double un, c;
-        speeds(q, un, c);
-        a0 = imax_nonneg(a0, iabs(un));
-        const float uf = f32_rz(un), cf = f32_rz(c);
-        const float xm = fabsf(uf - cf), xp = fabsf(uf + cf);
-        ah = fmaxf(ah, fabsf(uf) + cf);
-        sm = fmaxf(sm, fminf(xm, bm));
-        sp = fmaxf(sp, fminf(xp, bp));
-        if (xm > bm) {
-          bm = xm;
-          qm = q;
-        }
-        if (xp > bp) {
-          bp = xp;
-          qp = q;
-        }
-      }
-      const float tie = 10.f * 5.9604645e-8f * ah;
-      if (bm - sm > tie && bp - sp > tie && ah < 1e30f && ah > 1e-30f) {
-        double un, c;
-        speeds(qm, un, c);
-        am = iabs(un - c);
-        speeds(qp, un, c);
-        ap = iabs(un + c);
-      } else {
-#pragma unroll 1
-        for (int q = 0; q < K; ++q) {
-          double un, c;
-          speeds(q, un, c);
-          am = imax_nonneg(am, iabs(un - c));
-          ap = imax_nonneg(ap, iabs(un + c));
-        }
-      }
-      s_row[R::am * TH + tid] = am;
-      s_row[R::a0 * TH + tid] = a0;
-      s_row[R::ap * TH + tid] = ap;
+      for (int d = 0; d < D; ++d) src.vel[d] = A.P + (gc(1 + d) - 1) * A.ncell;
+      src.un = Pn;
+      src.c = Pc;
+      src.base = base;
+      src.sa = sa;
+      src.f = f;
+      src.na = na;
+      src.bc = bc;
+      face_rows<NV, K, TH>(src, s_row + tid, A.gamma - 1.0, A.rgm1, st);
       s_base[tid] = base;
       s_f[tid] = f;
       s_cm[tid] = A.sch.default_d ? (allf & ~mask) : 0u;
@@ -373,29 +517,9 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
     for (int it = tid; it < npass; it += TH) {
       const unsigned item = pass ? s_later[it] : s_item[it];
       const int fc = item & 255, s = item >> 8;
-      auto row = [&](int r) -> double { return s_row[r * TH + fc]; };
-      const bool acoustic = s == 0 || s == NV - 1, shear = s >= 2 && s <= NV - 2;
-      const double ha = 0.5 * row(s == 0 ? R::am : (s == NV - 1 ? R::ap : R::a0));
-      /* left eigenvector l_s (closed form of R^{-1}); shear: l = e_t - u_t e_0 */
+      const bool shear = s >= 2 && s <= NV - 2;
       double l[NV];
-      if (acoustic) {
-        const double ci = (s == 0) ? 0.5 * row(R::ci) : -0.5 * row(R::ci), b1 = 0.5 * row(R::b1), un = row(R::u);
-        l[0] = fma(un, ci, 0.5 * row(R::b2));
-        l[1] = -fma(b1, un, ci);
-#pragma unroll
-        for (int d = 1; d < D; ++d) l[1 + d] = -b1 * row(R::u + d);
-        l[NV - 1] = b1;
-      } else if (s == 1) {
-        const double b1 = row(R::b1);
-        l[0] = 1.0 - row(R::b2);
-#pragma unroll
-        for (int d = 0; d < D; ++d) l[1 + d] = b1 * row(R::u + d);
-        l[NV - 1] = -b1;
-      } else {
-        l[0] = -row(R::u + (s - 1));
-#pragma unroll
-        for (int v = 1; v < NV; ++v) l[v] = 0.0;
-      }
+      const double ha = left_vector<NV, TH>(s_row + fc, s, l);
       const double* const ut = A.U + gc(shear ? s : 1) * A.ncell;
       const long long base = s_base[fc];
       const int f = s_f[fc];
@@ -442,29 +566,7 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
           project(q, w[q], hg[q]);
           if constexpr (REC) wv[q] = w[q];
         }
-        /* the two split sides through one copy of the decisions and the reconstruction: f+ on
-           g+_q = G_q/2 + (alpha/2) W_q, f- on g-_q = G_q/2 - (alpha/2) W_q mirrored about x_{i+1/2} */
-#pragma unroll 1
-        for (int side = 0; side < 2; ++side) {
-          double v[K];
-#pragma unroll
-          for (int q = 0; q < K; ++q) v[q] = side ? fma(-ha, w[K - 1 - q], hg[K - 1 - q]) : fma(ha, w[q], hg[q]);
-          unsigned b = 0;
-          int e = 7;
-          if (!teno_decide_fast<K>(v, A.sch, b, e)) teno_decide_fp64<K>(v, A.sch, b, e, st);
-          if constexpr (REC) {
-            double wt[K];
-            fsum += teno_general<K, LIM, true>(v, A.sch, b, wt);
-#pragma unroll
-            for (int q = 0; q < K; ++q) {
-              if (side) om[q] = wt[q];
-              else op[q] = wt[q];
-            }
-          } else {
-            fsum += teno_general<K, LIM>(v, A.sch, b);
-          }
-          fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
-        }
+        general_sides<K, LIM, REC>(w, hg, ha, A.sch, fl, fsum, op, om, st);
       }
       s_fs[s * TH + fc] = fsum;
       /* a field found all smooth on both sides is central after all: the flux does not depend on
@@ -503,54 +605,14 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
     __syncthreads();
     }
 
-    /* ---- (2) Fhat = Fc when every field is central; Fc + sum_s r_s correction_s when the others
-       are corrections; else sum_s r_s fs with fs = l_s . Fc (+ correction) for the fields that are
-       not direct.  Both sums go through the vectors the eigenvectors share: a = (b2, -b1 u, b1)
-       and b = (u_n, -e_n, 0)/c give l_{u-c} = (a + b)/2, l_{u+c} = (a - b)/2, l_entropy = e_0 - a,
-       l_shear = e_t - u_t e_0, and with sigma = f_{u-c} + f_{u+c}, delta = (f_{u+c} - f_{u-c}) c:
-       F_0 = sigma + f_1,  F_d = (sigma + f_1) u_d + (delta if d = n, else f_shear(d)),
-       F_E = sigma H + delta u_n + f_1 |u|^2/2 + sum_t f_t u_t. ---- */
+    /* ---- (2) the face fluxes ---- */
     if (tid < nf && s_cm[tid] != allf) {
       const unsigned cm = s_cm[tid], dir = s_dir[tid];
-      auto row = [&](int r) -> double { return s_row[r * TH + tid]; };
       double* const Fo = A.Fhat[ax];
-      double Fc[NV], ut[D], fs[NV], Fh[NV], q2 = 0.0;
+      double Fh[NV];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) Fc[v] = Fo[gc(v) * nface + flin];
-#pragma unroll
-      for (int s = 0; s < NV; ++s) fs[s] = (cm >> s & 1u) ? 0.0 : s_fs[s * TH + tid];
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        ut[d] = row(R::u + d);
-        q2 = fma(ut[d], ut[d], q2);
-      }
-      if (dir) {
-        double uF = 0.0;
-#pragma unroll
-        for (int d = 0; d < D; ++d) uF = fma(ut[d], Fc[1 + d], uF);
-        const double a = fma(row(R::b2), Fc[0], row(R::b1) * (Fc[NV - 1] - uF));
-        const double b = row(R::ci) * fma(ut[0], Fc[0], -Fc[1]);
-        if (!(dir & 1u)) fs[0] += 0.5 * (a + b);
-        if (!(dir >> (NV - 1) & 1u)) fs[NV - 1] += 0.5 * (a - b);
-        if (!(dir >> 1 & 1u)) fs[1] += Fc[0] - a;
-#pragma unroll
-        for (int s = 2; s <= NV - 2; ++s)
-          if (!(dir >> s & 1u)) fs[s] += fma(-ut[s - 1], Fc[0], Fc[s]);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) Fc[v] = 0.0;
-      }
-      const double sigma = fs[0] + fs[NV - 1];
-      const double delta = (fs[NV - 1] - fs[0]) * row(R::ct);
-      const double m = sigma + fs[1];
-      double FE = fma(sigma, row(R::H), fma(delta, ut[0], 0.5 * q2 * fs[1]));
-      Fh[0] = Fc[0] + m;
-      Fh[1] = Fc[1] + fma(m, ut[0], delta);
-#pragma unroll
-      for (int s = 2; s <= NV - 2; ++s) {
-        Fh[s] = Fc[s] + fma(m, ut[s - 1], fs[s]);
-        FE = fma(ut[s - 1], fs[s], FE);
-      }
-      Fh[NV - 1] = Fc[NV - 1] + FE;
+      for (int v = 0; v < NV; ++v) Fh[v] = Fo[gc(v) * nface + flin];
+      compose<NV, TH>(s_row + tid, s_fs + tid, cm, dir, Fh);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         Fo[gc(v) * nface + flin] = Fh[v];

@@ -88,8 +88,9 @@ __device__ __forceinline__ bool quick_smooth(const float (&d)[K - 1], float E, c
   const float L = 0.966f * lo, U = fmaf(1.0315f, hi, (1.04f * BetaNorm<K>::kmax) * e2);
   const float r1 = (R - 1.f) * L;
   /* written so that a NaN fails; dm <= 1e15 keeps every form finite, and the product form
-     needs L away from the underflow range */
-  return dm <= 1e15f && lo >= 1e-30f && (T <= r1 || (lo >= 1e-18f && T * (U - R * L) <= r1 * U));
+     needs its factors away from under- and overflow */
+  return dm <= 1e15f && lo >= 1e-30f &&
+         (T <= r1 || (lo >= 1e-18f && U <= 1e15f && T <= 1e17f && T * (U - R * L) <= r1 * U));
 }
 
 /* FP32 data of a staged point (component c of point p at c * NP + p): rho, velocity, p and c as
@@ -111,6 +112,45 @@ __device__ __forceinline__ float f32_rest(double x) {
   if (e < -126 || e > 127) return 0.f;                          /* far outside the FP32 range: hi is 0 or inf, or the rest is below 2^-97 */
   const float r = m * __int_as_float((e + 127) << 23);
   return (int)hi < 0 ? -r : r;
+}
+
+/* the screen's data of point p, and (once all points are there) its differences to point p + step */
+template <int NV>
+__device__ __forceinline__ void stage_screen_point(const double (&u)[NV], const double (&vel)[NV - 2], double pr, double cs,
+                                                   float* sf, int NP, int p) {
+  using L = ScreenLayout<NV>;
+  unsigned chk = 0u;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const unsigned x = (unsigned)__double2loint(u[v]);
+    chk ^= __funnelshift_l(x, x, 6 * v);
+  }
+  sf[L::chk * NP + p] = __uint_as_float(chk);
+  auto put = [&](int c, double x) {
+    sf[(L::hi + c) * NP + p] = f32_rz(x);
+    sf[(L::lo + c) * NP + p] = f32_rest(x);
+  };
+  put(L::R, u[0]);
+#pragma unroll
+  for (int d = 0; d < NV - 2; ++d) put(L::V + d, vel[d]);
+  put(L::P, pr);
+  put(L::C, cs);
+}
+template <int NV>
+__device__ __forceinline__ void stage_screen_differences(float* sf, int NP, int p, int step) {
+  using L = ScreenLayout<NV>;
+  float any = 0.f;
+#pragma unroll
+  for (int c = L::NQ - 1; c >= 0; --c) {  /* rho (c = 0) last */
+    const float* h = sf + (L::hi + c) * NP + p;
+    const float* l = sf + (L::lo + c) * NP + p;
+    float x = (h[step] - h[0]) + (l[step] - l[0]);
+    any = fmaxf(any, fabsf(x));
+    /* equal to 47 bits but not bit for bit: not a constant stencil (nor one that can be certified) */
+    if (c == 0 && any == 0.f &&
+        __float_as_uint(sf[L::chk * NP + p + step]) != __float_as_uint(sf[L::chk * NP + p])) x = 1e-37f;
+    sf[(L::df + c) * NP + p] = x;
+  }
 }
 
 /* Fields of one face that are NOT certified central (bit s); the face's stencil point q is
@@ -459,39 +499,12 @@ screen_kernel(const FaceArgs A) {
 #pragma unroll
     for (int d = 0; d < D; ++d) F[1 + d] = (d == AXIS) ? fma(u[1 + d], vel[AXIS], pr) : u[1 + d] * vel[AXIS];
     F[NV - 1] = (u[NV - 1] + pr) * vel[AXIS];
-    unsigned chk = 0u;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      sF[v * NP + p] = F[v];
-      const unsigned x = (unsigned)__double2loint(u[v]);
-      chk ^= __funnelshift_l(x, x, 6 * v);
-    }
-    sf[L::chk * NP + p] = __uint_as_float(chk);
-    auto put = [&](int c, double x) {
-      sf[(L::hi + c) * NP + p] = f32_rz(x);
-      sf[(L::lo + c) * NP + p] = f32_rest(x);
-    };
-    put(L::R, u[0]);
-#pragma unroll
-    for (int d = 0; d < D; ++d) put(L::V + d, vel[d]);
-    put(L::P, pr);
-    put(L::C, cs);
+    for (int v = 0; v < NV; ++v) sF[v * NP + p] = F[v];
+    stage_screen_point<NV>(u, vel, pr, cs, sf, NP, p);
   }
   __syncthreads();
-  for (int p = tid; p < NP - T::LANES; p += T::THREADS) {
-    float any = 0.f;
-#pragma unroll
-    for (int c = L::NQ - 1; c >= 0; --c) {  /* rho (c = 0) last */
-      const float* h = sf + (L::hi + c) * NP + p;
-      const float* l = sf + (L::lo + c) * NP + p;
-      float x = (h[T::LANES] - h[0]) + (l[T::LANES] - l[0]);
-      any = fmaxf(any, fabsf(x));
-      /* equal to 47 bits but not bit for bit: not a constant stencil (nor one that can be certified) */
-      if (c == 0 && any == 0.f &&
-          __float_as_uint(sf[L::chk * NP + p + T::LANES]) != __float_as_uint(sf[L::chk * NP + p])) x = 1e-37f;
-      sf[(L::df + c) * NP + p] = x;
-    }
-  }
+  for (int p = tid; p < NP - T::LANES; p += T::THREADS) stage_screen_differences<NV>(sf, NP, p, T::LANES);
   __syncthreads();
 
   /* --- one face per thread --- */
