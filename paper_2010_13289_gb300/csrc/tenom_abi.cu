@@ -10,7 +10,7 @@
 
 #include "tenom.h"
 #include "tenom_internal.h"
-#include "tenom_adjoint_kernels.cuh"
+#include "tenom_adjoint.cuh"
 #include "tenom_nonlinear.cuh"
 #include "tenom_line.cuh"
 
@@ -1058,29 +1058,30 @@ static size_t lin_offset(const tenom_ctx* c, int axis) {
   return b;
 }
 
+/* Z = L'(U)^T w from one stage's flags or linearisation */
 static cudaError_t adj_sweeps(tenom_ctx* c, const double* U, const uint8_t* flags_stage, const double* lin_stage,
                               const double* w, double* Z) {
-  cudaError_t e = cudaMemsetAsync(Z, 0, sizeof(double) * c->nv * c->ncell, c->st);
-  if (e == cudaSuccess) e = launch_prims(c, U, true);
-  for (int a = 0; a < c->g.dim && e == cudaSuccess; ++a) {
-    AdjArgs A;
-    memset(&A, 0, sizeof(A));
-    A.U = U;
-    A.flags = flags_stage ? flags_stage + flags_offset(c, a) : nullptr;
-    A.lin = lin_stage ? lin_stage + lin_offset(c, a) : nullptr;
-    A.P = c->P;
-    A.w = w;
-    A.Z = Z;
-    A.status = c->status;
-    for (int d = 0; d < 3; ++d) {
-      A.n[d] = c->g.n[d];
-      A.bc[d] = c->g.bc[d];
+  AdjArgs A;
+  memset(&A, 0, sizeof(A));
+  A.U = U;
+  A.P = c->P;
+  A.w = w;
+  A.Z = Z;
+  for (int d = 0; d < 3; ++d) {
+    A.n[d] = c->g.n[d];
+    A.bc[d] = c->g.bc[d];
+    A.rdx[d] = 1.0 / c->g.dx[d];
+  }
+  A.ncell = c->ncell;
+  A.gamma = c->g.gamma;
+  A.sch = scheme_dev(c->s);
+  cudaError_t e = launch_prims(c, U, true);
+  for (int a = -1; a < c->g.dim && e == cudaSuccess; ++a) {
+    if (a >= 0) {
+      A.flags = flags_stage ? flags_stage + flags_offset(c, a) : nullptr;
+      A.lin = lin_stage ? lin_stage + lin_offset(c, a) : nullptr;
+      A.nface = c->nface[a];
     }
-    A.ncell = c->ncell;
-    A.nface = c->nface[a];
-    A.dx = c->g.dx[a];
-    A.gamma = c->g.gamma;
-    A.sch = scheme_dev(c->s);
     if (c->nv == 3) e = launch_adj_nv3(A, a, c->s.K, c->s.limiter, c->st);
     else if (c->nv == 4) e = launch_adj_nv4(A, a, c->s.K, c->s.limiter, c->st);
     else e = launch_adj_nv5(A, a, c->s.K, c->s.limiter, c->st);
@@ -1088,11 +1089,14 @@ static cudaError_t adj_sweeps(tenom_ctx* c, const double* U, const uint8_t* flag
   return e;
 }
 
+/* room for three stages' cutoff flags */
+static cudaError_t ensure_flags(tenom_ctx* c) {
+  return c->adj_flags ? cudaSuccess : cudaMalloc(&c->adj_flags, tenom_flags_bytes(c) * 3);
+}
+
 static cudaError_t ensure_adj(tenom_ctx* c) {
-  if (c->adj) return cudaSuccess;
-  cudaError_t e = cudaMalloc(&c->adj, sizeof(double) * c->nv * c->ncell * 7);
-  if (e == cudaSuccess) e = cudaMalloc(&c->adj_flags, tenom_flags_bytes(c) * 3);
-  return e;
+  cudaError_t e = c->adj ? cudaSuccess : cudaMalloc(&c->adj, sizeof(double) * c->nv * c->ncell * 7);
+  return e == cudaSuccess ? ensure_flags(c) : e;
 }
 
 static cudaError_t lincomb(tenom_ctx* c, double* out, double c0, const double* x0, double c1, const double* x1,
@@ -1107,7 +1111,13 @@ tenom_status tenom_rhs_vjp(tenom_ctx* c, const double* U, const double* w, doubl
   if (adjoint_unsupported(c, "rhs_vjp")) return TENOM_E_UNSUPPORTED;
   if (!aligned8(U) || !aligned8(w) || !aligned8(Ubar) || Ubar == U || Ubar == w)
     return fail(c, TENOM_E_INVALID, "rhs_vjp: bad pointers");
-  cudaError_t e = adj_sweeps(c, U, nullptr, nullptr, w, Ubar);
+  /* the branches at U: one forward pass over the faces with flags */
+  cudaError_t e = ensure_flags(c);
+  uint8_t* fl[3] = {nullptr, nullptr, nullptr};
+  for (int a = 0; a < c->g.dim && e == cudaSuccess; ++a) fl[a] = c->adj_flags + flags_offset(c, a);
+  if (e == cudaSuccess) e = launch_prims(c, U);
+  if (e == cudaSuccess) e = launch_faces(c, U, 0, c->g.dim, c->face, fl, nullptr);
+  if (e == cudaSuccess) e = adj_sweeps(c, U, c->adj_flags, nullptr, w, Ubar);
   return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "rhs_vjp");
 }
 

@@ -1,4 +1,4 @@
-/* Adjoint face-kernel instantiations for nvar = 5 (flags and linearisation-tape sweeps). */
+/* Adjoint instantiations for nvar = 5 (flags and linearisation tape). */
 #include "tenom_launch.cuh"
 
 namespace tenom {

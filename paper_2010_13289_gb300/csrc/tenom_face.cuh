@@ -17,7 +17,6 @@
 #pragma once
 #include <cstdint>
 #include "tenom_recon.cuh"
-#include "tenom_linear.cuh"
 #include "tenom_stats.cuh"
 #include "tenom_fastmath.cuh"
 

@@ -64,8 +64,8 @@ cudaError_t launch_rhs_divergence(int nv, double* const F[3], const int n[3], co
 
 namespace tenom {
 struct AdjArgs;
-/* Launch the adjoint face sweep of (NV, K, limiter, axis): Z += L_a'(U)^T w, from a.lin (the
-   recorded linearisation) when set, else from a.flags (or branches decided again). */
+/* Adjoint launches: axis < 0 writes the central part of L'(U)^T w (all axes) to a.Z; axis >= 0 adds the
+   axis's nonlinear fields, from a.lin (the recorded linearisation) when set, else from a.flags. */
 cudaError_t launch_adj_nv3(const AdjArgs& a, int axis, int K, int lim, cudaStream_t st);
 cudaError_t launch_adj_nv4(const AdjArgs& a, int axis, int K, int lim, cudaStream_t st);
 cudaError_t launch_adj_nv5(const AdjArgs& a, int axis, int K, int lim, cudaStream_t st);

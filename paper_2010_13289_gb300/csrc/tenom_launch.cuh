@@ -9,7 +9,7 @@
 #include "tenom_internal.h"
 #include "tenom_screen.cuh"
 #include "tenom_nonlinear.cuh"
-#include "tenom_adjoint_kernels.cuh"
+#include "tenom_adjoint.cuh"
 
 namespace tenom {
 
@@ -142,40 +142,37 @@ static cudaError_t launch_stats_nv(const FaceArgs& a, int axis, int K, int lim, 
   return cudaErrorNotSupported;
 }
 
-/* adjoint sweep with flags (or branches decided again) */
-template <int NV, int K, int LIM, int AXIS>
-static cudaError_t launch_adj_one(const AdjArgs& a, cudaStream_t st) {
+/* reverse of the axis's nonlinear fields (from a.lin, else from a.flags) */
+template <int NV, int K, int LIM, int AXIS, bool TAPE>
+static cudaError_t launch_adj_fields_one(const AdjArgs& a, cudaStream_t st) {
   static AttrOnce attr;
-  return launch_tile(adj_face_kernel<NV, K, LIM, AXIS>, attr, AdjTile<NV, K, AXIS>::SMEM, NV, AXIS, a.n, K, st,
-                     &a);
+  return launch_tile(adj_fields_kernel<NV, K, LIM, AXIS, TAPE>, attr, AdjTile<NV, K, AXIS>::SMEM, NV, AXIS, a.n, K, st, &a,
+                     false, true);
 }
 
-/* adjoint sweep from a recorded linearisation (no limiter dependence) */
 template <int NV, int K, int AXIS>
-static cudaError_t launch_adj_lin_one(const AdjArgs& a, cudaStream_t st) {
-  static AttrOnce attr;
-  return launch_tile(adj_lin_kernel<NV, K, AXIS>, attr, AdjLinTile<NV, K, AXIS>::SMEM, NV, AXIS, a.n, K, st, &a);
+static cudaError_t launch_adj_fields_k(const AdjArgs& a, int lim, cudaStream_t st) {
+  if (a.lin) return launch_adj_fields_one<NV, K, LIM_MP, AXIS, true>(a, st);  /* no limiter dependence */
+  if (lim == LIM_MP) return launch_adj_fields_one<NV, K, LIM_MP, AXIS, false>(a, st);
+  if (lim == LIM_TVD5) return launch_adj_fields_one<NV, K, LIM_TVD5, AXIS, false>(a, st);
+  return cudaErrorNotSupported;
 }
 
 template <int NV, int AXIS>
 static cudaError_t launch_adj_axis(const AdjArgs& a, int K, int lim, cudaStream_t st) {
-  if (a.lin) {
-    if (K == 6) return launch_adj_lin_one<NV, 6, AXIS>(a, st);
-    if (K == 8) return launch_adj_lin_one<NV, 8, AXIS>(a, st);
-    return cudaErrorNotSupported;
-  }
-  if (K == 6) {
-    if (lim == LIM_MP) return launch_adj_one<NV, 6, LIM_MP, AXIS>(a, st);
-    if (lim == LIM_TVD5) return launch_adj_one<NV, 6, LIM_TVD5, AXIS>(a, st);
-  } else if (K == 8) {
-    if (lim == LIM_MP) return launch_adj_one<NV, 8, LIM_MP, AXIS>(a, st);
-    if (lim == LIM_TVD5) return launch_adj_one<NV, 8, LIM_TVD5, AXIS>(a, st);
-  }
-  return cudaErrorNotSupported;
+  return K == 6 ? launch_adj_fields_k<NV, 6, AXIS>(a, lim, st) : launch_adj_fields_k<NV, 8, AXIS>(a, lim, st);
 }
 
+/* axis < 0: the central part (all axes), which writes a.Z; else the axis's fields added to it */
 template <int NV>
 static cudaError_t launch_adj_nv(const AdjArgs& a, int axis, int K, int lim, cudaStream_t st) {
+  if (axis < 0) {
+    const long long b = (a.ncell + 255) / 256;
+    const unsigned grid = (unsigned)(b < 152 * 64 ? b : 152 * 64);
+    if (K == 6) adj_central_kernel<NV, 6><<<grid, 256, 0, st>>>(a);
+    else adj_central_kernel<NV, 8><<<grid, 256, 0, st>>>(a);
+    return cudaGetLastError();
+  }
   if (axis == 0) return launch_adj_axis<NV, 0>(a, K, lim, st);
   if constexpr (NV >= 4)
     if (axis == 1) return launch_adj_axis<NV, 1>(a, K, lim, st);

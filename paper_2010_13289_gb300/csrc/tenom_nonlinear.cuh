@@ -31,6 +31,7 @@
 #include "tenom_recon.cuh"
 #include "tenom_face.cuh"
 #include "tenom_fixed.cuh"
+#include "tenom_adjoint.cuh"
 
 namespace tenom {
 
@@ -597,8 +598,9 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
             o[(2 + K + q) * nface] = dq;
             wW = fma(dq, wv[q], wW);
           }
+          const bool central = (fl & (allk | allk << 8)) == (allk | allk << 8) && A.sch.default_d;
           o[0] = fsum;
-          o[nface] = wW;
+          o[nface] = central ? __longlong_as_double((long long)kCentralMark) : wW + 0.0;
         }
       }
     }

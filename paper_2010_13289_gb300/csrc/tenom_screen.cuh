@@ -24,6 +24,7 @@
 #pragma once
 #include "tenom_recon.cuh"
 #include "tenom_face.cuh"
+#include "tenom_adjoint.cuh"
 
 namespace tenom {
 
@@ -444,7 +445,7 @@ constexpr size_t screen_smem() {
 }
 
 /* REC: also the linearisation of the certified fields (the record kernels' tape, see
-   nonlinear_kernel): sigma_q = c_q, delta_q = 0, omegaW = 0, fs = l_s . Fc. */
+   nonlinear_kernel): sigma_q = c_q, delta_q = 0, omegaW = -0 (kCentralMark), fs = l_s . Fc. */
 template <int NV, int K, int AXIS, bool REC>
 __global__ void __launch_bounds__(FaceTile<NV, K, AXIS, true>::THREADS,
                                   SCREEN_THREADS_PER_SM / FaceTile<NV, K, AXIS, true>::THREADS)
@@ -566,7 +567,7 @@ screen_kernel(const FaceArgs A) {
             if (bad >> s & 1u) continue;
             double* os = o + (long long)s * (2 * K + 2) * A.nface;
             os[0] = fs[s];
-            os[A.nface] = 0.0;
+            os[A.nface] = __longlong_as_double((long long)kCentralMark);  /* -0.0 */
 #pragma unroll
             for (int q = 0; q < K; ++q) {
               os[(2 + q) * A.nface] = 0.5 * (cw[q] + cw[K - 1 - q]);
