@@ -211,13 +211,18 @@ __device__ __forceinline__ void point_vjp(const double* sm, int NP, int p, doubl
 
 __device__ __forceinline__ double dsign(double x) { return ipos(x) ? 1.0 : (ineg(x) ? -1.0 : 0.0); }
 
-/* shared memory of adj_fields_kernel: the tile's points, per point the adjoints of U (NV), F (NV) and
-   |lambda| (3), per face the Roe-state adjoints of its two centre points */
+/* Tile of adj_fields_kernel (one thread per face) and its shared memory: the tile's points, per point
+   the adjoints of U (NV), F (NV) and |lambda| (3), per face the Roe-state adjoints of its two centre
+   points.  Along x 128 faces of a row; y/z 16 x columns by 16 faces (halving the tile would stage
+   1.9 points per face instead of 1.4).  A field's reverse is one serial chain, so a tile costs about
+   100 us however few faces it holds: small CTAs keep the tiles of a small grid in one wave. */
 template <int NV, int K, int AXIS>
 struct AdjTile {
-  using F = FaceTile<NV, K, AXIS, true>;
+  static constexpr int H = K / 2, LANES = AXIS == 0 ? 1 : 16;
+  static constexpr int FACES = AXIS == 0 ? 128 : 16;
+  static constexpr int THREADS = FACES * LANES, NP = (FACES + K - 1) * LANES;
   static constexpr int NA = 2 * NV + 3, NR = 2 * NV;
-  static constexpr size_t SMEM = sizeof(double) * ((size_t)(PointLayout<NV>::NC + NA) * F::NP + (size_t)NR * F::THREADS);
+  static constexpr size_t SMEM = sizeof(double) * ((size_t)(PointLayout<NV>::NC + NA) * NP + (size_t)NR * THREADS);
 };
 
 /* Adds the reverse of sum_s r_s f'_s of the axis's faces to Z.  A CTA finds its tile's faces with such
@@ -228,12 +233,12 @@ struct AdjTile {
    summed in shared memory in K phases (in phase q every face adds to its q-th point, all
    distinct); the reverse of the point quantities then runs once per touched point. */
 template <int NV, int K, int LIM, int AXIS, bool TAPE>
-__global__ void __launch_bounds__(FaceTile<NV, K, AXIS, true>::THREADS, NV == 3 ? 4 : (TAPE ? 2 : 1)) adj_fields_kernel(const AdjArgs A) {
-  using T = FaceTile<NV, K, AXIS, true>;
+__global__ void __launch_bounds__(AdjTile<NV, K, AXIS>::THREADS, (TAPE ? 512 : 256) / AdjTile<NV, K, AXIS>::THREADS)
+    adj_fields_kernel(const AdjArgs A) {
+  using T = AdjTile<NV, K, AXIS>;
   using L = PointLayout<NV>;
-  using TA = AdjTile<NV, K, AXIS>;
   constexpr int H = T::H, D = NV - 2, TH = T::THREADS, NP = T::NP, LANES = T::LANES, W = TH / 32;
-  constexpr int NA = TA::NA, NR = TA::NR, RS = 2 * K + 2;
+  constexpr int NA = T::NA, NR = T::NR, RS = 2 * K + 2;
   constexpr int aU = 0, aF = NV, aM = 2 * NV;  /* aM + 0 (u-c), 1 (u), 2 (u+c) */
   constexpr unsigned allk = (1u << (K - 2)) - 1u;
   extern __shared__ double sm[];

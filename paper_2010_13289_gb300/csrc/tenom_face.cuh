@@ -50,13 +50,12 @@ struct PointLayout {
   static constexpr int cLm = 3 * NV + 1, cLp = 3 * NV + 2;
 };
 
-constexpr int FX_FACES = 128;  /* faces per CTA, x sweeps of the statistics kernels and the adjoint */
+constexpr int FX_FACES = 128;  /* faces per CTA, x sweeps of the statistics kernels */
 /* threads (faces) per CTA of the screen: 256 in 2D and 3D (x sweeps 256 faces of a row, y/z
-   sweeps 16 x columns by 16 faces: 1.3-1.4 staged points per face), 64 for 1D grids (a short
-   line is latency-bound: it runs faster spread over more, smaller CTAs) */
-__host__ __device__ constexpr int fx_faces(int K, int NV) { return (void)K, NV > 3 ? 256 : 64; }
-/* faces per CTA along the axis of the statistics kernels and the adjoint sweeps, y/z
-   (x 32 lanes): 4, i.e. 128-thread CTAs */
+   sweeps 16 x columns by 16 faces: 1.3-1.4 staged points per face), 128 for 1D grids (the tile
+   index is the grid's y: 64 would halve the longest line) */
+__host__ __device__ constexpr int fx_faces(int K, int NV) { return (void)K, NV > 3 ? 256 : 128; }
+/* faces per CTA along the axis of the statistics kernels, y/z (x 32 lanes): 4, i.e. 128-thread CTAs */
 __host__ __device__ constexpr int ft_faces(int K) { return (void)K, 4; }
 /* screen, y/z sweeps: FWD_LANES x columns by fx_faces(K, NV) / FWD_LANES faces (a warp takes
    two face rows) */

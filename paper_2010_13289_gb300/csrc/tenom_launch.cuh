@@ -145,9 +145,15 @@ static cudaError_t launch_stats_nv(const FaceArgs& a, int axis, int K, int lim, 
 /* reverse of the axis's nonlinear fields (from a.lin, else from a.flags) */
 template <int NV, int K, int LIM, int AXIS, bool TAPE>
 static cudaError_t launch_adj_fields_one(const AdjArgs& a, cudaStream_t st) {
+  using T = AdjTile<NV, K, AXIS>;
   static AttrOnce attr;
-  return launch_tile(adj_fields_kernel<NV, K, LIM, AXIS, TAPE>, attr, AdjTile<NV, K, AXIS>::SMEM, NV, AXIS, a.n, K, st, &a,
-                     false, true);
+  const cudaError_t e = ensure_smem_attr(adj_fields_kernel<NV, K, LIM, AXIS, TAPE>, attr, T::SMEM);
+  if (e != cudaSuccess) return e;
+  const unsigned tiles = (unsigned)((a.n[AXIS] + T::FACES) / T::FACES);  /* n_a + 1 faces */
+  const dim3 grid = AXIS == 0 ? dim3((unsigned)(a.n[1] * a.n[2]), tiles)
+                              : dim3((unsigned)((a.n[0] + T::LANES - 1) / T::LANES), tiles, (unsigned)(AXIS == 1 ? a.n[2] : a.n[1]));
+  adj_fields_kernel<NV, K, LIM, AXIS, TAPE><<<grid, T::THREADS, T::SMEM, st>>>(a);
+  return cudaGetLastError();
 }
 
 template <int NV, int K, int AXIS>
