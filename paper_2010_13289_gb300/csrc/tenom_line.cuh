@@ -157,7 +157,7 @@ __device__ __forceinline__ void line_fluxes(LineTile<K, TILE, FACES>& S, int n, 
       }
       unsigned b = 0u;
       int e = 7;
-      if (!teno_decide_fast<K>(v, sch, b, e)) teno_decide_fp64<K>(v, sch, b, e, st);
+      if (!teno_decide_fast<K, false>(v, sch, b, e)) teno_decide_fp64<K>(v, sch, b, e, st);
       S.fs[(side * NV + s) * TILE + fc] = teno_general<K, LIM>(v, sch, b);
       if (b == allk && sch.default_d) atomicOr(&S.cm[side * TILE + fc], 1u << s);
     }
