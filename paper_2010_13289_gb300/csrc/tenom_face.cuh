@@ -60,8 +60,10 @@ __host__ __device__ constexpr int ft_faces(int K) { return (void)K, 4; }
 /* screen, y/z sweeps: FWD_LANES x columns by fx_faces(K, NV) / FWD_LANES faces (a warp takes
    two face rows) */
 constexpr int FWD_LANES = 16;
-/* resident threads per SM the screen is compiled for */
-constexpr int SCREEN_THREADS_PER_SM = 768;
+/* resident threads per SM the screen is compiled for.  1024 (64 registers) spill 100 bytes a thread
+   in TENO6, 210 in TENO8; 2048^2 steps 5.08 ms against 5.17 (TENO6) and 5.99 against 5.98 (TENO8),
+   777x531 TENO8 1.11 ms against 1.06 */
+__host__ __device__ constexpr int screen_threads_per_sm(int K, int NV) { return K == 6 && NV > 3 ? 1024 : 768; }
 /* statistics kernels: 3 CTAs of 128 threads, 168 registers */
 constexpr int FACE_CTAS_PER_SM_STATS = 3;
 

@@ -154,6 +154,13 @@ __device__ __forceinline__ void stage_screen_differences(float* sf, int NP, int 
   }
 }
 
+/* Shared-memory values read again after this point are loaded again: the compiler otherwise keeps
+   the tile values of a face's several passes (30-60 of them) in spilled registers, and the local
+   memory of 768 threads does not fit L1 beside the tile (2D TENO8 328 -> 108 bytes a thread at 80
+   registers, TENO6 128 -> 8; 2048^2 step 6.45 -> 5.98 ms and 5.44 -> 5.17 ms with the
+   differences of both sides formed together).  Not in 1D, where few threads wait on latency. */
+__device__ __forceinline__ void keep_loads_here() { asm volatile("" ::: "memory"); }
+
 /* Fields of one face that are NOT certified central (bit s); the face's stencil point q is
    tile point p0 + q * LANES.
 
@@ -257,6 +264,7 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
   const float kh = rh * fmaf(gh * (2.f * ct + gh), i2, hb1 * w2h);
   const float dcan = 120.f * u * fmaf(Tv, ic, Mn + Mc);
 
+  if constexpr (NV > 3) keep_loads_here();
   /* differences shared by the acoustic pair and the entropy field */
   float e[K - 1], m[K - 1], Q[K - 1], kn[K - 1];
   float mxm = -1e30f, mnm = 1e30f, mxp = -1e30f, mnp = 1e30f, mx0 = -1e30f, mn0 = 1e30f;
@@ -318,6 +326,7 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
     }
   }
 
+  if constexpr (NV > 3) keep_loads_here();
   unsigned bad = 0u;
   float off[2], del[2];  /* side f+, f-: off+- = lambda~ +- alpha and the bound of its error */
   auto offsets = [&](float lam, float lerr, float hi, float lo) {
@@ -328,23 +337,20 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
     del[0] = dcan + (neg ? 0.f : lerr);
     del[1] = dcan + (pos ? 0.f : lerr);
   };
-  float d[K - 1];
-  auto test = [&](const float (&dw)[K - 1], const float (&R)[K - 1], float MW, float Y) -> bool {
-    bool ok = true;
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      float lm = 0.f;
-#pragma unroll
-      for (int t = 0; t < K - 1; ++t) {
-        const int q = side ? K - 2 - t : t;  /* f-: the mirrored stencil (the forms are even in d) */
-        const float lam = wn[q + 1] + off[side];
-        lm = fmaxf(lm, fabsf(lam));
-        d[t] = fmaf(lam, dw[q], R[q]);
-      }
-      const float E = fmaf(fmaf(60.f * u * th, lm, del[side]), MW, 80.f * u * th * Y);
-      ok = ok && quick_smooth<K>(d, E, S, need_ex);
-    }
-    return ok;
+  /* differences of f+ and of f- on its mirrored stencil (the forms are even in d), formed together
+     so that the projections' terms are not kept over the two tests */
+  float dp[K - 1], dn[K - 1], lm[2];
+  auto diff = [&](int t, float dw, float R) {
+    const float l0 = wn[t + 1] + off[0], l1 = wn[t + 1] + off[1];
+    lm[0] = fmaxf(lm[0], fabsf(l0));
+    lm[1] = fmaxf(lm[1], fabsf(l1));
+    dp[t] = fmaf(l0, dw, R);
+    dn[K - 2 - t] = fmaf(l1, dw, R);
+  };
+  auto test = [&](float MW, float Y) -> bool {
+    const float u80 = 80.f * u * th, u60 = 60.f * u * th;
+    const bool ok = quick_smooth<K>(dp, fmaf(fmaf(u60, lm[0], del[0]), MW, u80 * Y), S, need_ex);
+    return quick_smooth<K>(dn, fmaf(fmaf(u60, lm[1], del[1]), MW, u80 * Y), S, need_ex) && ok;
   };
   {
     const float lerr = 20.f * u * th * (fabsf(un) + ct);
@@ -354,26 +360,24 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
     for (int i = 0; i < 2; ++i) {
       const float sg = i ? 1.f : -1.f;
       offsets(fmaf(sg, ct, un), lerr, i ? mxp : mxm, i ? mnp : mnm);
-      float dw[K - 1], R[K - 1];
+      if constexpr (NV > 3) keep_loads_here();
+      lm[0] = lm[1] = 0.f;
 #pragma unroll
-      for (int t = 0; t < K - 1; ++t) {
-        dw[t] = fmaf(sg, m[t], e[t]);
-        R[t] = fmaf(sg, Q[t], fmaf(-wn[t + 1], fmaf(-b1, dif(L::P, t), dif(L::R, t)), kn[t]));
-      }
-      bad |= test(dw, R, MW, Y) ? 0u : (i ? 1u << (NV - 1) : 1u);
+      for (int t = 0; t < K - 1; ++t)
+        diff(t, fmaf(sg, m[t], e[t]), fmaf(sg, Q[t], fmaf(-wn[t + 1], fmaf(-b1, dif(L::P, t), dif(L::R, t)), kn[t])));
+      bad |= test(MW, Y) ? 0u : (i ? 1u << (NV - 1) : 1u);
     }
   }
   /* entropy and shear fields: speed u_n */
   offsets(un, 10.f * u * fmaf(4.f, Mn, fabsf(un)), mx0, mn0);
 #pragma unroll 1
   for (int s = 1; s <= NV - 2; ++s) {
-    float dw[K - 1], R[K - 1], MW, Y;
+    float MW, Y;
+    if constexpr (NV > 3) keep_loads_here();
+    lm[0] = lm[1] = 0.f;
     if (s == 1) {
 #pragma unroll
-      for (int t = 0; t < K - 1; ++t) {
-        dw[t] = dif(L::R, t) - e[t];
-        R[t] = -fmaf(b1 * wn[t + 1], dif(L::P, t), kn[t]);
-      }
+      for (int t = 0; t < K - 1; ++t) diff(t, dif(L::R, t) - e[t], -fmaf(b1 * wn[t + 1], dif(L::P, t), kn[t]));
       MW = Mr + Me;
       Y = fmaf(kh, Mn, b1 * whn * Mp);
     } else {
@@ -386,8 +390,7 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
 #pragma unroll
       for (int t = H - 2; t >= 0; --t) {
         const float dvt = sd[t * LANES], w0 = w1 - dvt, r0 = val(L::R, t);
-        dw[t] = fmaf(w1, dif(L::R, t), r0 * dvt);
-        R[t] = r0 * w0 * dif(L::V + AXIS, t);
+        diff(t, fmaf(w1, dif(L::R, t), r0 * dvt), r0 * w0 * dif(L::V + AXIS, t));
         w1 = w0;
       }
       float w0 = -wr * sd[(H - 1) * LANES];
@@ -395,15 +398,14 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
       for (int t = H - 1; t < K - 1; ++t) {
         const float dvt = sd[t * LANES], r0 = val(L::R, t);
         w1 = (t == H - 1) ? wl * dvt : w0 + dvt;
-        dw[t] = fmaf(w1, dif(L::R, t), r0 * dvt);
-        R[t] = r0 * w0 * dif(L::V + AXIS, t);
+        diff(t, fmaf(w1, dif(L::R, t), r0 * dvt), r0 * w0 * dif(L::V + AXIS, t));
         w0 = w1;
       }
       const float wht = (float)H * Mt;
       MW = fmaf(wht, Mr, rh * Mt);
       Y = rh * wht * Mn;
     }
-    bad |= ((still >> s & 1u) || test(dw, R, MW, Y)) ? 0u : 1u << s;
+    bad |= ((still >> s & 1u) || test(MW, Y)) ? 0u : 1u << s;
   }
   return bad;
 }
@@ -448,7 +450,7 @@ constexpr size_t screen_smem() {
    nonlinear_kernel): sigma_q = c_q, delta_q = 0, omegaW = -0 (kCentralMark), fs = l_s . Fc. */
 template <int NV, int K, int AXIS, bool REC>
 __global__ void __launch_bounds__(FaceTile<NV, K, AXIS, true>::THREADS,
-                                  SCREEN_THREADS_PER_SM / FaceTile<NV, K, AXIS, true>::THREADS)
+                                  screen_threads_per_sm(K, NV) / FaceTile<NV, K, AXIS, true>::THREADS)
 screen_kernel(const FaceArgs A) {
   using T = FaceTile<NV, K, AXIS, true>;
   using L = ScreenLayout<NV>;
@@ -525,9 +527,13 @@ screen_kernel(const FaceArgs A) {
   const long long flin = face_index(f);
   unsigned bad = 0u;
   if (active) {
+    const int p0 = jf * T::LANES + lane;
+    constexpr unsigned allf = (1u << NV) - 1u;
+    const bool adaptive = A.sch.ct_mode == CT_ADAPTIVE;
+    bad = A.sch.screen ? screen_face<NV, K, AXIS, T::LANES>(sf, NP, p0, (float)(A.gamma - 1.0), A.sch, A.flags && adaptive)
+                       : allf;
     double cw[K], Fc[NV];
     central_weights<K>(cw);
-    const int p0 = jf * T::LANES + lane;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const double* s = sF + v * NP + p0;
@@ -542,10 +548,6 @@ screen_kernel(const FaceArgs A) {
 #pragma unroll
       for (int v = 0; v < NV; ++v) A.Fhat[v * A.nface + fn] = Fc[v];
     }
-    constexpr unsigned allf = (1u << NV) - 1u;
-    const bool adaptive = A.sch.ct_mode == CT_ADAPTIVE;
-    bad = A.sch.screen ? screen_face<NV, K, AXIS, T::LANES>(sf, NP, p0, (float)(A.gamma - 1.0), A.sch, A.flags && adaptive)
-                       : allf;
     if (A.flags) {  /* the certified fields' bytes: every candidate smooth, [beta] = 10 */
       const unsigned allk = ((1u << (K - 2)) - 1u) | (adaptive ? 3u << 6 : 0u);
       for (int r = 0; r < ((wrapped && f == 0) ? 2 : 1); ++r) {
