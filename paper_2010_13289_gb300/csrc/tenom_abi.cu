@@ -572,7 +572,9 @@ tenom_status tenom_create(tenom_ctx** out, const tenom_grid* grid, const tenom_s
     return at;
   };
   const size_t small = part(256);  /* status, list lengths, CFL maximum, dt, t */
-  const size_t w1 = part(sizeof(double) * c->nv * c->ncell), prims = part(sizeof(double) * (c->nv + 2) * c->ncell);
+  size_t stage = sizeof(double) * c->nv * c->ncell, flags = 0;  /* tenom_rhs_vjp keeps its flags in the stage buffer */
+  for (int a = 0; a < grid->dim; ++a) flags += (size_t)c->nface[a] * c->nv * 2;
+  const size_t w1 = part(stage > flags ? stage : flags), prims = part(sizeof(double) * (c->nv + 2) * c->ncell);
   size_t face[3], list[3];
   for (int a = 0; a < grid->dim; ++a) {
     face[a] = part(sizeof(double) * c->nv * c->nface[a]);
@@ -1089,14 +1091,10 @@ static cudaError_t adj_sweeps(tenom_ctx* c, const double* U, const uint8_t* flag
   return e;
 }
 
-/* room for three stages' cutoff flags */
-static cudaError_t ensure_flags(tenom_ctx* c) {
-  return c->adj_flags ? cudaSuccess : cudaMalloc(&c->adj_flags, tenom_flags_bytes(c) * 3);
-}
-
 static cudaError_t ensure_adj(tenom_ctx* c) {
   cudaError_t e = c->adj ? cudaSuccess : cudaMalloc(&c->adj, sizeof(double) * c->nv * c->ncell * 7);
-  return e == cudaSuccess ? ensure_flags(c) : e;
+  if (e == cudaSuccess && !c->adj_flags) e = cudaMalloc(&c->adj_flags, tenom_flags_bytes(c) * 3);
+  return e;
 }
 
 static cudaError_t lincomb(tenom_ctx* c, double* out, double c0, const double* x0, double c1, const double* x1,
@@ -1111,13 +1109,14 @@ tenom_status tenom_rhs_vjp(tenom_ctx* c, const double* U, const double* w, doubl
   if (adjoint_unsupported(c, "rhs_vjp")) return TENOM_E_UNSUPPORTED;
   if (!aligned8(U) || !aligned8(w) || !aligned8(Ubar) || Ubar == U || Ubar == w)
     return fail(c, TENOM_E_INVALID, "rhs_vjp: bad pointers");
-  /* the branches at U: one forward pass over the faces with flags */
-  cudaError_t e = ensure_flags(c);
+  /* the branches at U: one forward pass over the faces with flags, in the stage buffer (no
+     allocation, so that the call can be captured) */
+  uint8_t* const flags = reinterpret_cast<uint8_t*>(c->W1);
   uint8_t* fl[3] = {nullptr, nullptr, nullptr};
-  for (int a = 0; a < c->g.dim && e == cudaSuccess; ++a) fl[a] = c->adj_flags + flags_offset(c, a);
-  if (e == cudaSuccess) e = launch_prims(c, U);
+  for (int a = 0; a < c->g.dim; ++a) fl[a] = flags + flags_offset(c, a);
+  cudaError_t e = launch_prims(c, U);
   if (e == cudaSuccess) e = launch_faces(c, U, 0, c->g.dim, c->face, fl, nullptr);
-  if (e == cudaSuccess) e = adj_sweeps(c, U, c->adj_flags, nullptr, w, Ubar);
+  if (e == cudaSuccess) e = adj_sweeps(c, U, flags, nullptr, w, Ubar);
   return e == cudaSuccess ? TENOM_OK : cuda_fail(c, e, "rhs_vjp");
 }
 
