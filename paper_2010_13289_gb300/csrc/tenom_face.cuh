@@ -149,16 +149,13 @@ __device__ __forceinline__ void stage_point(const double (&u)[NV], double gamma,
   stage_point_from<NV, AXIS>(u, vel, pr, Hh, c, sr, sm, NP, p);
 }
 
-/* Flux at the face whose K stencil points are shared-memory points (jf + q) * LANES + lane,
-   q = 0..K-1, of a tile laid out by PointLayout<NV> with NP points per component:
-   Roe average of points K/2-1 and K/2, characteristic projection, LLF split, TENO-M per
-   field and side (each lane its own), back-projection.  flags (may be null) receives NV x 2
-   bytes.  The batched stage kernel's face flux; STATS: the decision statistics of both
-   sides of every field into cnt (SC_COUNT counters) instead of the flux. */
-template <int NV, int K, int LIM, int AXIS, int LANES, bool STATS = false>
-__device__ __forceinline__ void face_flux_smem(const double* sm, int NP, int jf, int lane, double gamma,
-                                               const SchemeDev& sch, double (&Fh)[NV], uint8_t* flags, int& st,
-                                               unsigned* cnt = nullptr) {
+/* Decision statistics of the face whose K stencil points are shared-memory points
+   (jf + q) * LANES + lane, q = 0..K-1, of a tile laid out by PointLayout<NV> with NP points per
+   component: Roe average of points K/2-1 and K/2, characteristic projection, LLF split, both sides
+   of every field counted into cnt. */
+template <int NV, int K, int LIM, int AXIS, int LANES>
+__device__ __forceinline__ void face_stats(const double* sm, int NP, int jf, int lane, double gamma,
+                                           const SchemeDev& sch, unsigned (&cnt)[SC_COUNT], int& st) {
   using L = PointLayout<NV>;
   constexpr int D = NV - 2;
   constexpr int H = K / 2;
@@ -178,7 +175,6 @@ __device__ __forceinline__ void face_flux_smem(const double* sm, int NP, int jf,
   const double c2 = (gamma - 1.0) * (Ht - 0.5 * q2);
   if (!ipos(c2)) st |= ST_ROE;
   const double cinv = rsqrt_nr(c2);
-  const double ct = c2 * cinv;
   const double b1 = (gamma - 1.0) * (cinv * cinv);
   const double b2 = 0.5 * q2 * b1;
   const double una = ut[AXIS];
@@ -191,31 +187,6 @@ __device__ __forceinline__ void face_flux_smem(const double* sm, int NP, int jf,
     a_p = imax_nonneg(a_p, P(L::cLp, q));
   }
 
-#pragma unroll
-  for (int v = 0; v < NV; ++v) Fh[v] = 0.0;
-  /* back-projection F += r_s fs (right eigenvector of field s) */
-  auto backproj = [&](int s, double fs) {
-    if ((s == 0) || (s == NV - 1)) {
-      const double sr = (s == 0) ? -1.0 : 1.0;         /* r: -c for u-c, +c for u+c */
-      Fh[0] += fs;
-#pragma unroll
-      for (int d = 0; d < D; ++d) Fh[1 + d] += (ut[d] + (d == AXIS ? sr * ct : 0.0)) * fs;
-      Fh[NV - 1] += (Ht + sr * una * ct) * fs;
-    } else if (s == 1) {
-      Fh[0] += fs;
-#pragma unroll
-      for (int d = 0; d < D; ++d) Fh[1 + d] += ut[d] * fs;
-      Fh[NV - 1] += 0.5 * q2 * fs;
-    } else {
-      const int dt = (s - 2) < AXIS ? (s - 2) : (s - 1);
-#pragma unroll
-      for (int d = 0; d < D; ++d)
-        if (d == dt) {
-          Fh[1 + d] += fs;
-          Fh[NV - 1] += ut[d] * fs;
-        }
-    }
-  };
   /* The acoustic pair and the entropy field share the vectors a = (b2, -b1 u, b1) and
      b = (u_n / c, -e_n / c, 0): l_{u-+c} = (a +- b)/2, l_0 = e_0 - a.  Per stencil point
      A = a.U/2, B = b.U/2, AF = a.F/4, BF = b.F/4 once, then W_{u-+c} = A +- B,
@@ -303,19 +274,8 @@ __device__ __forceinline__ void face_flux_smem(const double* sm, int NP, int jf,
     double vm[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) vm[q] = gm[K - 1 - q];
-    if constexpr (STATS) {  /* statistics of both sides' decisions instead of the flux */
-      side_stats<K, LIM>(gp, sch, *reinterpret_cast<unsigned(*)[SC_COUNT]>(cnt));
-      side_stats<K, LIM>(vm, sch, *reinterpret_cast<unsigned(*)[SC_COUNT]>(cnt));
-      continue;
-    }
-    unsigned flp, flm;
-    const double fplus = teno_m<K, LIM>(gp, sch, flp, st);
-    const double fminus = teno_m<K, LIM>(vm, sch, flm, st);
-    if (flags) {
-      flags[s * 2 + 0] = (uint8_t)flp;
-      flags[s * 2 + 1] = (uint8_t)flm;
-    }
-    backproj(s, fplus + fminus);
+    side_stats<K, LIM>(gp, sch, cnt);
+    side_stats<K, LIM>(vm, sch, cnt);
   }
 }
 
@@ -370,8 +330,7 @@ stats_kernel(const FaceArgs A) {
 #pragma unroll
   for (int q = 0; q < SC_COUNT; ++q) cnt[q] = 0u;
   if (f0 + jf <= na && (AXIS == 0 || x0 + lane < A.n[0])) {
-    double Fh[NV];
-    face_flux_smem<NV, K, LIM, AXIS, T::LANES, true>(sm, T::NP, jf, lane, A.gamma, A.sch, Fh, nullptr, st, cnt);
+    face_stats<NV, K, LIM, AXIS, T::LANES>(sm, T::NP, jf, lane, A.gamma, A.sch, cnt, st);
   }
   /* warp sums, one 64-bit atomic per counter and warp */
 #pragma unroll

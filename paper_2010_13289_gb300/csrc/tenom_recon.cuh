@@ -678,16 +678,4 @@ __device__ __forceinline__ double teno_general(const double (&v)[K], const Schem
   return f;
 }
 
-/* One TENO-M reconstruction: decisions (certified FP32 filter, FP64 where it cannot decide)
-   then teno_general.  flag receives delta bits | ([beta]-7) << 6. */
-template <int K, int LIM, bool WT = false>
-__device__ __forceinline__ double teno_m(const double (&v)[K], const SchemeDev& S, unsigned& flag, int& st,
-                                         double* om = nullptr) {
-  unsigned bits = 0;
-  int ex = 7;
-  if (!teno_decide_fast<K>(v, S, bits, ex)) teno_decide_fp64<K>(v, S, bits, ex, st);
-  flag = bits | ((unsigned)((ex - 7) & 3) << 6);
-  return teno_general<K, LIM, WT>(v, S, bits, om);
-}
-
 }  // namespace tenom

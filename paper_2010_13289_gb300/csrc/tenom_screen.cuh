@@ -15,12 +15,13 @@
  * The FP64 pipe of GB300 runs at 1/64 of the FP32 rate, so a face that is certified costs the
  * K nvar FMAs of Fc and a share of its points' fluxes; everything the certificate needs --
  * Roe average, differences, projections, indicators -- runs in FP32 and on the integer pipe
- * with rigorous error bounds.  What bounds it (ncu, 2D 1024^2 TENO8): FP64 pipe 50 % and issue
- * 56 % busy, 0.15 ms for 1.05 M faces (20 FP64 pipe cycles a face, 95 instructions issued per
+ * with rigorous error bounds.  What bounds it (ncu, 2D 1024^2 TENO8): FP64 pipe 57 % and issue
+ * 65 % busy, 0.124 ms for 1.05 M faces (16 FP64 pipe cycles a face, 93 instructions issued per
  * warp and face).  The single kernel this pair replaced formed Roe state, eigenvectors and the
  * composition in FP64 for every warp that held an uncertified face and waited for its own
  * queue at CTA barriers: 1024^2 TENO8 sweeps 0.72 ms against 0.43 ms for the pair, one step of
- * 2048^2 TENO8-TVD5 17.8 -> 7.0 ms, TENO6-MP 13.2 -> 6.3, 256^3 TENO8-MP 133 -> 77. */
+ * 2048^2 TENO8-TVD5 17.8 -> 5.6 ms, TENO6-MP 13.2 -> 5.1, 256^3 TENO8-MP 133 -> 53 with the
+ * nonlinear kernel's later forms. */
 #pragma once
 #include "tenom_recon.cuh"
 #include "tenom_face.cuh"
