@@ -271,6 +271,8 @@ tenom_status tenom_rk3_step_adjoint_tape(tenom_ctx* ctx, const double* U_n, cons
  *   fs = f+ + f- = sum_q sigma_q G_q + (alpha_s / 2) delta_q W_q,
  *   sigma_q = (op_q + om_{K-1-q}) / 2,  delta_q = op_q - om_{K-1-q},
  * the record is (fs, omegaW = sum_q delta_q W_q, sigma_0..K-1, delta_0..K-1): 2K + 2 doubles.
+ * A central field (every candidate of both sides smooth, maximal-order d_k: sigma_q = the K-point
+ * central weights, delta_q = 0) is marked by omegaW = -0.0; the reverse skips its row.
  * Layout of one stage: axis after axis; inside axis a, [nvar][2K+2][nface_a] doubles
  * (face order as the face buffers of tenom_face_dump). */
 
