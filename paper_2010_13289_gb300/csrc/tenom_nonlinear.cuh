@@ -288,52 +288,54 @@ __device__ __forceinline__ void compose(const double* face, const double* fsv, u
 
 /* The rare FP64 paths of the fixed-point kernel, called rather than inlined: they are larger
    than the path every item takes, and instruction fetch is what that path waits for.  w, g: the
-   item's W and G/2 of point q at q * NL_THREADS; side 1: the mirrored stencil of f-. */
+   item's W and G of point q at q * NL_THREADS; side 1: the mirrored stencil of f-.  The item keeps
+   twice the split sequences (G +- alpha W), which saves a product per point (256^3 TENO8: FP64
+   pipe 74 % busy); halving is exact. */
 template <int K>
-__device__ __forceinline__ void split_side(const double* w, const double* g, double ha, int side, double (&v)[K]) {
+__device__ __forceinline__ void split_side(const double* w, const double* g, double al, int side, double (&v)[K]) {
 #pragma unroll
   for (int q = 0; q < K; ++q) {
     const int p = (side ? K - 1 - q : q) * NL_THREADS;
-    v[q] = fma(side ? -ha : ha, w[p], g[p]);
+    v[q] = 0.5 * fma(side ? -al : al, w[p], g[p]);
   }
 }
 template <int K>
-__device__ __noinline__ unsigned decide_cold(const double* w, const double* g, double ha, int side, const SchemeDev& S,
+__device__ __noinline__ unsigned decide_cold(const double* w, const double* g, double al, int side, const SchemeDev& S,
                                              int& st) {
   double v[K];
-  split_side<K>(w, g, ha, side, v);
+  split_side<K>(w, g, al, side, v);
   unsigned b;
   int e;
   teno_decide_fp64<K>(v, S, b, e, st);
   return b | ((unsigned)((e - 7) & 3) << 6);
 }
 template <int K, int LIM>
-__device__ __noinline__ double general_cold(const double* w, const double* g, double ha, unsigned fl, const SchemeDev& S) {
+__device__ __noinline__ double general_cold(const double* w, const double* g, double al, unsigned fl, const SchemeDev& S) {
   constexpr unsigned allk = (1u << (K - 2)) - 1u;
   double f = 0.0;
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
     double v[K];
-    split_side<K>(w, g, ha, side, v);
+    split_side<K>(w, g, al, side, v);
     f += teno_general<K, LIM>(v, S, fl >> (8 * side) & allk);
   }
   return f;
 }
 
-/* Both split sides of an item from its projected W and G/2 (columns w, g in shared memory):
+/* Both split sides of an item from its projected W and G (columns w, g in shared memory):
    decisions, and the corrections of the nonsmooth sides in fixed point.  Returns false when the
    FP32 filter leaves a side undecided and `defer` is set.  Dx: K - 1 scratch words of the item's
-   thread.  em: biased exponent of a power of two above every |G/2| + |alpha W/2|.  The loops over
+   thread.  em: biased exponent of a power of two above every |G| + |alpha W|.  The loops over
    the points are rolled and everything rare is called, to keep the code that an item runs
    small (unrolled 4 or 8 times: 256^3 step 64 ms against 59, 64^3 turbulence 5.6 against 5.1). */
 template <int K, int LIM>
-__device__ __forceinline__ bool fixed_item(const double* w, const double* g, double ha, int em, long long* Dx,
+__device__ __forceinline__ bool fixed_item(const double* w, const double* g, double al, int em, long long* Dx,
                                            const SchemeDev& S, bool defer, unsigned& fl, double& fsum, bool& direct,
                                            int& st) {
   constexpr int c = K / 2 - 1, TH = NL_THREADS;
   constexpr unsigned allk = (1u << (K - 2)) - 1u;
-  const bool inside = em >= 1023 - 40 && em <= 1023 + 40;
-  const float unit = __int_as_float((inside ? em - 1076 + 127 : 0) << 23);  /* 2^(em - 1076) */
+  const bool inside = em >= 1024 - 40 && em <= 1024 + 40;
+  const float unit = __int_as_float((inside ? em - 1077 + 127 : 0) << 23);  /* 2^(em - 1077): of the halved values */
   Acc96 acc;
   fl = 0u;
   direct = false;
@@ -344,7 +346,7 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
     auto expo = [](double x) -> int { return (int)((unsigned)__double2hiint(x) >> 20 & 0x7ffu); };
     {
       const int p0 = side ? (K - 1) * TH : 0, dp = side ? -TH : TH;
-      const double hs = side ? -ha : ha;
+      const double hs = side ? -al : al;
       double v0 = fma(hs, w[p0], g[p0]);
       long long x0 = to_fixed(v0, em);
       es = expo(v0);
@@ -368,7 +370,7 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
     int e = 7;
     if (S.exact_decisions || !inside || !cutoff_filter<K>(d, 1.01f * unit, zero, S, b, e)) {
       if (defer) return false;
-      const unsigned f = decide_cold<K>(w, g, ha, side, S, st);
+      const unsigned f = decide_cold<K>(w, g, al, side, S, st);
       b = f & allk;
       e = 7 + (int)(f >> 6);
     }
@@ -384,8 +386,8 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
       }
     }
   }
-  fsum = direct ? general_cold<K, LIM>(w, g, ha, fl, S)
-                : acc.value() * (__hiloint2double((em - 1076 + 1023) << 20, 0) * (1.0 / fixed_den<K, LIM>()));
+  fsum = direct ? general_cold<K, LIM>(w, g, al, fl, S)
+                : acc.value() * (__hiloint2double((em - 1077 + 1023) << 20, 0) * (1.0 / fixed_den<K, LIM>()));
   return true;
 }
 
@@ -402,7 +404,7 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
   __shared__ unsigned s_dir[TH];            /* fields whose s_fs is f+ + f- (else the correction to l_s . Fc) */
   __shared__ unsigned short s_item[NV * TH];
   __shared__ unsigned short s_later[FIX ? NV * TH : 1];
-  __shared__ double s_w[FIX ? K * TH : 1], s_g[FIX ? K * TH : 1];  /* an item's W and G/2 */
+  __shared__ double s_w[FIX ? K * TH : 1], s_g[FIX ? K * TH : 1];  /* an item's W and G */
   __shared__ long long s_D[FIX ? (K - 1) * TH : 1];
   __shared__ int s_nlater;
   __shared__ int s_wc[NV * W + 1];
@@ -525,19 +527,20 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       const double* const ut = A.U + gc(shear ? s : 1) * A.ncell;
       const long long base = s_base[fc];
       const int f = s_f[fc];
-      /* W and G/2 of stencil point q, G = l . F = u_n W + p (l_n + u_n l_E) */
+      /* W and G/2 (FIX: G) of stencil point q, G = l . F = u_n W + p (l_n + u_n l_E) */
       auto project = [&](int q, double& w, double& hg) {
         const long long cell = base + sa * bc_near(f - H + q, na, bc);
         const double un = __ldg(Pn + cell);
         if (shear) {
           w = fma(l[0], __ldg(up[0] + cell), __ldg(ut + cell));
-          hg = 0.5 * un * w;
+          hg = un * w;
         } else {
           w = l[0] * __ldg(up[0] + cell);
 #pragma unroll
           for (int v = 1; v < NV; ++v) w = fma(l[v], __ldg(up[v] + cell), w);
-          hg = 0.5 * fma(__ldg(Pp + cell), fma(un, l[NV - 1], l[1]), un * w);
+          hg = fma(__ldg(Pp + cell), fma(un, l[NV - 1], l[1]), un * w);
         }
+        if constexpr (!FIX) hg *= 0.5;
       };
       unsigned fl = 0u;
       double fsum = 0.0;
@@ -554,9 +557,10 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
           eg = max(eg, (int)((unsigned)__double2hiint(hg) >> 20 & 0x7ffu));
           ew = max(ew, (int)((unsigned)__double2hiint(w) >> 20 & 0x7ffu));
         }
-        /* |v| <= |G/2| + |alpha W/2| < 2^(em - 1022) */
-        const int em = 1 + max(eg, ew + (int)((unsigned)__double2hiint(ha) >> 20 & 0x7ffu) - 1022);
-        if (!fixed_item<K, LIM>(s_w + tid, s_g + tid, ha, em, s_D + tid, A.sch, pass == 0 && nitem > TH, fl, fsum,
+        /* 2 |v| <= |G| + |alpha W| < 2^(em - 1022) */
+        const double al = ha + ha;
+        const int em = 1 + max(eg, ew + (int)((unsigned)__double2hiint(al) >> 20 & 0x7ffu) - 1022);
+        if (!fixed_item<K, LIM>(s_w + tid, s_g + tid, al, em, s_D + tid, A.sch, pass == 0 && nitem > TH, fl, fsum,
                                 direct, st)) {
           s_later[atomicAdd(&s_nlater, 1)] = (unsigned short)item;
           continue;
