@@ -52,7 +52,7 @@ ADJOINT_DEFAULT = "adjoint_broadband_2d_512_teno6_mp"
 FP64_LANES_PER_CLK = 304  # FP64 pipe: 2 lanes per clock per SM x 152 SMs
 
 
-FACE_SOURCES = ("tenom_screen.cuh", "tenom_nonlinear.cuh", "tenom_face.cuh", "tenom_recon.cuh", "teno_coeffs.cuh",
+FACE_SOURCES = ("tenom_screen.cuh", "tenom_nonlinear.cuh", "tenom_fixed.cuh", "tenom_face.cuh", "tenom_recon.cuh", "teno_coeffs.cuh",
                 "tenom_fastmath.cuh", "tenom_launch.cuh", "tenom_internal.h")
 
 
@@ -69,7 +69,7 @@ def face_source_hash(sources=FACE_SOURCES):
     return h.hexdigest()[:16]
 
 
-def profile_figures(name, kernel="face_kernel", sources=FACE_SOURCES):
+def profile_figures(name, kernel="face_sweeps", sources=FACE_SOURCES):
     """ncu figures of a kernel committed for this workload (profiles/<kernel>_<name>.md), or
     None when there are none or they were taken from other kernel sources than the ones
     built now."""
