@@ -3,13 +3,13 @@
  * With the cutoff decisions taken, fhat = sum_k d_k f_k + sum_{k nonsmooth} d_k (limited_k - f_k);
  * the first sum is the central scheme, and the correction depends only on the differences of
  * the sequence: every term is a combination with rational coefficients, a minimum or a
- * maximum.  On integers v_q = trunc(value / unit), unit = 2^-54 of a power of two above the
+ * maximum.  On integers v_q = floor(value / unit), unit = 2^-54 of a power of two above the
  * largest |v_q|, those are exact (a few floor divisions lose one unit each), so the correction
  * carries the rounding of FP64 values of the sequence's size, and runs on the integer pipe:
  * about 250 instructions a side where the FP64 form has 50-80 operations of 64 issue slots
  * each on GB300's FP64 pipe, paid by the whole warp when one lane needs them.
  *
- * Overflow: |v| < 2^54, differences < 2^55, second differences < 2^56, 4 d - d' < 5 2^56,
+ * Overflow: |v| <= 2^54, differences <= 2^55, second differences < 2^56, 4 d - d' < 5 2^56,
  * candidates and bounds (alpha, beta/3 <= 8, scheme's fixed flag) < 2^60; the TVD5 terms in 60ths
  * < 94 2^55 + 60 2^55 < 2^62.3. */
 #pragma once
@@ -17,13 +17,15 @@
 
 namespace tenom {
 
-/* trunc(v 2^(1076 - em)) for a finite v with biased exponent at most em: |result| < 2^54 */
+/* floor(v 2^(1076 - em)) for a finite v with biased exponent at most em: |result| <= 2^54.  Floored and
+   not truncated, so that a difference of two results is within one unit of the exact one whatever
+   their signs: the filter is given that bound.  (Subnormal v: 0.) */
 __device__ __forceinline__ long long to_fixed(double v, int em) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
   const int e = (int)((hi >> 20) & 0x7ffu), sh = em - e;
-  unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 1;
-  m = (e == 0 || sh > 63) ? 0ull : m >> sh;
-  return (int)hi < 0 ? -(long long)m : (long long)m;
+  long long m = (long long)((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 1;
+  m = (int)hi < 0 ? -m : m;
+  return e == 0 ? 0 : m >> (sh < 63 ? sh : 63);
 }
 
 /* D q 2^-60 for a coefficient q = coef 2^60 (coef <= 8 exclusive), |D| < 2^58 */
