@@ -364,18 +364,22 @@ __device__ __forceinline__ bool cutoff_filter(const float (&d)[K - 1], float E, 
   float CTf = S.ct_const_f;
   ex = 7;
   if (S.ct_mode == CT_ADAPTIVE) {
-    /* E moves eta by at most 8 E / max(|d|, sqrt(eps) = 5e-4) and beta by 32 times that: below the
-       1e-4 margin (FP32 rounding: 32 x 12 u) for E <= 1e-10 */
-    if (!(E <= 1e-10f)) return false;
+    /* E moves an eta by at most 8 E / s, s = max(|a|, |b|, sqrt(eps) = 5e-4) of its two differences, and
+       beta by 32 times that: with E <= 2e-7 s 5.2e-5, below the 1e-4 margin with the FP32 rounding
+       (32 x 12 u).  The bound goes with the differences, not with 5e-4 alone: E is relative to the
+       values, and in large units (shear fluxes of 1e6) an absolute limit refused every side */
     const float xi = 1e-3f, Cr = 0.23f, a1 = 10.5f, a2 = 3.5f;
     const float eps = 0.9f * Cr / (1.f - 0.9f * Cr) * xi * xi;
-    float eh = 0.f;
+    float eh = 0.f, sm = 0.f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float dfp = d[c + q - 1], dfm = d[c + q - 2];
       const float eta = __fdividef(fabsf(2.f * dfp * dfm) + eps, dfp * dfp + dfm * dfm + eps);
+      const float s = fmaxf(fabsf(dfp), fabsf(dfm));
       eh = (q == 0) ? eta : fminf(eh, eta);
+      sm = (q == 0) ? s : fminf(sm, s);
     }
+    if (!(E <= 2e-7f * fmaxf(sm, 5e-4f))) return false;
     const float m = 1.f - fminf(1.f, eh * (1.f / Cr));
     const float om = 1.f - m;
     const float g = om * om * om * om * (1.f + 4.f * m);

@@ -155,6 +155,36 @@ static int run() {
       v[left ? 0 : K - 1] = left ? -0.999 : 0.999;
       bad += item<K>(v, S, false, und, dec);
     }
+    /* waves of any size: what is decided at size 1 is decided at every size */
+    for (int i = 0; i < 100000 && !bad; ++i) {
+      double v[K];
+      const double s = std::ldexp(1.0, (int)uni(-8, 36)), ph = uni(0, 6.3), k = uni(0.05, 1.5), off = uni(-2, 2);
+      for (int q = 0; q < K; ++q) v[q] = s * (off + std::sin(ph + k * q) + (q > K / 2 && i % 3 == 0 ? 1.0 : 0.0));
+      double least = 1e300;
+      for (int t = 0; t + 1 < K; ++t) least = std::fmin(least, std::fabs(v[t + 1] - v[t]));
+      bad += item<K>(v, S, least > 1e-3 * s, und, dec);
+    }
+    /* a bound E near the largest for which eta is certain: [beta] holds for every sequence within it */
+    for (int i = 0; i < 200000 && !bad && mode == CT_ADAPTIVE; ++i) {
+      float d[K - 1];
+      const double s = std::ldexp(1.0, (int)uni(-12, 30));
+      const float E = (float)(std::fmax(s * 0.05, 5e-4) * std::exp(uni(std::log(1e-9), std::log(1e-5))));
+      for (int t = 0; t < K - 1; ++t) d[t] = (float)(s * uni(0.02, 1.0) * (uni(0, 1) < 0.3 ? -1 : 1));
+      unsigned b;
+      int e;
+      if (!cutoff_filter<K>(d, E, 0u, S, b, e)) continue;
+      for (int r = 0; r < 8 && !bad; ++r) {
+        real D[K - 1], margin;
+        unsigned rb;
+        int re;
+        for (int t = 0; t < K - 1; ++t) D[t] = (real)d[t] + (real)E * (uni(0, 1) < 0.5 ? -1 : 1);
+        decide<K>(D, S, rb, re, margin);
+        if (rb != b || re != e) {
+          std::printf("K %d E %g s %g: decided %x [%d], within E %x [%d]\n", K, E, s, b, e, rb, re);
+          ++bad;
+        }
+      }
+    }
   }
   std::printf("K %d: %d decided, %d undecided\n", K, dec, und);
   return bad;
