@@ -17,10 +17,9 @@
  * FIX: a nonsmooth side only adds its limiter's correction sum_k d_k (limited_k - f_k), in fixed
  * point (tenom_fixed.cuh), and the face flux is Fc + sum_s r_s correction_s (the smooth part of
  * every field sums to Fc, R L = I): what is left of FP64 per field is the projection, in full
- * warps, whatever the decisions.  A side whose two centre values are below 2^-10 of the
- * stencil's largest (a contaminated candidate would leave its rounding on a far smaller flux)
- * and values outside the fixed-point range take the general FP64 reconstruction, as do all
- * other schemes (!FIX).
+ * warps, whatever the decisions.  Items whose stencil reaches across a jump (reaches_jump: the large
+ * values beyond it would leave their rounding on a smaller flux) and values outside the
+ * fixed-point range take the general FP64 reconstruction, as do all other schemes (!FIX).
  *
  * What bounds it (ncu, 64^3 turbulence TENO8, 4 of 5 fields of 98 % of the faces listed): FP64
  * pipe 69 % busy, then waiting at the CTA's barriers.  Per 3-sweep launch 2.9 ms in FP64 (the
@@ -101,8 +100,12 @@ struct GridFace {
 
 /* Roe state and LLF speeds of one face into its row (entry r at row[r * TH]).  src.centre(e, rho,
    c, v): density, sound speed and velocity (normal first) of the face's left (0) and right (1)
-   cell; src.speed(q, u_n, c): stencil point q, speed32: truncated to FP32.  c~^2 in its cancellation-free form (weighted c^2
-   plus (gamma - 1)/2 wl wr |dv|^2), H~ = c~^2/(gamma - 1) + |u~|^2/2. */
+   cell; src.speed(q, u_n, c): stencil point q, speed32: truncated to FP32.  H~ = h + |u~|^2/2 with h =
+   c~^2/(gamma - 1) in its cancellation-free form (weighted c^2 plus (gamma - 1)/2 wl wr |dv|^2), then
+   c~^2 = (gamma - 1)(H~ - |u~|^2/2) back from the rounded H~: at Mach M the fields are of size M^2,
+   and R L = I has to hold to the rounding of c~^2 against that H~ (a c~^2 that H~ does not give
+   leaves M^2 times the rounding of H~ in the pressure: limited near-vacuum steps were up to 5 times
+   further off). */
 template <int NV, int K, int TH, class Src>
 __device__ __forceinline__ void face_rows(const Src& src, double* row, double gm1, double rgm1, int& st) {
   using R = NlRow<NV>;
@@ -123,11 +126,13 @@ __device__ __forceinline__ void face_rows(const Src& src, double* row, double gm
     dv2 = fma(y, y, dv2);
     row[(R::u + d) * TH] = x;
   }
-  const double c2 = fma(wl * cs[0], cs[0], fma(wr * cs[1], cs[1], 0.5 * gm1 * (wl * wr) * dv2));
+  const double c2f = fma(wl * cs[0], cs[0], fma(wr * cs[1], cs[1], 0.5 * gm1 * (wl * wr) * dv2));
+  const double Ht = fma(c2f, rgm1, 0.5 * q2);
+  const double c2 = gm1 * (Ht - 0.5 * q2);
   if (!(c2 > 0.0)) st |= ST_ROE;
   const double ci = rsqrt_nr(c2);
   const double b1 = gm1 * (ci * ci);
-  row[R::H * TH] = fma(c2, rgm1, 0.5 * q2);
+  row[R::H * TH] = Ht;
   row[R::ci * TH] = ci;
   row[R::ct * TH] = c2 * ci;
   row[R::b1 * TH] = b1;
@@ -236,9 +241,14 @@ __device__ __forceinline__ void general_sides(const double (&w)[K], const double
   }
 }
 
+template <int NV>
+__host__ __device__ constexpr unsigned allshear() { return ((1u << (NV - 1)) - 1u) & ~3u; }
+
 /* Face flux from the central one, F = Fc on entry (components in the axis's frame): Fc + sum_s r_s
-   correction_s; when a field is direct (dir), sum_s r_s fs with fs = l_s . Fc (+ correction) for
-   the others.  cm: central fields.  Both sums go through the vectors the eigenvectors share: a =
+   correction_s; when an acoustic or entropy field is direct (dir), sum_s r_s fs with fs = l_s . Fc (+
+   correction) for the others.  Where only shear fields are direct their component alone is, F_t = f_t +
+   u_t F_rho: l_s . Fc of the other fields, of size M^2 at Mach M, would not cancel against their
+   corrections to the rounding of the internal energy.  cm: central fields.  Both sums go through the vectors the eigenvectors share: a =
    (b2, -b1 u, b1) and b = (u_n, -e_n, 0)/c give l_{u-c} = (a + b)/2, l_{u+c} = (a - b)/2,
    l_entropy = e_0 - a, l_shear = e_t - u_t e_0, and with sigma = f_{u-c} + f_{u+c}, delta =
    (f_{u+c} - f_{u-c}) c:  F_0 = sigma + f_1,  F_d = (sigma + f_1) u_d + (delta if d = n, else
@@ -257,7 +267,15 @@ __device__ __forceinline__ void compose(const double* face, const double* fsv, u
     ut[d] = row(R::u + d);
     q2 = fma(ut[d], ut[d], q2);
   }
-  if (dir) {
+  const unsigned sh = allshear<NV>();
+  double raw[NV > 3 ? NV - 3 : 1];  /* f+ + f- of the direct shear fields */
+  if (!(dir & ~sh)) {
+#pragma unroll
+    for (int s = 2; s <= NV - 2; ++s) {
+      raw[s - 2] = fs[s];
+      if (dir >> s & 1u) fs[s] -= fma(-ut[s - 1], F[0], F[s]);
+    }
+  } else {
     double uF = 0.0;
 #pragma unroll
     for (int d = 0; d < D; ++d) uF = fma(ut[d], F[1 + d], uF);
@@ -280,7 +298,7 @@ __device__ __forceinline__ void compose(const double* face, const double* fsv, u
   F[1] += fma(m, ut[0], delta);
 #pragma unroll
   for (int s = 2; s <= NV - 2; ++s) {
-    F[s] += fma(m, ut[s - 1], fs[s]);
+    F[s] = (!(dir & ~sh) && (dir >> s & 1u)) ? fma(ut[s - 1], F[0], raw[s - 2]) : F[s] + fma(m, ut[s - 1], fs[s]);
     FE = fma(ut[s - 1], fs[s], FE);
   }
   F[NV - 1] += FE;
@@ -322,17 +340,73 @@ __device__ __noinline__ double general_cold(const double* w, const double* g, do
   return f;
 }
 
+/* FP32 value of a double from its high word (20 mantissa bits; below the FP32 range 0, above it inf) */
+__device__ __forceinline__ float f32_hi(const double* x) {
+  const int h = __ldg(reinterpret_cast<const int*>(x) + 1), m = (h & 0x7fffffff) - 0x38000000;
+  const int f = m < 0x100000 ? 0 : (m >= 0x0ff00000 ? 0x7f800000 : m << 3);
+  return __int_as_float(f | (h & (int)0x80000000));
+}
+
+/* Whether the stencil reaches across a jump: a point's density, or its size in the face's frame p +
+   (gamma - 1)/2 rho w^2 (w = v - v~; what the acoustic and entropy fields are made of), is more than
+   `most` times the larger of the face's two cells.  Up to there the limiters are applied as
+   corrections to Fc.  Fc and the corrections carry the rounding of the stencil's largest values, the
+   FP64 reconstruction that of the values it keeps, so the correction form is the more exact one where
+   the values are of one size and loses with the ratio where they are not: rms errors of the face
+   flux against 80-bit, in units of 2^-53 of the cells' |lambda U|, FP64 form | correction (2D, jumps
+   of rho and p every 7 cells, TENO6): MP ratio 1 0.71 | 0.50, 2 0.71 | 0.69, 4 0.75 | 1.08, 10 0.73 | 2.4,
+   1000 0.76 | 57; TVD5 ratio 1 0.58 | 0.24, 4 0.71 | 0.65 (jumps of p), 10 0.88 | 1.8.  It holds for the
+   face, not for a field: beside a field in FP64 another one's l_s . Fc would bring the far values
+   back.  (A NaN reaches.) */
+template <int NV, int K, int LIM, int TH>
+__device__ __forceinline__ bool reaches_jump(const GridFace<NV, K>& src, const double* p, const double* row, double gm1) {
+  constexpr int D = NV - 2, H = K / 2;
+  const float most = LIM == LIM_TVD5 ? 2.8f : 2.f, hg = 0.5f * f32_rz(gm1);
+  float ut[D], far[2] = {0.f, 0.f}, near[2] = {0.f, 0.f};
+#pragma unroll
+  for (int d = 0; d < D; ++d) ut[d] = f32_rz(row[(NlRow<NV>::u + d) * TH]);
+  bool nan = false;
+#pragma unroll 1
+  for (int q = 0; q < K; ++q) {
+    const long long x = src.cell(q);
+    const float rho = f32_hi(src.rho + x);
+    float w2 = 0.f;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const float w = f32_hi(src.vel[d] + x) - ut[d];
+      w2 = fmaf(w, w, w2);
+    }
+    const float s = fmaf(hg * rho, w2, f32_hi(p + x));
+    nan |= !(s <= 3e38f);
+    far[0] = fmaxf(far[0], rho);
+    far[1] = fmaxf(far[1], s);
+    if (q == H - 1 || q == H) {
+      near[0] = fmaxf(near[0], rho);
+      near[1] = fmaxf(near[1], s);
+    }
+  }
+  return nan || !(far[0] <= most * near[0] && far[1] <= most * near[1]);
+}
+
+/* The same for a shear field's own terms |u_t rho|, |m_t|, which vanish where the tangential velocity
+   does, as a difference of high words: up to 16 the error of the tangential flux stays at that of the
+   acoustic fields' part (0.58 | 0.65 at a ratio of 10; 0.77 | 13 at 100 without the rule). */
+constexpr unsigned kShearJump = 4u << 20;
+constexpr unsigned kJumpFace = 1u << 31;  /* s_dir: no field of the face takes the correction form */
+__device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
 /* Both split sides of an item from its projected W and G (columns w, g in shared memory):
    decisions, and the corrections of the nonsmooth sides in fixed point.  Returns false when the
    FP32 filter leaves a side undecided and `defer` is set.  Dx: K - 1 scratch words of the item's
-   thread.  em: biased exponent of a power of two above every |G| + |alpha W|.  The loops over
+   thread.  em: biased exponent of a power of two above every |G| + |alpha W|.  jump: the item's
+   corrections would cancel values far above the centre's (reaches_jump, kShearJump).  The loops over
    the points are rolled and everything rare is called, to keep the code that an item runs
    small (unrolled 4 or 8 times: 256^3 step 64 ms against 59, 64^3 turbulence 5.6 against 5.1). */
 template <int K, int LIM>
-__device__ __forceinline__ bool fixed_item(const double* w, const double* g, double al, int em, long long* Dx,
-                                           const SchemeDev& S, bool defer, unsigned& fl, double& fsum, bool& direct,
-                                           int& st) {
-  constexpr int c = K / 2 - 1, TH = NL_THREADS;
+__device__ __forceinline__ bool fixed_item(const double* w, const double* g, double al, int em, bool jump,
+                                           long long* Dx, const SchemeDev& S, bool defer, unsigned& fl, double& fsum,
+                                           bool& direct, int& st) {
+  constexpr int TH = NL_THREADS;
   constexpr unsigned allk = (1u << (K - 2)) - 1u;
   const bool inside = em >= 1024 - 40 && em <= 1024 + 40;
   const float unit = __int_as_float((inside ? em - 1077 + 127 : 0) << 23);  /* 2^(em - 1077): of the halved values */
@@ -342,14 +416,11 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
     unsigned zero = 0u;
-    int ec = 0, es;  /* exponents of the larger of the two centre values and of the side's largest */
-    auto expo = [](double x) -> int { return (int)((unsigned)__double2hiint(x) >> 20 & 0x7ffu); };
     {
       const int p0 = side ? (K - 1) * TH : 0, dp = side ? -TH : TH;
       const double hs = side ? -al : al;
       double v0 = fma(hs, w[p0], g[p0]);
       long long x0 = to_fixed(v0, em);
-      es = expo(v0);
 #pragma unroll 1
       for (int t = 0; t < K - 1; ++t) {
         const int p = p0 + (t + 1) * dp;
@@ -357,8 +428,6 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
         const long long x1 = to_fixed(v1, em);
         Dx[t * TH] = x1 - x0;
         zero |= dbits(v1) == dbits(v0) ? 1u << t : 0u;
-        es = max(es, expo(v1));
-        if (t == c) ec = max(expo(v0), expo(v1));
         x0 = x1;
         v0 = v1;
       }
@@ -376,7 +445,7 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
     }
     fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
     if (b != allk) {
-      if (!inside || ec < es - 10) {
+      if (!inside || jump) {
         direct = true;
       } else {
         long long D[K - 1];
@@ -481,7 +550,7 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       s_base[tid] = base;
       s_f[tid] = f;
       s_cm[tid] = A.sch.default_d ? (allf & ~mask) : 0u;
-      s_dir[tid] = 0u;
+      s_dir[tid] = FIX && reaches_jump<NV, K, LIM, TH>(src, Pp, s_row + tid, A.gamma - 1.0) ? kJumpFace : 0u;
     }
     /* the chunk's (face, field) items, field after field */
 #pragma unroll
@@ -527,13 +596,16 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       const double* const ut = A.U + gc(shear ? s : 1) * A.ncell;
       const long long base = s_base[fc];
       const int f = s_f[fc];
-      /* W and G/2 (FIX: G) of stencil point q, G = l . F = u_n W + p (l_n + u_n l_E) */
-      auto project = [&](int q, double& w, double& hg) {
+      /* W and G/2 (FIX: G) of stencil point q, G = l . F = u_n W + p (l_n + u_n l_E); term: the larger
+         of a shear field's |l_0 rho|, |m_t|, as the sum of the factors' high words (FIX only) */
+      auto project = [&](int q, double& w, double& hg, unsigned& term) {
         const long long cell = base + sa * bc_near(f - H + q, na, bc);
         const double un = __ldg(Pn + cell);
         if (shear) {
-          w = fma(l[0], __ldg(up[0] + cell), __ldg(ut + cell));
+          const double rho = __ldg(up[0] + cell), m = __ldg(ut + cell);
+          w = fma(l[0], rho, m);
           hg = un * w;
+          if constexpr (FIX) term = max(abs_hi(l[0]) + abs_hi(rho), 0x3ff00000u + abs_hi(m));
         } else {
           w = l[0] * __ldg(up[0] + cell);
 #pragma unroll
@@ -548,10 +620,14 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       double wv[REC ? K : 1], op[REC ? K : 1], om[REC ? K : 1];  /* W; frozen linear weights of f+ and f- */
       if constexpr (FIX) {
         int eg = 0, ew = 0;
+        unsigned far = 0u, near = 0u;
 #pragma unroll 1
         for (int q = 0; q < K; ++q) {
           double w, hg;
-          project(q, w, hg);
+          unsigned term = 0u;
+          project(q, w, hg, term);
+          far = max(far, term);
+          if (q == H - 1 || q == H) near = max(near, term);
           s_w[q * TH + tid] = w;
           s_g[q * TH + tid] = hg;
           eg = max(eg, (int)((unsigned)__double2hiint(hg) >> 20 & 0x7ffu));
@@ -560,16 +636,18 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
         /* 2 |v| <= |G| + |alpha W| < 2^(em - 1022) */
         const double al = ha + ha;
         const int em = 1 + max(eg, ew + (int)((unsigned)__double2hiint(al) >> 20 & 0x7ffu) - 1022);
-        if (!fixed_item<K, LIM>(s_w + tid, s_g + tid, al, em, s_D + tid, A.sch, pass == 0 && nitem > TH, fl, fsum,
-                                direct, st)) {
+        const bool jump = far - near > kShearJump || (s_dir[fc] & kJumpFace);
+        if (!fixed_item<K, LIM>(s_w + tid, s_g + tid, al, em, jump, s_D + tid, A.sch, pass == 0 && nitem > TH, fl,
+                                fsum, direct, st)) {
           s_later[atomicAdd(&s_nlater, 1)] = (unsigned short)item;
           continue;
         }
       } else {
         double w[K], hg[K];
+        unsigned term = 0u;
 #pragma unroll
         for (int q = 0; q < K; ++q) {
-          project(q, w[q], hg[q]);
+          project(q, w[q], hg[q], term);
           if constexpr (REC) wv[q] = w[q];
         }
         general_sides<K, LIM, REC>(w, hg, ha, A.sch, fl, fsum, op, om, st);
@@ -614,7 +692,7 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
 
     /* ---- (2) the face fluxes ---- */
     if (tid < nf && s_cm[tid] != allf) {
-      const unsigned cm = s_cm[tid], dir = s_dir[tid];
+      const unsigned cm = s_cm[tid], dir = s_dir[tid] & allf;
       double* const Fo = A.Fhat[ax];
       double Fh[NV];
 #pragma unroll
