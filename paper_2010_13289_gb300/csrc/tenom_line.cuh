@@ -52,10 +52,12 @@ struct LineFace {
 
 /* Stages the points of faces f0 .. f0 + nf - 1 (nf <= FACES) of a line of n cells at U (component v
    at v * stride; read through L2, other CTAs of a cluster may have written it).  All threads of the
-   CTA call it.  Returns the largest |u| + c of the tile's nf - 1 own cells seen by this thread. */
+   CTA call it.  Returns the largest |u| + c of the tile's nf - 1 own cells seen by this thread.
+   cfl: the CFL maximum is taken here, and a state that is not positive reported as the grid's signal
+   speed kernel does (point_prims' integer tests let a NaN pass). */
 template <int K, int TILE, int FACES>
 __device__ __forceinline__ double line_stage(LineTile<K, TILE, FACES>& S, const double* U, long long stride, int n, int bc,
-                                             int f0, int nf, double gamma, int& st) {
+                                             int f0, int nf, double gamma, int& st, bool cfl = false) {
   using T = LineTile<K, TILE, FACES>;
   constexpr int NV = 3, H = K / 2, NP = T::NP;
   const int tid = threadIdx.x;
@@ -76,6 +78,10 @@ __device__ __forceinline__ double line_stage(LineTile<K, TILE, FACES>& S, const 
     S.pt[T::F1 * NP + p] = fma(u[1], vel[0], pr);
     S.pt[T::F2 * NP + p] = (u[2] + pr) * vel[0];
     stage_screen_point<NV>(u, vel, pr, cs, S.sf, NP, p);
+    if (cfl) {
+      if (!(u[0] > 0.0)) st |= ST_RHO;
+      if (!(pr > 0.0)) st |= ST_P;
+    }
     const double s = fabs(vel[0]) + cs;
     if (p >= H && p < H + nf - 1 && f0 - H + p < n && s > smax) smax = s;
   }

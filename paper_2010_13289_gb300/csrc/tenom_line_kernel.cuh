@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(LINE_TILE) line_kernel(const LineArgs A) {
 #pragma unroll 1
   for (int step = 0; step < A.nsteps; ++step) {
     /* the CFL maximum comes with the first stage's points */
-    double dt, m = nf ? line_stage(S, A.U, n, n, A.bc, f0, nf, A.gamma, st) * A.rdx : 0.0;
+    double dt, m = nf ? line_stage(S, A.U, n, n, A.bc, f0, nf, A.gamma, st, !A.dt) * A.rdx : 0.0;
     if (A.dt) {
       dt = *A.dt;
     } else {  /* dt = min(cfl / max (|u| + c)/dx, t_end - t), 0 once t reaches t_end */
@@ -62,7 +62,6 @@ __global__ void __launch_bounds__(LINE_TILE) line_kernel(const LineArgs A) {
       dt = rem < dt ? rem : dt;
       if (!(rem > 0.0)) dt = 0.0;
     }
-    if (dt == 0.0) break;  /* nothing moves, now or in a later step (the same on every CTA) */
 #pragma unroll 1
     for (int stage = 0; stage < 3; ++stage) {
       const double* Us = stage == 0 ? A.U : (stage == 1 ? A.W1 : A.W2);
@@ -71,7 +70,7 @@ __global__ void __launch_bounds__(LINE_TILE) line_kernel(const LineArgs A) {
       if (nf) {
         if (stage > 0) line_stage(S, Us, n, n, A.bc, f0, nf, A.gamma, st);
         line_fluxes<K, LIM, TILE, PP>(S, n, f0, nf, A.gamma, A.rgm1, A.sch, 2.0 * dt * A.rdx, st);
-        if (tid < cells) {
+        if (tid < cells && dt != 0.0) {
 #pragma unroll
           for (int v = 0; v < 3; ++v) {
             const long long g = (long long)v * n + c;
@@ -81,8 +80,12 @@ __global__ void __launch_bounds__(LINE_TILE) line_kernel(const LineArgs A) {
           }
         }
       }
+      if (dt == 0.0) break;
       cl.sync();  /* the stage's state is complete, and S free */
     }
+    /* nothing moves, now or in a later step (the same on every CTA); the fluxes of the state were
+       formed once for what they report */
+    if (dt == 0.0) break;
     t = t + dt;
   }
   cl.sync();  /* no CTA leaves while another may still write its shared memory */

@@ -147,10 +147,15 @@ __device__ __forceinline__ void stage_screen_differences(float* sf, int NP, int 
     const float* h = sf + (L::hi + c) * NP + p;
     const float* l = sf + (L::lo + c) * NP + p;
     float x = (h[step] - h[0]) + (l[step] - l[0]);
-    any = fmaxf(any, fabsf(x));
-    /* equal to 47 bits but not bit for bit: not a constant stencil (nor one that can be certified) */
-    if (c == 0 && any == 0.f &&
-        __float_as_uint(sf[L::chk * NP + p + step]) != __float_as_uint(sf[L::chk * NP + p])) x = 1e-37f;
+    any += fabsf(x);  /* a sum, which keeps a NaN */
+    if (c == 0) {
+      /* equal to 47 bits but not bit for bit: not a constant stencil (nor one that can be certified) */
+      if (any == 0.f &&
+          __float_as_uint(sf[L::chk * NP + p + step]) != __float_as_uint(sf[L::chk * NP + p])) x = 1e-37f;
+      /* a point that is not finite in FP32 (infinite here: f32_rz): its maxima would drop the NaN of
+         inf - inf, and a stencil of such points would pass for a constant one */
+      if (!(any <= 3e38f)) x = __int_as_float(0x7f800000);
+    }
     sf[(L::df + c) * NP + p] = x;
   }
 }
@@ -237,7 +242,7 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
   for (int d = 0; d < D; ++d) mx = fmaxf(mx, Mv[d]);
   /* a constant stencil: every sequence is constant, beta = tau = 0, all smooth (and eta = 1, [beta] = 10) */
   if (mx == 0.f) return 0u;
-  if (!(th <= 2.f && q2 <= 1e8f * c2)) return all;
+  if (!(th <= 2.f && q2 <= 1e8f * c2 && mx <= 3e38f)) return all;  /* (mx: not finite) */
   unsigned still = 0u;  /* shear fields with no tangential velocity at all: the sequence is zero */
 #pragma unroll
   for (int d = 0; d < D; ++d)
