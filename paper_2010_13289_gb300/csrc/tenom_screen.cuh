@@ -242,7 +242,8 @@ __device__ __forceinline__ unsigned screen_face(const float* sf, int NP, int p0,
   for (int d = 0; d < D; ++d) mx = fmaxf(mx, Mv[d]);
   /* a constant stencil: every sequence is constant, beta = tau = 0, all smooth (and eta = 1, [beta] = 10) */
   if (mx == 0.f) return 0u;
-  if (!(th <= 2.f && q2 <= 1e8f * c2 && mx <= 3e38f)) return all;  /* (mx: not finite) */
+  /* (c2: the fast division returns 0 for divisors above 2^126; mx: not finite) */
+  if (!(th <= 2.f && q2 <= 1e8f * c2 && c2 <= 8e37f && mx <= 3e38f)) return all;
   unsigned still = 0u;  /* shear fields with no tangential velocity at all: the sequence is zero */
 #pragma unroll
   for (int d = 0; d < D; ++d)
