@@ -408,14 +408,33 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
                                            bool& direct, int& st) {
   constexpr int TH = NL_THREADS;
   constexpr unsigned allk = (1u << (K - 2)) - 1u;
-  const bool inside = em >= 1024 - 40 && em <= 1024 + 40;
-  const float unit = __int_as_float((inside ? em - 1077 + 127 : 0) << 23);  /* 2^(em - 1077): of the halved values */
-  Acc96 acc;
   fl = 0u;
   direct = false;
+  if (em < 1024 - 40 || em > 1024 + 40) {  /* outside the fixed-point range: FP64, and at once (no pass can do better) */
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) fl |= decide_cold<K>(w, g, al, side, S, st) << (8 * side);
+    direct = (fl & (allk | allk << 8)) != (allk | allk << 8);
+    fsum = general_cold<K, LIM>(w, g, al, fl, S);
+    return true;
+  }
+  const float unit = __int_as_float((em - 1077 + 127) << 23);  /* 2^(em - 1077): of the halved values */
+  Acc96 acc;
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
-    unsigned zero = 0u;
+    unsigned zero = 0u, b = 0u;
+    int e = 7;
+    auto cold = [&]() {
+      const unsigned f = decide_cold<K>(w, g, al, side, S, st);
+      b = f & allk;
+      e = 7 + (int)(f >> 6);
+    };
+    if (S.exact_decisions) {  /* decided first: a smooth side needs no differences */
+      cold();
+      if (b == allk) {
+        fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
+        continue;
+      }
+    }
     {
       const int p0 = side ? (K - 1) * TH : 0, dp = side ? -TH : TH;
       const double hs = side ? -al : al;
@@ -432,20 +451,18 @@ __device__ __forceinline__ bool fixed_item(const double* w, const double* g, dou
         v0 = v1;
       }
     }
-    float d[K - 1];
+    if (!S.exact_decisions) {
+      float d[K - 1];
 #pragma unroll
-    for (int t = 0; t < K - 1; ++t) d[t] = __ll2float_rz(Dx[t * TH]) * unit;
-    unsigned b = 0;
-    int e = 7;
-    if (S.exact_decisions || !inside || !cutoff_filter<K>(d, 1.01f * unit, zero, S, b, e)) {
-      if (defer) return false;
-      const unsigned f = decide_cold<K>(w, g, al, side, S, st);
-      b = f & allk;
-      e = 7 + (int)(f >> 6);
+      for (int t = 0; t < K - 1; ++t) d[t] = __ll2float_rz(Dx[t * TH]) * unit;
+      if (!cutoff_filter<K>(d, 1.01f * unit, zero, S, b, e)) {
+        if (defer) return false;
+        cold();
+      }
     }
     fl |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
     if (b != allk) {
-      if (!inside || jump) {
+      if (jump) {
         direct = true;
       } else {
         long long D[K - 1];
