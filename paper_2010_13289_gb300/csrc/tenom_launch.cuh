@@ -91,11 +91,13 @@ static cudaError_t launch_nonlinear_one(const NonlinArgs& a, cudaStream_t st) {
 
 template <int NV, int K, bool REC>
 static cudaError_t launch_nonlinear_k(const NonlinArgs& a, int lim, cudaStream_t st) {
-  if constexpr (!REC) {
-    if (NV > 3 && a.sch.fixed) {  /* a line's few listed faces are latency-bound: 45 us a launch in fixed point, 30 in FP64 */
-      if (lim == LIM_MP) return launch_nonlinear_one<NV, K, LIM_MP, false, true>(a, st);
-      if (lim == LIM_TVD5) return launch_nonlinear_one<NV, K, LIM_TVD5, false, true>(a, st);
+  if constexpr (NV > 3) {  /* a line's few listed faces are latency-bound: 45 us a launch in fixed point, 30 in FP64 */
+    if (a.sch.fixed) {
+      if (lim == LIM_MP) return launch_nonlinear_one<NV, K, LIM_MP, REC, true>(a, st);
+      if (lim == LIM_TVD5) return launch_nonlinear_one<NV, K, LIM_TVD5, REC, true>(a, st);
     }
+  }
+  if constexpr (!REC) {
     /* Van Albada: forward only (no frozen linear form to record) */
     if (lim == LIM_VA) return launch_nonlinear_one<NV, K, LIM_VA, false, false>(a, st);
   }

@@ -340,6 +340,48 @@ __device__ __noinline__ double general_cold(const double* w, const double* g, do
   return f;
 }
 
+/* A field's rows of the tape at o (and at oc, unless null), stride nface: fs, omegaW = sum_q delta_q W_q,
+   sigma_q, delta_q with fs = sum_q sigma_q G_q + (alpha/2) delta_q W_q, sigma_q = (op_q +
+   om_{K-1-q})/2, delta_q = op_q - om_{K-1-q} (op, om: the frozen linear weights of f+ and f-) */
+template <int K, class Wq>
+__device__ __forceinline__ void put_tape(const Wq& w, const double* op, const double* om, double fs, bool central,
+                                         double* o, double* oc, long long nface) {
+  double wW = 0.0;
+#pragma unroll
+  for (int q = 0; q < K; ++q) wW = fma(op[q] - om[K - 1 - q], w(q), wW);
+  for (double* p = o; p; p = p == o ? oc : nullptr) {
+    p[0] = fs;
+    p[nface] = central ? __longlong_as_double((long long)kCentralMark) : wW + 0.0;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      p[(2 + q) * nface] = 0.5 * (op[q] + om[K - 1 - q]);
+      p[(2 + K + q) * nface] = op[q] - om[K - 1 - q];
+    }
+  }
+}
+/* The tape of a fixed-point item.  The face flux comes from the same fixed-point form as the forward
+   kernel's, so that a recorded step has its bits (a rollout is recomputed from its checkpoints for the
+   reverse, and branches frozen on states that differ in the last bits are another trajectory's);
+   only the frozen weights are formed in FP64. */
+template <int K, int LIM>
+__device__ __noinline__ void record_item(const double* w, const double* g, double al, unsigned fl, const SchemeDev& S,
+                                         double* o, double* oc, long long nface, bool central) {
+  constexpr unsigned allk = (1u << (K - 2)) - 1u;
+  double op[K], om[K], f = 0.0;
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    double v[K], wt[K];
+    split_side<K>(w, g, al, side, v);
+    f += teno_general<K, LIM, true>(v, S, fl >> (8 * side) & allk, wt);
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      if (side) om[q] = wt[q];
+      else op[q] = wt[q];
+    }
+  }
+  put_tape<K>([&](int q) { return w[q * NL_THREADS]; }, op, om, f, central, o, oc, nface);
+}
+
 /* FP32 value of a double from its high word (20 mantissa bits; below the FP32 range 0, above it inf) */
 __device__ __forceinline__ float f32_hi(const double* x) {
   const int h = __ldg(reinterpret_cast<const int*>(x) + 1), m = (h & 0x7fffffff) - 0x38000000;
@@ -634,7 +676,8 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       unsigned fl = 0u;
       double fsum = 0.0;
       bool direct = !FIX;
-      double wv[REC ? K : 1], op[REC ? K : 1], om[REC ? K : 1];  /* W; frozen linear weights of f+ and f- */
+      constexpr int KR = REC && !FIX ? K : 1;
+      double wv[KR], op[KR], om[KR];  /* W; frozen linear weights of f+ and f- */
       if constexpr (FIX) {
         int eg = 0, ew = 0;
         unsigned far = 0u, near = 0u;
@@ -685,23 +728,11 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
         }
       }
       if constexpr (REC) {
-        /* the tape's rows of this field: fs, omegaW = sum_q delta_q W_q, sigma_q, delta_q with
-           fs = sum_q sigma_q G_q + (alpha/2) delta_q W_q, sigma_q = (op_q + om_{K-1-q})/2,
-           delta_q = op_q - om_{K-1-q} */
-        for (int r = 0; r < (copy ? 2 : 1); ++r) {
-          double* o = A.lin[ax] + (r ? fcp : fi) + (long long)s * (2 * K + 2) * nface;
-          double wW = 0.0;
-#pragma unroll
-          for (int q = 0; q < K; ++q) {
-            const double dq = op[q] - om[K - 1 - q];
-            o[(2 + q) * nface] = 0.5 * (op[q] + om[K - 1 - q]);
-            o[(2 + K + q) * nface] = dq;
-            wW = fma(dq, wv[q], wW);
-          }
-          const bool central = (fl & (allk | allk << 8)) == (allk | allk << 8) && A.sch.default_d;
-          o[0] = fsum;
-          o[nface] = central ? __longlong_as_double((long long)kCentralMark) : wW + 0.0;
-        }
+        double* const o = A.lin[ax] + fi + (long long)s * (2 * K + 2) * nface;
+        double* const oc = copy ? A.lin[ax] + fcp + (long long)s * (2 * K + 2) * nface : nullptr;
+        const bool central = (fl & (allk | allk << 8)) == (allk | allk << 8) && A.sch.default_d;
+        if constexpr (FIX) record_item<K, LIM>(s_w + tid, s_g + tid, ha + ha, fl, A.sch, o, oc, nface, central);
+        else put_tape<K>([&](int q) { return wv[q]; }, op, om, fsum, central, o, oc, nface);
       }
     }
     __syncthreads();
