@@ -101,7 +101,7 @@ __device__ __forceinline__ void cell_update(const CellUpdate& A, long long nc, l
     } else {
       const double us = A.Us[v * nc + c];
       const double t1 = us + dt * r;
-      un[v] = (A.mode == 1) ? t1 : A.cA * A.U0[v * nc + c] + A.cB * t1;
+      un[v] = (A.mode == 1) ? t1 : fma(A.cA, A.U0[v * nc + c], __dmul_rn(A.cB, t1));
     }
     A.out[v * nc + c] = un[v];
   }

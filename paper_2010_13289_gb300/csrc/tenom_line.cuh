@@ -76,7 +76,8 @@ __device__ __forceinline__ double line_stage(LineTile<K, TILE, FACES>& S, const 
     S.pt[T::pr * NP + p] = pr;
     S.pt[T::cs * NP + p] = cs;
     S.pt[T::F1 * NP + p] = fma(u[1], vel[0], pr);
-    S.pt[T::F2 * NP + p] = (u[2] + pr) * vel[0];
+    /* no contraction of u + pr into pr's product, which the grid sweeps load: the same bits */
+    S.pt[T::F2 * NP + p] = __dmul_rn(__dadd_rn(u[2], pr), vel[0]);
     stage_screen_point<NV>(u, vel, pr, cs, S.sf, NP, p);
     if (cfl) {
       if (!(u[0] > 0.0)) st |= ST_RHO;

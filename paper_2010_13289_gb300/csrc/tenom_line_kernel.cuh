@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(LINE_TILE) line_kernel(const LineArgs A) {
             const long long g = (long long)v * n + c;
             const double r = 0.0 - (S.F[v * TILE + tid + 1] - S.F[v * TILE + tid]) * A.rdx;
             const double t1 = __ldcg(Us + g) + dt * r;
-            __stcg(out + g, stage == 0 ? t1 : cA * __ldcg(A.U + g) + cB * t1);
+            /* rounded as stage_kernel's cA U0 + cB t1 is: a step has the bits of the grid sweeps' */
+            __stcg(out + g, stage == 0 ? t1 : fma(cA, __ldcg(A.U + g), __dmul_rn(cB, t1)));
           }
         }
       }

@@ -8,7 +8,7 @@ from paper_2010_13289_gb300 import problems as PB
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-SHAPES = [((100, 37), (0, 1)), ((30, 11, 17), (0, 1, 0))]
+SHAPES = [((9,), (1,)), ((500,), (1,)), ((1901,), (0,)), ((3000,), (0,)), ((100, 37), (0, 1)), ((30, 11, 17), (0, 1, 0))]
 
 
 @pytest.mark.parametrize("shape,bc", SHAPES)
