@@ -852,8 +852,14 @@ static cudaError_t rk3_core(tenom_ctx* c, double* U) {
   return e;
 }
 
-/* 1D grids that one cluster covers advance in one launch (line_kernel) */
-static bool is_line(const tenom_ctx* c) { return c->nv == 3 && c->ncell <= line_cells_max(c->s.K); }
+/* 1D grids that one cluster covers advance in one launch (line_kernel), where the device can hold it */
+static bool is_line(const tenom_ctx* c) {
+  if (!use_line(c->nv, c->ncell, c->s.K, 1)) return false;
+  const bool pp = c->s.positivity == TENOM_PP_ON;
+  const int n = c->g.n[0];
+  return use_line(c->nv, c->ncell, c->s.K,
+                  c->s.K == 6 ? line_clusters_k6(n, c->s.limiter, pp) : line_clusters_k8(n, c->s.limiter, pp));
+}
 
 /* nsteps steps of a short line: CFL steps from *t_dev, or one of length *dt_dev */
 static cudaError_t launch_line(tenom_ctx* c, double* U, const double* dt_dev, double* t_dev, double t_end, double cfl,

@@ -215,10 +215,21 @@ struct LineArgs {
 constexpr int LINE_TILE = 128;
 constexpr int LINE_CLUSTER = 16;
 inline int line_cells_max(int K) { return LINE_CLUSTER * (LINE_TILE - K); }
+/* CTAs for a line of n cells: four cells each until the cluster is full */
+inline int line_ctas(int n) { return n < 4 * LINE_CLUSTER ? (n + 3) / 4 : LINE_CLUSTER; }
+/* Whether a grid advances in line_kernel.  clusters: how many clusters of line_ctas CTAs the device can
+   hold at once, as the runtime reports it (16 CTAs are above the portable 8, and a partition of the
+   GPU may have no such group of SMs); none: the grid sweeps, which give the same bits. */
+inline bool use_line(int nv, long long ncell, int K, int clusters) {
+  return nv == 3 && ncell <= line_cells_max(K) && clusters > 0;
+}
 
-/* nsteps SSP-RK3 steps of a 1D grid of at most line_cells_max cells in one launch of one cluster
+/* nsteps SSP-RK3 steps of a 1D grid of at most line_cells_max cells in one launch of one cluster,
+   and the clusters that fit on the current device (asked once per device and size)
    (tenom_line_k6.cu, tenom_line_k8.cu) */
 cudaError_t launch_line_k6(const LineArgs& a, int lim, bool pp, cudaStream_t st);
 cudaError_t launch_line_k8(const LineArgs& a, int lim, bool pp, cudaStream_t st);
+int line_clusters_k6(int n, int lim, bool pp);
+int line_clusters_k8(int n, int lim, bool pp);
 
 }  // namespace tenom

@@ -3,6 +3,9 @@
 
 namespace tenom {
 
-cudaError_t launch_line_k8(const LineArgs& a, int lim, bool pp, cudaStream_t st) { return launch_line_k<8>(a, lim, pp, st); }
+cudaError_t launch_line_k8(const LineArgs& a, int lim, bool pp, cudaStream_t st) {
+  return line_ops_k<8>(lim, pp).launch(a, st);
+}
+int line_clusters_k8(int n, int lim, bool pp) { return line_ops_k<8>(lim, pp).clusters(n); }
 
 }  // namespace tenom

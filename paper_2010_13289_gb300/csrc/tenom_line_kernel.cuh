@@ -95,33 +95,64 @@ __global__ void __launch_bounds__(LINE_TILE) line_kernel(const LineArgs A) {
 }
 
 template <int K, int LIM, bool PP>
-static cudaError_t launch_line_one(const LineArgs& a, cudaStream_t st) {
-  static AttrOnce attr;
-  const size_t smem = sizeof(LineTile<K, LINE_TILE, LINE_TILE - K + 1>);
-  cudaError_t e = ensure_smem_attr(line_kernel<K, LIM, PP>, attr, smem, true);
-  if (e != cudaSuccess) return e;
-  const int C = a.n < 4 * LINE_CLUSTER ? (a.n + 3) / 4 : LINE_CLUSTER;
+struct LineLaunch {
+  static constexpr size_t smem = sizeof(LineTile<K, LINE_TILE, LINE_TILE - K + 1>);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)C);
-  cfg.blockDim = dim3(LINE_TILE);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)C;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, line_kernel<K, LIM, PP>, a);
-}
+  LineLaunch(int n, cudaStream_t st) {
+    cfg.gridDim = dim3((unsigned)line_ctas(n));
+    cfg.blockDim = dim3(LINE_TILE);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cfg.gridDim.x;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  static cudaError_t prepare() {
+    static AttrOnce attr;
+    return ensure_smem_attr(line_kernel<K, LIM, PP>, attr, smem, true);
+  }
+  static cudaError_t launch(const LineArgs& a, cudaStream_t st) {
+    const cudaError_t e = prepare();
+    if (e != cudaSuccess) return e;
+    const LineLaunch l(a.n, st);
+    return cudaLaunchKernelEx(&l.cfg, line_kernel<K, LIM, PP>, a);
+  }
+  static int clusters(int n) {
+    static std::atomic<signed char> known[AttrOnce::kMaxDevices][LINE_CLUSTER + 1];  /* 0: not asked, else 1 + clusters (0 or 1) */
+    int dev = -1, fit = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= AttrOnce::kMaxDevices) return 0;
+    std::atomic<signed char>& k = known[dev][line_ctas(n)];
+    if (const signed char v = k.load(std::memory_order_relaxed)) return v - 1;
+    const LineLaunch l(n, nullptr);
+    cudaError_t e = prepare();
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&fit, line_kernel<K, LIM, PP>, &l.cfg);
+    if (e != cudaSuccess) {
+      (void)cudaGetLastError();
+      fit = 0;
+    }
+    k.store((signed char)(fit > 0 ? 2 : 1), std::memory_order_relaxed);
+    return fit > 0 ? 1 : 0;
+  }
+};
 
+struct LineOps {
+  cudaError_t (*launch)(const LineArgs&, cudaStream_t);
+  int (*clusters)(int);
+};
+template <int K, int LIM>
+static LineOps line_ops(bool pp) {
+  if (pp) return {LineLaunch<K, LIM, true>::launch, LineLaunch<K, LIM, true>::clusters};
+  return {LineLaunch<K, LIM, false>::launch, LineLaunch<K, LIM, false>::clusters};
+}
 template <int K>
-static cudaError_t launch_line_k(const LineArgs& a, int lim, bool pp, cudaStream_t st) {
-  if (lim == LIM_MP) return pp ? launch_line_one<K, LIM_MP, true>(a, st) : launch_line_one<K, LIM_MP, false>(a, st);
-  if (lim == LIM_TVD5) return pp ? launch_line_one<K, LIM_TVD5, true>(a, st) : launch_line_one<K, LIM_TVD5, false>(a, st);
-  if (lim == LIM_VA) return pp ? launch_line_one<K, LIM_VA, true>(a, st) : launch_line_one<K, LIM_VA, false>(a, st);
-  return cudaErrorNotSupported;
+static LineOps line_ops_k(int lim, bool pp) {
+  if (lim == LIM_MP) return line_ops<K, LIM_MP>(pp);
+  if (lim == LIM_TVD5) return line_ops<K, LIM_TVD5>(pp);
+  return line_ops<K, LIM_VA>(pp);
 }
 
 }  // namespace tenom
