@@ -309,7 +309,8 @@ const char* tenom_last_error(const tenom_ctx* ctx);
 
 /* Measurement helper (not part of the method): average duration in ms of the face sweep
  * of one axis (its screen and its share of the stage's nonlinear launch) over the last tenom_rk3_step/tenom_advance calls, timed with CUDA events on
- * the context stream when timing is enabled.  enable != 0 turns timing on and resets. */
+ * the context stream when timing is enabled.  enable != 0 turns timing on and resets.  While it is
+ * on, 1D grids that otherwise advance in one launch per call take separate sweeps (same results). */
 tenom_status tenom_kernel_timing(tenom_ctx* ctx, int enable, double* face_ms_per_launch, long long* launches);
 
 /* FP64 pipe throughput probe (not part of the method): runs `iters` dependent-chain DFMA

@@ -852,9 +852,10 @@ static cudaError_t rk3_core(tenom_ctx* c, double* U) {
   return e;
 }
 
-/* 1D grids that one cluster covers advance in one launch (line_kernel), where the device can hold it */
+/* 1D grids that one cluster covers advance in one launch (line_kernel), where the device can hold it; not
+   while face sweeps are timed: the line launch has none (and the sweeps give the same bits) */
 static bool is_line(const tenom_ctx* c) {
-  if (!use_line(c->nv, c->ncell, c->s.K, 1)) return false;
+  if (c->timing || !use_line(c->nv, c->ncell, c->s.K, 1)) return false;
   const bool pp = c->s.positivity == TENOM_PP_ON;
   const int n = c->g.n[0];
   return use_line(c->nv, c->ncell, c->s.K,
