@@ -212,8 +212,8 @@ tenom_status tenom_batch_autotune(tenom_batch* b, double* U, int* tile, int* cta
 tenom_status tenom_batch_set_tiling(tenom_batch* b, int tile, int ctas_per_sm);
 
 /* Size of the static device scratch for the face fluxes of tenom_rhs_noalloc: 16 MiB, held on
- * every GPU that loads this library until the process exits (with 20 MiB more for the face lists and the
- * cell primitives). */
+ * every GPU that loads this library until the process exits (with 4 MiB more for the face lists; the
+ * cell primitives of a call go through dUdt). */
 #define TENOM_NOALLOC_SCRATCH_BYTES (16u << 20)
 
 /* tenom_rhs without a context and without any device allocation.  The paper has no

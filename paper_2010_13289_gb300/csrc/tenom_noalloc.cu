@@ -15,10 +15,10 @@ namespace tenom {
 
 /* first 256 bytes: status word, list lengths; then the face buffers, axis after axis; after
    TENOM_NOALLOC_SCRATCH_BYTES the face lists of the nonlinear kernel (5 bytes per face, at most
-   (16 MiB / 8) / 3 faces in 1D, 3.4 MiB) and the cell primitives (nvar values per cell, never
-   more than the face fluxes) */
+   (16 MiB / 8) / 3 faces in 1D, 3.4 MiB).  The cell primitives, nvar values per cell, need no room of
+   their own: dUdt has their size and is written last, by a kernel that reads faces only. */
 static constexpr size_t kListBytes = 4u << 20;
-static __device__ __align__(256) double g_noalloc_scratch[(2 * TENOM_NOALLOC_SCRATCH_BYTES + kListBytes) / sizeof(double)];
+static __device__ __align__(256) double g_noalloc_scratch[(TENOM_NOALLOC_SCRATCH_BYTES + kListBytes) / sizeof(double)];
 static_assert(5 * (TENOM_NOALLOC_SCRATCH_BYTES / sizeof(double) / 3 + 1) + 64 <= kListBytes, "face lists fit");
 
 static constexpr long long kStatusDoubles = 256 / sizeof(double);
@@ -91,7 +91,7 @@ extern "C" tenom_status tenom_rhs_noalloc(const tenom_grid* grid, const tenom_sc
     e = cudaMemsetAsync(status, 0, sizeof(int), st);  /* the shared word keeps the last call's bits */
     if (e != cudaSuccess) return TENOM_E_CUDA;
   }
-  double* P = scratch + cap + kListBytes / sizeof(double);
+  double* const P = dUdt;
   double* F[3] = {nullptr, nullptr, nullptr};
   long long off = kStatusDoubles;
   for (int a = 0; a < grid->dim; ++a) {
