@@ -1084,8 +1084,10 @@ static cudaError_t adj_sweeps(tenom_ctx* c, const double* U, const uint8_t* flag
   A.ncell = c->ncell;
   A.gamma = c->g.gamma;
   A.sch = scheme_dev(c->s);
+  A.whole = A.sch.default_d ? 0 : 1;
   cudaError_t e = launch_prims(c, U, true);
-  for (int a = -1; a < c->g.dim && e == cudaSuccess; ++a) {
+  if (A.whole && e == cudaSuccess) e = cudaMemsetAsync(Z, 0, sizeof(double) * c->nv * c->ncell, c->st);
+  for (int a = A.whole ? 0 : -1; a < c->g.dim && e == cudaSuccess; ++a) {
     if (a >= 0) {
       A.flags = flags_stage ? flags_stage + flags_offset(c, a) : nullptr;
       A.lin = lin_stage ? lin_stage + lin_offset(c, a) : nullptr;

@@ -36,6 +36,8 @@ struct AdjArgs {
   double rdx[3];
   double gamma;
   SchemeDev sch;
+  int whole;             /* 1: no field is ever central (d_k of the caller's), so the fields carry the whole flux
+                            (sigma instead of sigma') and there is no central part */
 };
 
 /* omegaW of a recorded field whose correction vanishes: -0.0 (sum_q delta_q W_q = 0), which a
@@ -213,29 +215,33 @@ __device__ __forceinline__ double dsign(double x) { return ipos(x) ? 1.0 : (ineg
 
 /* Tile of adj_fields_kernel (one thread per face) and its shared memory: the tile's points, per point
    the adjoints of U (NV), F (NV) and |lambda| (3), per face the Roe-state adjoints of its two centre
-   points.  Along x 128 faces of a row; y/z 16 x columns by 16 faces (halving the tile would stage
-   1.9 points per face instead of 1.4).  A field's reverse is one serial chain, so a tile costs about
-   100 us however few faces it holds: small CTAs keep the tiles of a small grid in one wave. */
-template <int NV, int K, int AXIS>
+   points.  Along x 128 faces of a row; y/z 16 x columns by YZ faces: 16, or 8 on grids whose tiles
+   would leave SMs without one (1.9 staged points per face instead of 1.4, but a full tile is 256
+   faces of FP64 on one SM: 32^2 TENO6 102 -> 84 us a call, 1024^2 1516 -> 1547). */
+template <int NV, int K, int AXIS, int YZ>
 struct AdjTile {
   static constexpr int H = K / 2, LANES = AXIS == 0 ? 1 : 16;
-  static constexpr int FACES = AXIS == 0 ? 128 : 16;
+  static constexpr int FACES = AXIS == 0 ? 128 : YZ;
   static constexpr int THREADS = FACES * LANES, NP = (FACES + K - 1) * LANES;
   static constexpr int NA = 2 * NV + 3, NR = 2 * NV;
   static constexpr size_t SMEM = sizeof(double) * ((size_t)(PointLayout<NV>::NC + NA) * NP + (size_t)NR * THREADS);
 };
 
 /* Adds the reverse of sum_s r_s f'_s of the axis's faces to Z.  A CTA finds its tile's faces with such
-   a field, gives each to a thread (dense warps, faces with most fields first; a tile without any
-   ends at once), and every face takes its i-th field in step i.  Per field: f'_s = l_s . (S_F + alpha/2 S_U) with S_F = sum_q
-   sigma'_q F_q, S_U = sum_q delta_q U_q, so the adjoint of l_s is fbar (S_F + alpha/2 S_U) and point q
-   receives fbar sigma'_q l_s (flux) and fbar (alpha/2) delta_q l_s (state).  Point adjoints are
-   summed in shared memory in K phases (in phase q every face adds to its q-th point, all
-   distinct); the reverse of the point quantities then runs once per touched point. */
-template <int NV, int K, int LIM, int AXIS, bool TAPE>
-__global__ void __launch_bounds__(AdjTile<NV, K, AXIS>::THREADS, (TAPE ? 512 : 256) / AdjTile<NV, K, AXIS>::THREADS)
+   a field and gives each to a thread (dense warps; a tile without any ends at once).  Per field: f'_s =
+   l_s . (S_F + alpha/2 S_U) with S_F = sum_q sigma'_q F_q, S_U = sum_q delta_q U_q, so the adjoint of l_s
+   is fbar (S_F + alpha/2 S_U) and point q receives fbar sigma'_q l_s (flux) and fbar (alpha/2) delta_q
+   l_s (state).  Point adjoints are summed in shared memory in K phases (in phase q every face adds to
+   its q-th point, all distinct); the reverse of the point quantities then runs once per touched point.
+   From the tape all fields of a face are taken together, point by point, in the basis that the
+   eigenvectors share; from the flags, where a field's weights have to be rebuilt first, one field after
+   the other (faces with most fields first, so that a step fills whole warps).  One field at a time
+   from the tape too cost a set of phases per field: 64x56x48 TENO6 with most faces listed 1007 us
+   against 883 (965 with every face reversed whole), with d_k of the caller's 1607 against 1048 (964). */
+template <int NV, int K, int LIM, int AXIS, bool TAPE, int YZ>
+__global__ void __launch_bounds__(AdjTile<NV, K, AXIS, YZ>::THREADS, (TAPE ? 512 : 256) / AdjTile<NV, K, AXIS, YZ>::THREADS)
     adj_fields_kernel(const AdjArgs A) {
-  using T = AdjTile<NV, K, AXIS>;
+  using T = AdjTile<NV, K, AXIS, YZ>;
   using L = PointLayout<NV>;
   constexpr int H = T::H, D = NV - 2, TH = T::THREADS, NP = T::NP, LANES = T::LANES, W = TH / 32;
   constexpr int NA = T::NA, NR = T::NR, RS = 2 * K + 2;
@@ -391,6 +397,135 @@ __global__ void __launch_bounds__(AdjTile<NV, K, AXIS>::THREADS, (TAPE ? 512 : 2
     }
   }
   const double una = ut[AXIS];
+  double tb[D];  /* adjoint of -u_t in l_shear */
+#pragma unroll
+  for (int d = 0; d < D; ++d) tb[d] = 0.0;
+  if constexpr (TAPE) {
+    /* all fields at once: the adjoints of a point's F and U are combined in the basis (e_0, a, b, e_t)
+       that the eigenvectors share before they are expanded, one set of phases for the face */
+    const double* const lin = A.lin + fi;
+    double kG[NV], kW[NV], Fc[NV], fp[NV], alb[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int s = 0; s < NV; ++s) {
+      kG[s] = kW[s] = fp[s] = Fc[s] = 0.0;
+      if (todo >> s & 1u) {
+        const int fam = s == 0 ? 0 : (s == NV - 1 ? 2 : 1);
+        double k = 0.0, hf = 1.0;  /* adjoint of f'_s; the 1/2 of l_{u-+c} = (a +- b)/2 */
+        if (s == 0 || s == NV - 1) {
+          const double sr = s == 0 ? -1.0 : 1.0;
+          k = fma(Ht + sr * una * ct, Fb[NV - 1], Fb[0]);
+#pragma unroll
+          for (int d = 0; d < D; ++d) k = fma(ut[d] + (d == AXIS ? sr * ct : 0.0), Fb[1 + d], k);
+          hf = 0.5;
+        } else if (s == 1) {
+          k = fma(0.5 * q2, Fb[NV - 1], Fb[0]);
+#pragma unroll
+          for (int d = 0; d < D; ++d) k = fma(ut[d], Fb[1 + d], k);
+        } else {
+          const int dt = (s - 2) < AXIS ? (s - 2) : (s - 1);
+          k = fma(ut[dt], Fb[NV - 1], Fb[1 + dt]);
+        }
+        fp[s] = __ldg(lin + (long long)(s * RS) * A.nface);
+        alb[fam] = fma(0.5 * k, __ldg(lin + (long long)(s * RS + 1) * A.nface), alb[fam]);
+        kG[s] = hf * k;
+        kW[s] = kG[s] * (0.5 * am[fam]);
+      }
+    }
+    const double b0v = una * cinv;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      double xu[NV], xf[NV];
+      if (has) {
+        double cU[NV], cF[NV];
+        const double cs = A.whole ? 0.0 : 0.5 * (cw[q] + cw[K - 1 - q]);
+#pragma unroll
+        for (int s = 0; s < NV; ++s) {
+          cF[s] = cU[s] = 0.0;
+          if (todo >> s & 1u) {
+            cF[s] = kG[s] * (__ldg(lin + (long long)(s * RS + 2 + q) * A.nface) - cs);
+            cU[s] = kW[s] * __ldg(lin + (long long)(s * RS + 2 + K + q) * A.nface);
+          }
+        }
+        const double AU = cU[0] + cU[NV - 1] - cU[1], BU = cU[0] - cU[NV - 1];
+        const double AF = cF[0] + cF[NV - 1] - cF[1], BF = cF[0] - cF[NV - 1];
+        double RU = cU[1], RF = cF[1];
+#pragma unroll
+        for (int s = 2; s < NV - 1; ++s) {
+          const int dt = (s - 2) < AXIS ? (s - 2) : (s - 1);
+          RU = fma(-ut[dt], cU[s], RU);
+          RF = fma(-ut[dt], cF[s], RF);
+        }
+        xu[0] = fma(AU, b2, fma(BU, b0v, RU));
+        xf[0] = fma(AF, b2, fma(BF, b0v, RF));
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          const int s = d < AXIS ? d + 2 : d + 1;  /* shear field of tangential axis d */
+          xu[1 + d] = fma(-AU * b1, ut[d], d == AXIS ? -BU * cinv : cU[s]);
+          xf[1 + d] = fma(-AF * b1, ut[d], d == AXIS ? -BF * cinv : cF[s]);
+        }
+        xu[NV - 1] = AU * b1;
+        xf[NV - 1] = AF * b1;
+        /* adjoints of the entries of a (all components), b (rho, m_n) and l_shear; Fc */
+        const double U0 = P(L::cU, q), F0 = P(L::cF, q);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const double Fv = v == 0 ? F0 : P(L::cF + v, q), Uv = v == 0 ? U0 : P(L::cU + v, q);
+          ab[v] = fma(AU, Uv, fma(AF, Fv, ab[v]));
+          Fc[v] = fma(cs, Fv, Fc[v]);
+        }
+        bb0 = fma(BU, U0, fma(BF, F0, bb0));
+        bb1 = fma(BU, P(L::cU + 1 + AXIS, q), fma(BF, P(L::cF + 1 + AXIS, q), bb1));
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          if (d == AXIS) continue;
+          const int s = d < AXIS ? d + 2 : d + 1;
+          tb[d] = fma(cU[s], U0, fma(cF[s], F0, tb[d]));
+        }
+      }
+      __syncthreads();  /* the previous phase's additions are complete */
+      if (has) {
+        const int pq = (jf + q) * LANES + lane;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          acc[(aU + v) * NP + pq] += xu[v];
+          acc[(aF + v) * NP + pq] += xf[v];
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          if (im[i] == q) acc[(aM + i) * NP + pq] += alb[i];
+      }
+    }
+    if (has) {  /* f'_s = fs - l_s . Fc, and the adjoints of r_s (= f'_s Fbar) */
+      double uF = 0.0;
+#pragma unroll
+      for (int d = 0; d < D; ++d) uF = fma(ut[d], Fc[1 + d], uF);
+      const double a = fma(b2, Fc[0], b1 * (Fc[NV - 1] - uF)), b = cinv * fma(una, Fc[0], -Fc[1 + AXIS]);
+      const double FE = Fb[NV - 1];
+#pragma unroll
+      for (int s = 0; s < NV; ++s) {
+        if (!(todo >> s & 1u)) continue;
+        if (s == 0 || s == NV - 1) {
+          const double sr = s == 0 ? -1.0 : 1.0, f1 = fp[s] - 0.5 * (a - sr * b);
+#pragma unroll
+          for (int d = 0; d < D; ++d) utb[d] = fma(f1, Fb[1 + d], utb[d]);
+          ctb = fma(sr * f1, fma(una, FE, Fb[1 + AXIS]), ctb);
+          Htb = fma(f1, FE, Htb);
+          utb[AXIS] = fma(sr * ct * f1, FE, utb[AXIS]);
+        } else if (s == 1) {
+          const double f1 = fp[s] - (Fc[0] - a);
+#pragma unroll
+          for (int d = 0; d < D; ++d) utb[d] = fma(f1, fma(ut[d], FE, Fb[1 + d]), utb[d]);
+        } else {
+          const int dt = (s - 2) < AXIS ? (s - 2) : (s - 1);
+          const double f1 = fp[s] - fma(-ut[dt], Fc[0], Fc[1 + dt]);
+          utb[dt] = fma(f1, FE, utb[dt]);
+        }
+      }
+#pragma unroll
+      for (int d = 0; d < D; ++d)
+        if (d != AXIS) utb[d] -= tb[d];
+    }
+  } else {
 #pragma unroll 1
   for (int step = 0; step < steps; ++step) {
     const bool on = todo != 0u;
@@ -424,14 +559,7 @@ __global__ void __launch_bounds__(AdjTile<NV, K, AXIS>::THREADS, (TAPE ? 512 : 2
         for (int d = 0; d < D; ++d) l[1 + d] = (d == dt) ? 1.0 : 0.0;
         l[NV - 1] = 0.0;
       }
-      if constexpr (TAPE) {
-        const double* o = A.lin + (long long)s * RS * A.nface + fi;
-#pragma unroll
-        for (int q = 0; q < K; ++q) {
-          sg[q] = __ldg(o + (long long)(2 + q) * A.nface) - 0.5 * (cw[q] + cw[K - 1 - q]);
-          dl[q] = __ldg(o + (long long)(2 + K + q) * A.nface);
-        }
-      } else {
+      {
         double Wv[K], Gv[K];
 #pragma unroll
         for (int q = 0; q < K; ++q) {
@@ -456,7 +584,7 @@ __global__ void __launch_bounds__(AdjTile<NV, K, AXIS>::THREADS, (TAPE ? 512 : 2
           for (int q = 0; q < K; ++q) {
             if (side) {
               dl[q] = sg[q] - om[K - 1 - q];
-              sg[q] = 0.5 * (sg[q] + om[K - 1 - q]) - 0.5 * (cw[q] + cw[K - 1 - q]);
+              sg[q] = 0.5 * (sg[q] + om[K - 1 - q]) - (A.whole ? 0.0 : 0.5 * (cw[q] + cw[K - 1 - q]));
             } else {
               sg[q] = om[q];
             }
@@ -537,6 +665,7 @@ __global__ void __launch_bounds__(AdjTile<NV, K, AXIS>::THREADS, (TAPE ? 512 : 2
         if (imax == q) acc[(aM + fam) * NP + pq] += alb;
       }
     }
+  }
   }
 
   /* ---- eigenvector adjoints -> Roe average -> the two centre points ---- */

@@ -145,17 +145,24 @@ static cudaError_t launch_stats_nv(const FaceArgs& a, int axis, int K, int lim, 
 }
 
 /* reverse of the axis's nonlinear fields (from a.lin, else from a.flags) */
-template <int NV, int K, int LIM, int AXIS, bool TAPE>
-static cudaError_t launch_adj_fields_one(const AdjArgs& a, cudaStream_t st) {
-  using T = AdjTile<NV, K, AXIS>;
+template <int NV, int K, int LIM, int AXIS, bool TAPE, int YZ>
+static cudaError_t launch_adj_fields_tile(const AdjArgs& a, cudaStream_t st) {
+  using T = AdjTile<NV, K, AXIS, YZ>;
   static AttrOnce attr;
-  const cudaError_t e = ensure_smem_attr(adj_fields_kernel<NV, K, LIM, AXIS, TAPE>, attr, T::SMEM);
+  const cudaError_t e = ensure_smem_attr(adj_fields_kernel<NV, K, LIM, AXIS, TAPE, YZ>, attr, T::SMEM);
   if (e != cudaSuccess) return e;
   const unsigned tiles = (unsigned)((a.n[AXIS] + T::FACES) / T::FACES);  /* n_a + 1 faces */
   const dim3 grid = AXIS == 0 ? dim3((unsigned)(a.n[1] * a.n[2]), tiles)
                               : dim3((unsigned)((a.n[0] + T::LANES - 1) / T::LANES), tiles, (unsigned)(AXIS == 1 ? a.n[2] : a.n[1]));
-  adj_fields_kernel<NV, K, LIM, AXIS, TAPE><<<grid, T::THREADS, T::SMEM, st>>>(a);
+  adj_fields_kernel<NV, K, LIM, AXIS, TAPE, YZ><<<grid, T::THREADS, T::SMEM, st>>>(a);
   return cudaGetLastError();
+}
+template <int NV, int K, int LIM, int AXIS, bool TAPE>
+static cudaError_t launch_adj_fields_one(const AdjArgs& a, cudaStream_t st) {
+  if constexpr (TAPE && AXIS > 0) {  /* fewer tiles of 256 faces than two a SM: tiles of 128 */
+    if (a.nface < 2ll * 152 * 256) return launch_adj_fields_tile<NV, K, LIM, AXIS, TAPE, 8>(a, st);
+  }
+  return launch_adj_fields_tile<NV, K, LIM, AXIS, TAPE, 16>(a, st);
 }
 
 template <int NV, int K, int AXIS>
