@@ -92,18 +92,10 @@ __global__ void batch_init_kernel(const double* prim, double* U, long long total
   }
 }
 
-template <int K, int LIM, int TILE>
-static StageFn stage_fn() { return batch_stage_kernel<K, LIM, TILE, false>; }
-
-static StageFn pick_stage(int K, int lim, int tile, bool pp) {
-  if (pp) return pick_stage_pp(K, lim, tile);
-#define TENOM_PICK(KK, LL, TT) if (K == KK && lim == LL && tile == TT) return stage_fn<KK, LL, TT>();
-  TENOM_PICK(6, LIM_MP, 64) TENOM_PICK(6, LIM_MP, 128) TENOM_PICK(6, LIM_MP, 256)
-  TENOM_PICK(6, LIM_TVD5, 64) TENOM_PICK(6, LIM_TVD5, 128) TENOM_PICK(6, LIM_TVD5, 256)
-  TENOM_PICK(8, LIM_MP, 64) TENOM_PICK(8, LIM_MP, 128) TENOM_PICK(8, LIM_MP, 256)
-  TENOM_PICK(8, LIM_TVD5, 64) TENOM_PICK(8, LIM_TVD5, 128) TENOM_PICK(8, LIM_TVD5, 256)
-#undef TENOM_PICK
-  return nullptr;
+static StageFn pick_stage(const tenom_scheme& s, int tile) {
+  const bool all = !scheme_for_device(s).screen;
+  if (s.positivity == TENOM_PP_ON) return pick_stage_pp(s.K, s.limiter, tile, all);
+  return all ? pick_stage_of<false, true>(s.K, s.limiter, tile) : pick_stage_of<false, false>(s.K, s.limiter, tile);
 }
 
 /* dynamic shared memory of the stage kernel of (K, tile): the kernel's own layout */
@@ -176,7 +168,7 @@ static cudaError_t build_items(tenom_batch* b, int tile) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
   b->tile = tile;
   /* shared-memory size of the stage kernel for this tile (set outside any graph capture) */
-  StageFn fn = pick_stage(b->s.K, b->s.limiter, tile, b->s.positivity == TENOM_PP_ON);
+  StageFn fn = pick_stage(b->s, tile);
   if (e == cudaSuccess && fn)
     e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)stage_smem(b->s.K, tile));
@@ -203,7 +195,7 @@ static BatchArgs batch_args(tenom_batch* b, int stage) {
 }
 
 static cudaError_t launch_stage_b(tenom_batch* b, int stage, double* U, cudaStream_t st) {
-  StageFn fn = pick_stage(b->s.K, b->s.limiter, b->tile, b->s.positivity == TENOM_PP_ON);
+  StageFn fn = pick_stage(b->s, b->tile);
   if (!fn) return cudaErrorNotSupported;
   const size_t smem = stage_smem(b->s.K, b->tile);
   BatchArgs a = batch_args(b, stage);
@@ -435,7 +427,7 @@ tenom_status tenom_batch_autotune(tenom_batch* b, double* U, int* tile_out, int*
   int bt = b->tile, bc = b->ctas_per_sm;
   for (int ti = 0; ti < 3 && e == cudaSuccess; ++ti) {
     e = build_items(b, tiles[ti]);
-    StageFn fn = pick_stage(b->s.K, b->s.limiter, tiles[ti], b->s.positivity == TENOM_PP_ON);
+    StageFn fn = pick_stage(b->s, tiles[ti]);
     int occ = 0;
     const size_t smem = stage_smem(b->s.K, tiles[ti]);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)fn, tiles[ti], smem);

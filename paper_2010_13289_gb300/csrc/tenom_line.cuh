@@ -93,8 +93,9 @@ __device__ __forceinline__ double line_stage(LineTile<K, TILE, FACES>& S, const 
 }
 
 /* Fluxes of the staged tile's nf faces (those <= n) into S.F, limited for a stage with mu = 2 dt/dx
-   when PP.  All threads of the CTA call it; S.F is complete on return. */
-template <int K, int LIM, int TILE, bool PP, int FACES>
+   when PP.  ALL: the scheme is not screened (sch.screen = 0).  All threads of the CTA call it; S.F is
+   complete on return. */
+template <int K, int LIM, int TILE, bool PP, bool ALL = false, int FACES>
 __device__ __forceinline__ void line_fluxes(LineTile<K, TILE, FACES>& S, int n, int f0, int nf, double gamma, double rgm1,
                                             const SchemeDev& sch, double mu, int& st) {
   using T = LineTile<K, TILE, FACES>;
@@ -118,7 +119,9 @@ __device__ __forceinline__ void line_fluxes(LineTile<K, TILE, FACES>& S, int n, 
 #pragma unroll
       for (int q = 1; q < K; ++q) Fh[v] = fma(cw[q], s[q], Fh[v]);
     }
-    bad = sch.screen ? screen_face<NV, K, 0, 1>(S.sf, NP, tid, (float)gm1, sch, false) : allf;
+    bad = allf;
+    if constexpr (!ALL)
+      if (sch.screen) bad = screen_face<NV, K, 0, 1>(S.sf, NP, tid, (float)gm1, sch, false);
     if (bad) {
       const LineFace<T, K> src{S.pt, S.sf, tid};
       face_rows<NV, K, TILE>(src, S.row + tid, gm1, rgm1, st);
@@ -146,27 +149,53 @@ __device__ __forceinline__ void line_fluxes(LineTile<K, TILE, FACES>& S, int n, 
   }
   if (nitem) {  /* uniform over the CTA */
     __syncthreads();
-    /* one (face, field, side) per thread: a short line is all latency, and projecting a second
-       time costs less of it than two sides one after the other */
-#pragma unroll 1
-    for (int it = tid; it < 2 * nitem; it += TILE) {
-      const int side = it >= nitem ? 1 : 0, item = S.item[it - (side ? nitem : 0)], fc = item & 511, s = item >> 9;
-      double l[NV], v[K];
-      const double ha = left_vector<NV, TILE>(S.row + fc, s, l);
-#pragma unroll
-      for (int q = 0; q < K; ++q) {
-        const int p = fc + (side ? K - 1 - q : q);  /* f- on the mirrored stencil */
-        const double un = S.pt[T::un * NP + p];
-        double x = l[0] * S.pt[T::rho * NP + p];
-        x = fma(l[1], S.pt[T::m * NP + p], x);
-        x = fma(l[2], S.pt[T::E * NP + p], x);
-        v[q] = fma(side ? -ha : ha, x, 0.5 * fma(S.pt[T::pr * NP + p], fma(un, l[2], l[1]), un * x));
-      }
+    auto project = [&](const double (&l)[NV], int p, double& w, double& hg) {  /* W and G/2 of tile point p */
+      const double un = S.pt[T::un * NP + p];
+      w = l[0] * S.pt[T::rho * NP + p];
+      w = fma(l[1], S.pt[T::m * NP + p], w);
+      w = fma(l[2], S.pt[T::E * NP + p], w);
+      hg = 0.5 * fma(S.pt[T::pr * NP + p], fma(un, l[2], l[1]), un * w);
+    };
+    auto reconstruct = [&](const double (&v)[K], int side, int s, int fc) {
       unsigned b = 0u;
       int e = 7;
       if (!teno_decide_fast<K, false>(v, sch, b, e)) teno_decide_fp64<K>(v, sch, b, e, st);
       S.fs[(side * NV + s) * TILE + fc] = teno_general<K, LIM>(v, sch, b);
       if (b == allk && sch.default_d) atomicOr(&S.cm[side * TILE + fc], 1u << s);
+    };
+    if constexpr (ALL) {
+      /* every field of every face: both sides from one projection */
+#pragma unroll 1
+      for (int it = tid; it < nitem; it += TILE) {
+        const int item = S.item[it], fc = item & 511, s = item >> 9;
+        double l[NV], w[K], hg[K];
+        const double ha = left_vector<NV, TILE>(S.row + fc, s, l);
+#pragma unroll
+        for (int q = 0; q < K; ++q) project(l, fc + q, w[q], hg[q]);
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+          double v[K];
+#pragma unroll
+          for (int q = 0; q < K; ++q) v[q] = side ? fma(-ha, w[K - 1 - q], hg[K - 1 - q]) : fma(ha, w[q], hg[q]);
+          reconstruct(v, side, s, fc);
+        }
+      }
+    } else {
+      /* one (face, field, side) per thread: a short line is all latency, and projecting a second
+         time costs less of it than two sides one after the other */
+#pragma unroll 1
+      for (int it = tid; it < 2 * nitem; it += TILE) {
+        const int side = it >= nitem ? 1 : 0, item = S.item[it - (side ? nitem : 0)], fc = item & 511, s = item >> 9;
+        double l[NV], v[K];
+        const double ha = left_vector<NV, TILE>(S.row + fc, s, l);
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          double w, hg;
+          project(l, fc + (side ? K - 1 - q : q), w, hg);  /* f- on the mirrored stencil */
+          v[q] = fma(side ? -ha : ha, w, hg);
+        }
+        reconstruct(v, side, s, fc);
+      }
     }
     __syncthreads();
     if (bad) {
