@@ -56,7 +56,7 @@ FACE_SOURCES = ("tenom_screen.cuh", "tenom_nonlinear.cuh", "tenom_fixed.cuh", "t
                 "tenom_fastmath.cuh", "tenom_launch.cuh", "tenom_internal.h")
 
 
-BATCH_SOURCES = FACE_SOURCES + ("tenom_batch.cu", "tenom_batch_kernel.cuh", "tenom_positivity.cuh")
+BATCH_SOURCES = FACE_SOURCES + ("tenom_line.cuh", "tenom_batch.cu", "tenom_batch_kernel.cuh", "tenom_positivity.cuh")
 
 
 def face_source_hash(sources=FACE_SOURCES):
@@ -310,9 +310,10 @@ def oracle_rate_batch(name, seconds):
 
 
 def launches_per_step(dim, positivity):
-    """Kernel launches of one SSP-RK3 step of a grid workload: the signal-speed reduction, dt
-    and the time update, and per stage the primitives, one face sweep per axis (plus one
-    limiter pass per axis when the positivity limiter is on) and the cell update."""
+    """Kernel launches of one SSP-RK3 step of a 2D or 3D grid workload: the signal-speed reduction
+    (which also leaves the first stage's primitives), dt and the time update, and per stage one
+    screen per axis, the nonlinear launch, one limiter pass per axis when the positivity limiter is on,
+    and the cell update (which leaves the next stage's primitives)."""
     return 3 + 3 * (dim * (2 if positivity else 1) + 2)
 
 

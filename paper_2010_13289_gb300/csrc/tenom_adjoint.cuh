@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) adj_central_kernel(const AdjArgs A) {
   }
 }
 
-/* Reverse of the point quantities (stage_point): adjoints of the physical flux F_AXIS (Fb),
+/* Reverse of the point quantities (stage_point_from): adjoints of the physical flux F_AXIS (Fb),
    of the velocity (velb), sound speed (cb), enthalpy (Hb) and sqrt(rho) (sb) of one point
    -> adjoint of its conserved state, added to Ub. */
 template <int NV, int AXIS>

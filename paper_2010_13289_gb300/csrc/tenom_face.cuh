@@ -108,15 +108,6 @@ __device__ __forceinline__ void point_prims(const double (&u)[NV], double gamma,
   if (!ipos(pr)) st |= ST_P;
 }
 
-/* ... and total enthalpy H = (E + p)/rho, sqrt(rho). */
-template <int NV>
-__device__ __forceinline__ void point_prims(const double (&u)[NV], double gamma, double (&vel)[NV - 2], double& pr,
-                                            double& Hh, double& c, double& sr, int& st) {
-  point_prims<NV>(u, gamma, vel, pr, c, st);
-  Hh = (u[NV - 1] + pr) * rcp_nr(u[0]);
-  sr = sqrt(u[0]);
-}
-
 /* Point quantities of the Euler equations for sweep axis AXIS, written to the tile from U
    and its primitives: U, the physical flux F_AXIS(U), velocity, H, c, sqrt(rho),
    |u_a - c|, |u_a + c|. */
@@ -139,14 +130,6 @@ __device__ __forceinline__ void stage_point_from(const double (&u)[NV], const do
   sm[L::cS * NP + p] = sr;
   sm[L::cLm * NP + p] = iabs(un - c);
   sm[L::cLp * NP + p] = iabs(un + c);
-}
-
-/* Point quantities computed here (once per point of the tile). */
-template <int NV, int AXIS>
-__device__ __forceinline__ void stage_point(const double (&u)[NV], double gamma, double* sm, int NP, int p, int& st) {
-  double vel[NV - 2], pr, Hh, c, sr;
-  point_prims<NV>(u, gamma, vel, pr, Hh, c, sr, st);
-  stage_point_from<NV, AXIS>(u, vel, pr, Hh, c, sr, sm, NP, p);
 }
 
 /* Decision statistics of the face whose K stencil points are shared-memory points

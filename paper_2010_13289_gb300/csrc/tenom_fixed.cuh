@@ -10,8 +10,8 @@
  * each on GB300's FP64 pipe, paid by the whole warp when one lane needs them.
  *
  * Overflow: |v| <= 2^54, differences <= 2^55, second differences < 2^56, 4 d - d' < 5 2^56,
- * candidates and bounds (alpha, beta/3 <= 8, scheme's fixed flag) < 2^60; the TVD5 terms in 60ths
- * < 94 2^55 + 60 2^55 < 2^62.3. */
+ * bounds (alpha, beta/3 <= 8, scheme's fixed flag) < 2^60; the candidates' numerators and the TVD5
+ * terms in 60ths at most 130 2^55 (candidate 4) + 60 2^55 < 2^62.6. */
 #pragma once
 #include "tenom_recon.cuh"
 
@@ -53,7 +53,7 @@ __device__ __forceinline__ long long cand60(int k, const long long* D) {
 }
 
 /* floor((60 (f_k - f_i)) / 60) within one unit, through the candidate's own denominator (so that
-   the numerator stays below 2^60) */
+   the numerator stays below 2^62) */
 template <int c>
 __device__ __forceinline__ long long cand_unit(int k, const long long* D) {
   const long long q6 = 0x2aaaaaaaaaaaaaaall;   /* 2^64 / 6 */

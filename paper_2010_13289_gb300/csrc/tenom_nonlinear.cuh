@@ -327,6 +327,7 @@ __device__ __noinline__ unsigned decide_cold(const double* w, const double* g, d
   teno_decide_fp64<K>(v, S, b, e, st);
   return b | ((unsigned)((e - 7) & 3) << 6);
 }
+/* f+ + f- with the decisions fl taken: a shear item that turned out to reach across a jump */
 template <int K, int LIM>
 __device__ __noinline__ double general_cold(const double* w, const double* g, double al, unsigned fl, const SchemeDev& S) {
   constexpr unsigned allk = (1u << (K - 2)) - 1u;
@@ -337,6 +338,26 @@ __device__ __noinline__ double general_cold(const double* w, const double* g, do
     split_side<K>(w, g, al, side, v);
     f += teno_general<K, LIM>(v, S, fl >> (8 * side) & allk);
   }
+  return f;
+}
+/* an item that takes the FP64 form from the start (a jump face's, or outside the fixed-point range):
+   decisions and reconstruction of both sides from the FP64 sequence; returns f+ + f- */
+template <int K, int LIM>
+__device__ __noinline__ double direct_cold(const double* w, const double* g, double al, const SchemeDev& S, unsigned& fl,
+                                           int& st) {
+  double f = 0.0;
+  unsigned bits = 0u;
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    double v[K];
+    split_side<K>(w, g, al, side, v);
+    unsigned b = 0u;
+    int e = 7;
+    if (!teno_decide_fast<K>(v, S, b, e)) teno_decide_fp64<K>(v, S, b, e, st);
+    f += teno_general<K, LIM>(v, S, b);
+    bits |= (b | ((unsigned)((e - 7) & 3) << 6)) << (8 * side);
+  }
+  fl = bits;
   return f;
 }
 
@@ -440,25 +461,23 @@ __device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double
 /* Both split sides of an item from its projected W and G (columns w, g in shared memory):
    decisions, and the corrections of the nonsmooth sides in fixed point.  Returns false when the
    FP32 filter leaves a side undecided and `defer` is set.  Dx: K - 1 scratch words of the item's
-   thread.  em: biased exponent of a power of two above every |G| + |alpha W|.  jump: the item's
-   corrections would cancel values far above the centre's (reaches_jump, kShearJump).  The loops over
+   thread.  em: biased exponent of a power of two above every |G| + |alpha W|.  fp64: the item's
+   face takes the FP64 form (reaches_jump); jump: the shear item's corrections would cancel values far
+   above the centre's (kShearJump).  The loops over
    the points are rolled and everything rare is called, to keep the code that an item runs
    small (unrolled 4 or 8 times: 256^3 step 64 ms against 59, 64^3 turbulence 5.6 against 5.1). */
 template <int K, int LIM>
-__device__ __forceinline__ bool fixed_item(const double* w, const double* g, double al, int em, bool jump,
+__device__ __forceinline__ bool fixed_item(const double* w, const double* g, double al, int em, bool fp64, bool jump,
                                            long long* Dx, const SchemeDev& S, bool defer, unsigned& fl, double& fsum,
                                            bool& direct, int& st) {
   constexpr int TH = NL_THREADS;
   constexpr unsigned allk = (1u << (K - 2)) - 1u;
-  fl = 0u;
-  direct = false;
-  if (em < 1024 - 40 || em > 1024 + 40) {  /* outside the fixed-point range: FP64, and at once (no pass can do better) */
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) fl |= decide_cold<K>(w, g, al, side, S, st) << (8 * side);
-    direct = (fl & (allk | allk << 8)) != (allk | allk << 8);
-    fsum = general_cold<K, LIM>(w, g, al, fl, S);
+  direct = fp64 || em < 1024 - 40 || em > 1024 + 40;  /* FP64, and at once (no pass can do better) */
+  if (direct) {
+    fsum = direct_cold<K, LIM>(w, g, al, S, fl, st);
     return true;
   }
+  fl = 0u;
   const float unit = __int_as_float((em - 1077 + 127) << 23);  /* 2^(em - 1077): of the halved values */
   Acc96 acc;
 #pragma unroll 1
@@ -535,7 +554,8 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
   __shared__ double s_w[FIX ? K * TH : 1], s_g[FIX ? K * TH : 1];  /* an item's W and G */
   __shared__ long long s_D[FIX ? (K - 1) * TH : 1];
   __shared__ int s_nlater;
-  __shared__ int s_wc[NV * W + 1];
+  constexpr int NS = FIX ? 2 * NV : NV;  /* the item order's sorts: field, and jump faces last */
+  __shared__ int s_wc[NS * W + 1];
   const int tid = threadIdx.x, wid = tid >> 5, ln = tid & 31;
   int st = 0;
 
@@ -575,6 +595,7 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
 
     /* ---- (0) Roe state and LLF speeds, one thread per face ---- */
     unsigned mask = 0u;
+    bool jump_face = false;
     long long flin = 0, fcopy = -1;  /* face n of a periodic line is face 0's copy */
     if (tid < nf) {
       const unsigned idx = A.list[ax][i0 + tid];
@@ -609,34 +630,38 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
       s_base[tid] = base;
       s_f[tid] = f;
       s_cm[tid] = A.sch.default_d ? (allf & ~mask) : 0u;
-      s_dir[tid] = FIX && reaches_jump<NV, K, LIM, TH>(src, Pp, s_row + tid, A.gamma - 1.0) ? kJumpFace : 0u;
+      jump_face = FIX && reaches_jump<NV, K, LIM, TH>(src, Pp, s_row + tid, A.gamma - 1.0);
+      s_dir[tid] = jump_face ? kJumpFace : 0u;
     }
-    /* the chunk's (face, field) items, field after field */
+    /* the chunk's (face, field) items, field after field; those of jump faces, which take the FP64
+       form, after the others, in warps of their own */
+    auto has_item = [&](int e) -> bool { return (mask >> (e % NV) & 1u) && (!FIX || jump_face == (e >= NV)); };
 #pragma unroll
-    for (int s = 0; s < NV; ++s) {
-      const unsigned b = __ballot_sync(0xffffffffu, mask >> s & 1u);
-      if (ln == 0) s_wc[s * W + wid] = __popc(b);
+    for (int e = 0; e < NS; ++e) {
+      const unsigned b = __ballot_sync(0xffffffffu, has_item(e));
+      if (ln == 0) s_wc[e * W + wid] = __popc(b);
     }
     __syncthreads();
-    if (wid == 0) {  /* exclusive scan of the NV * W counts */
-      static_assert(NV * W <= 32, "one warp scans the counts");
-      const int c = ln < NV * W ? s_wc[ln] : 0;
-      int x = c;
+    if (wid == 0) {  /* exclusive scan of the NS * W counts, two a lane */
+      static_assert(NS * W <= 64, "one warp scans the counts");
+      const int c0 = 2 * ln < NS * W ? s_wc[2 * ln] : 0, c1 = 2 * ln + 1 < NS * W ? s_wc[2 * ln + 1] : 0;
+      int x = c0 + c1;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (ln >= o) x += y;
       }
-      if (ln < NV * W) s_wc[ln] = x - c;
-      if (ln == 31) s_wc[NV * W] = x;
+      if (2 * ln < NS * W) s_wc[2 * ln] = x - c0 - c1;
+      if (2 * ln + 1 < NS * W) s_wc[2 * ln + 1] = x - c1;
+      if (ln == 31) s_wc[NS * W] = x;
     }
     __syncthreads();
 #pragma unroll
-    for (int s = 0; s < NV; ++s) {
-      const unsigned b = __ballot_sync(0xffffffffu, mask >> s & 1u);
-      if (mask >> s & 1u) s_item[s_wc[s * W + wid] + __popc(b & ((1u << ln) - 1u))] = (unsigned short)(tid | (s << 8));
+    for (int e = 0; e < NS; ++e) {
+      const unsigned b = __ballot_sync(0xffffffffu, has_item(e));
+      if (has_item(e)) s_item[s_wc[e * W + wid] + __popc(b & ((1u << ln) - 1u))] = (unsigned short)(tid | ((e % NV) << 8));
     }
-    const int nitem = s_wc[NV * W];
+    const int nitem = s_wc[NS * W];
     if (tid == 0) s_nlater = 0;
     __syncthreads();
 
@@ -696,9 +721,8 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS_PER_SM) nonlinear_kernel(c
         /* 2 |v| <= |G| + |alpha W| < 2^(em - 1022) */
         const double al = ha + ha;
         const int em = 1 + max(eg, ew + (int)((unsigned)__double2hiint(al) >> 20 & 0x7ffu) - 1022);
-        const bool jump = far - near > kShearJump || (s_dir[fc] & kJumpFace);
-        if (!fixed_item<K, LIM>(s_w + tid, s_g + tid, al, em, jump, s_D + tid, A.sch, pass == 0 && nitem > TH, fl,
-                                fsum, direct, st)) {
+        if (!fixed_item<K, LIM>(s_w + tid, s_g + tid, al, em, (s_dir[fc] & kJumpFace) != 0u, far - near > kShearJump,
+                                s_D + tid, A.sch, pass == 0 && nitem > TH, fl, fsum, direct, st)) {
           s_later[atomicAdd(&s_nlater, 1)] = (unsigned short)item;
           continue;
         }
