@@ -15,7 +15,7 @@
  *     with the fields' weights from the recorded linearisation or rebuilt from the flags.
  * Reversing the whole characteristic decomposition of every face instead took 550-610 FP64
  * operations a face.  Per stage of the 2D 512^2 TENO6 workload (55 % of the faces listed, two
- * fields each): two sweeps of 317 us before, 47 us central and 2 x 258 us now, FP64 pipe 80 %
+ * fields each): two sweeps of 317 us before, 47 us central and 2 x 260 us now, FP64 pipe 80 %
  * busy; with the flags on 256^2 TENO8 waves (13 % listed) two of 480 us before, 26 + 223 + 113 now. */
 #pragma once
 #include "tenom_face.cuh"

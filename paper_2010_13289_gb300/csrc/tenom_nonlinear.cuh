@@ -26,7 +26,8 @@
  * limiter's divergent lanes and, for any lane the FP32 filter left undecided, the whole warp in
  * FP64 decisions), 1.9 ms with fixed-point corrections and the second pass, 1.45 ms with the
  * rolled loops and called rare paths (instruction fetch had been the largest stall), 1.19 ms since
- * the filter decides all but 0.01 % of the sides. */
+ * the filter decides all but 0.01 % of the sides, 1.04 ms with jumps found per face instead of
+ * exponents kept per side. */
 #pragma once
 #include "tenom_recon.cuh"
 #include "tenom_face.cuh"
@@ -380,7 +381,8 @@ __device__ __forceinline__ void put_tape(const Wq& w, const double* op, const do
     }
   }
 }
-/* The tape of a fixed-point item.  The face flux comes from the same fixed-point form as the forward
+/* The tape of a fixed-point item (a record launch of the 512^2 rollout: 600 us, 470 with FP64 items
+   alone, 245 without a tape).  The face flux comes from the same fixed-point form as the forward
    kernel's, so that a recorded step has its bits (a rollout is recomputed from its checkpoints for the
    reverse, and branches frozen on states that differ in the last bits are another trajectory's);
    only the frozen weights are formed in FP64. */
@@ -420,7 +422,8 @@ __device__ __forceinline__ float f32_hi(const double* x) {
    of rho and p every 7 cells, TENO6): MP ratio 1 0.71 | 0.50, 2 0.71 | 0.69, 4 0.75 | 1.08, 10 0.73 | 2.4,
    1000 0.76 | 57; TVD5 ratio 1 0.58 | 0.24, 4 0.71 | 0.65 (jumps of p), 10 0.88 | 1.8.  It holds for the
    face, not for a field: beside a field in FP64 another one's l_s . Fc would bring the far values
-   back.  (A NaN reaches.) */
+   back.  What it costs: 2048^2 TENO6-MP, whose discs jump by 2-10, 5.0 -> 5.3 ms a step, TENO8-TVD5 5.6
+   -> 5.8; 256^3 nothing.  (A NaN reaches.) */
 template <int NV, int K, int LIM, int TH>
 __device__ __forceinline__ bool reaches_jump(const GridFace<NV, K>& src, const double* p, const double* row, double gm1) {
   constexpr int D = NV - 2, H = K / 2;

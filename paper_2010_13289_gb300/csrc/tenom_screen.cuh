@@ -20,7 +20,7 @@
  * warp and face).  The single kernel this pair replaced formed Roe state, eigenvectors and the
  * composition in FP64 for every warp that held an uncertified face and waited for its own
  * queue at CTA barriers: 1024^2 TENO8 sweeps 0.72 ms against 0.43 ms for the pair, one step of
- * 2048^2 TENO8-TVD5 17.8 -> 5.6 ms, TENO6-MP 13.2 -> 5.1, 256^3 TENO8-MP 133 -> 53 with the
+ * 2048^2 TENO8-TVD5 17.8 -> 5.8 ms, TENO6-MP 13.2 -> 5.3, 256^3 TENO8-MP 133 -> 52 with the
  * nonlinear kernel's later forms. */
 #pragma once
 #include "tenom_recon.cuh"
